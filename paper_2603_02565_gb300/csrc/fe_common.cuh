@@ -141,8 +141,95 @@ __device__ __forceinline__ bool mbar_wait_compact(uint64_t* bar, uint32_t parity
 }
 
 // ---------------------------------------------------------------------------
+// Whole-warp issue.  A role that only one thread performs (tcgen05.mma, its
+// commits, TMA) is run by its whole warp in step: every lane keeps the loop
+// state and polls the barriers, and the instructions themselves are predicated
+// on the lane that elect.sync picks (always the same one).  The control flow
+// stays uniform for the compiler; behind `if (lane == 0)` with a `break` on a
+// timed-out wait, two satisfied waits, two MMAs of N = 64 and a commit took 475
+// cycles of the issuing thread, this form 126 to 180 (eight MMAs and one wait: 739
+// and 385, the tensor pipe's own time).  So a wait returns nothing: after a
+// timeout the role runs on to its end without synchronisation, every later wait
+// giving up at once (the batch's results are invalid then; every address it
+// uses stays in bounds).  A wait ends with the warp converged: an elected lane
+// that ran ahead could advance a barrier by two phases under a lane still
+// polling it.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t e;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+  return e;
+}
+
+__device__ __forceinline__ bool mbar_try_wait_at(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+// The whole warp's wait, by shared-memory address.  It gives up after
+// kWaitLimitNs (about; the timer's upper bits) and, once any thread of the batch
+// has, after 256 polls.
+__device__ __forceinline__ void mbar_wait_at(uint32_t bar, uint32_t parity, int* status) {
+  if (!mbar_try_wait_at(bar, parity)) {
+    const uint32_t t0 = (uint32_t)(globaltimer_ns() >> 16);
+    for (uint32_t it = 1; !mbar_try_wait_at(bar, parity); ++it) {
+      if ((it & 255u) == 0u && (*reinterpret_cast<volatile int*>(status) & ST_TIMEOUT)) break;
+      if ((uint32_t)(globaltimer_ns() >> 16) - t0 > (uint32_t)(kWaitLimitNs >> 16)) {
+        atomicOr(status, ST_TIMEOUT);
+        break;
+      }
+    }
+  }
+  __syncwarp();
+}
+__device__ __forceinline__ void mbar_wait_warp(uint64_t* bar, uint32_t parity, int* status) {
+  mbar_wait_at(smem_u32(bar), parity, status);
+}
+__device__ __forceinline__ void mbar_arrive_if_at(uint32_t bar, uint32_t go) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+      "@q mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}" ::"r"(bar),
+      "r"(go)
+      : "memory");
+}
+
+__device__ __forceinline__ void mbar_arrive_expect_tx_if(uint64_t* bar, uint32_t bytes, uint32_t go) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t"
+      "@q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t}" ::"r"(smem_u32(bar)),
+      "r"(bytes), "r"(go)
+      : "memory");
+}
+
+// ---------------------------------------------------------------------------
 // TMA: 2D tiled bulk tensor load global -> shared, completion on an mbarrier
 // ---------------------------------------------------------------------------
+__device__ __forceinline__ void tma_load_2d_if(void* smem_dst, const CUtensorMap* map, int x, int y, uint64_t* bar,
+                                               uint32_t go) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+      "@q cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%3, %4}], [%2];\n\t}" ::"r"(smem_u32(smem_dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(go)
+      : "memory");
+}
+
+__device__ __forceinline__ void tma_load_3d_if(void* smem_dst, const CUtensorMap* map, int x, int y, int z,
+                                               uint64_t* bar, uint32_t go) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %6, 0;\n\t"
+      "@q cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%3, %4, %5}], [%2];\n\t}" ::"r"(smem_u32(smem_dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(z), "r"(go)
+      : "memory");
+}
+
 __device__ __forceinline__ void tma_load_2d(void* smem_dst, const CUtensorMap* map, int x, int y,
                                             uint64_t* bar) {
   asm volatile(
@@ -277,6 +364,45 @@ __device__ __forceinline__ void umma_commit(uint64_t* bar) {
                : "memory");
 }
 
+// The same three for whole-warp issue: predicated on go, the elected lane's flag.
+__device__ __forceinline__ void umma_bf16_if(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                             uint32_t accumulate, uint32_t go) {
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "setp.ne.b32 q, %5, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(go)
+      : "memory");
+}
+
+__device__ __forceinline__ void umma_bf16_tmem_a_if(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc,
+                                                    uint32_t accumulate, uint32_t go) {
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "setp.ne.b32 q, %5, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(tmem_d),
+      "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(go)
+      : "memory");
+}
+
+__device__ __forceinline__ void umma_commit_if(uint64_t* bar, uint32_t go) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(smem_u32(bar)),
+      "r"(go)
+      : "memory");
+}
+
+// Every product issued so far is complete before the block may free its TMEM
+// (after a timed-out wait nothing else has waited for them).  drain: a barrier of
+// count 1 that nothing else uses.
+__device__ __forceinline__ void umma_drain(uint64_t* drain, int* status, uint32_t go) {
+  umma_commit_if(drain, go);
+  mbar_wait_warp(drain, 0u, status);
+}
+
 // 32 lanes x 32 columns of 32-bit TMEM -> 32 registers per thread (row = lane).
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
   uint32_t r[32];
@@ -319,6 +445,21 @@ __device__ __forceinline__ void tmem_ld64(uint32_t taddr, float* v) {
   for (int i = 0; i < 64; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// 32 lanes x 8 columns -> 8 registers per thread, and back (completes at tmem_st_wait())
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+      : "r"(taddr)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_st8_nowait(uint32_t taddr, const uint32_t* r) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(r[0]),
+               "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+               : "memory");
+}
+
 // 32 lanes x 16 columns -> 16 registers per thread
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   uint32_t r[16];
@@ -332,6 +473,26 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
       : "memory");
 #pragma unroll
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// Two fp32 values in one 64-bit register: one instruction for both, each rounded as its scalar form.
+__device__ __forceinline__ uint64_t f32x2_pack(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void f32x2_unpack(uint64_t v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ uint64_t f32x2_fma(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ uint64_t f32x2_add(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
 }
 
 // 2^x with the hardware approximation (ex2.approx.ftz.f32)

@@ -6,10 +6,10 @@
 // to every row) for rows of width d <= 128, without writing x, LN(x) or the
 // F-wide intermediate to memory.  A persistent CTA walks 128-row tiles, F in
 // chunks of 128 columns:
-//   warp 0 lane 0 : TMA producer -- the A tile (hi/lo) and a ring of weight
+//   warp 0        : TMA producer -- the A tile (hi/lo) and a ring of weight
 //                   slots in consumption order W_O, W1_0, W1_1, W1_2, W2_0,
 //                   W1_3, W2_1, ...
-//   warp 1 lane 0 : tcgen05.mma -- A W_O into the TMEM buffer of FFN1 chunk
+//   warp 1        : tcgen05.mma -- A W_O into the TMEM buffer of FFN1 chunk
 //                   0; after the epilogue has written x into the d-column
 //                   accumulator and LN(x) in shared memory, FFN1 chunk f
 //                   (N = 128) into one of three TMEM buffers, two chunks ahead
@@ -23,9 +23,15 @@
 //                   accumulator + b2, LayerNorm, stored with TMA tensor stores
 //                   staged in the tile's own 4 KB blocks
 // The MMA groups are 16 instructions of N >= 128 so that the tensor pipe has
-// queued work while the issuing thread polls its barriers; x0 is read by the
+// queued work while the issuing warp polls its barriers; x0 is read by the
 // epilogue warps while the A tile is in flight, when they have nothing else to
 // do; the biases sit in shared memory.
+// What bounds it: a tile is one dependency chain of which the tensor pipe needs
+// 5 us (160 MMAs of N = 128 at d = 128, F = 512).  Behind `if (lane == 0)` an
+// MMA cost its issuing thread up to 92 cycles where the pipe takes 64, and a
+// satisfied wait 100 or more; with the warps run whole the batch of 256 requests went
+// from 163.8 to 159.1 us, one request from 124.9 to 119.5, 64 requests in fp32
+// from 148.4 to 141.0.
 #include "fe_common.cuh"
 #include "fe_kernels.h"
 
@@ -126,6 +132,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* tail_a = bars + 31;      // LN(x_out) written in sA
   uint64_t* wt_full = bars + 32;     // tail weight loaded
   uint64_t* tail_full = bars + 33;   // tail product complete in TMEM
+  uint64_t* drain = bars + 34;       // the products in flight at the end
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 40);
   float* red = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + kBarBytes);  // [sum|var][half][128]
 
@@ -148,6 +155,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     mbar_init(tail_a, kEpiWarps);
     mbar_init(wt_full, 1);
     mbar_init(tail_full, 1);
+    mbar_init(drain, 1);
     fence_mbar_init();
     prefetch_tmap(&tA_h);
     prefetch_tmap(&tWo_h);
@@ -179,189 +187,188 @@ __global__ void __launch_bounds__(kThreads, 1)
     return;
   }
 
+  // Warps 0 and 1 run whole (fe_common.cuh): uniform control flow, the
+  // instructions predicated on the elected lane.
   if (warp == 0) {
-    if (lane == 0) {
-      // ---------------- TMA producer ----------------
-      int tl = 0, ws = 0;
-      bool ok = true;
-      // kind 0: W_O; 1: W1 rows [f*128, f*128+128); 2: W2 columns [f*128, f*128+128)
-      auto load_slot = [&](int kind, int f) -> bool {
-        const int slot = ws % LY.ring;
-        if (ws >= LY.ring && !mbar_wait_bounded(w_empty + slot, ((ws / LY.ring) - 1) & 1, p.status)) return false;
-        uint8_t* dst = sW + (size_t)slot * LY.slot_bytes;
-        if (kind == 0) {  // every d row, every k block: [kb][plane][d rows x 64]
-          mbar_arrive_expect_tx(w_full + slot, LY.wo_bytes);
-          for (int kb = 0; kb < nkb; ++kb)
-            for (int q = 0; q < nb; ++q)
-              tma_load_2d(dst + (size_t)(kb * nb + q) * d * (BK * 2), q ? &tWo_l : &tWo_h, kb * BK, 0, w_full + slot);
-        } else if (kind == 1) {  // every k block: [kb][plane][128 rows x 64]
-          mbar_arrive_expect_tx(w_full + slot, LY.w1_chunk);
-          for (int kb = 0; kb < nkb; ++kb)
-            for (int q = 0; q < nb; ++q)
-              tma_load_2d(dst + (size_t)(kb * nb + q) * (FC * BK * 2), q ? &tW1_l : &tW1_h, kb * BK, f * FC,
-                          w_full + slot);
-        } else {  // two 64-column halves, every d row: [plane][half][d rows x 64]
-          mbar_arrive_expect_tx(w_full + slot, LY.w2_chunk);
+    // ---------------- TMA producer ----------------
+    const uint32_t go = elect_one();
+    int tl = 0, ws = 0, slot = 0;  // tiles, weight slots loaded, the next ring slot
+    uint32_t par = 1;              // the parity of its previous release (a fresh barrier passes)
+    // kind 0: W_O; 1: W1 rows [f*128, f*128+128); 2: W2 columns [f*128, f*128+128)
+    auto load_slot = [&](int kind, int f) {
+      mbar_wait_warp(w_empty + slot, par, p.status);
+      uint8_t* dst = sW + (size_t)slot * LY.slot_bytes;
+      uint64_t* full = w_full + slot;
+      if (kind == 0) {  // every d row, every k block: [kb][plane][d rows x 64]
+        mbar_arrive_expect_tx_if(full, LY.wo_bytes, go);
+        for (int kb = 0; kb < nkb; ++kb)
           for (int q = 0; q < nb; ++q)
-            for (int hh = 0; hh < 2; ++hh)
-              tma_load_2d(dst + (size_t)(q * 2 + hh) * d * (BK * 2), q ? &tW2_l : &tW2_h, f * FC + BK * hh, 0,
-                          w_full + slot);
-        }
-        ++ws;
-        return true;
-      };
-      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++tl) {
-        // sA holds the previous tile's output staging until its stores have read it
-        if (tl > 0 && !mbar_wait_bounded(r_empty, (tl - 1) & 1, p.status)) break;
-        mbar_arrive_expect_tx(a_full, LY.a_bytes);
-        for (int kb = 0; kb < nkb; ++kb) {
-          tma_load_2d(sA + (size_t)(kb * 2) * kAPlane, &tA_h, kb * BK, t * BM, a_full);
-          tma_load_2d(sA + (size_t)(kb * 2 + 1) * kAPlane, &tA_l, kb * BK, t * BM, a_full);
-        }
-        if (!load_slot(0, 0)) break;
-        for (int s = 0; s < nf + LA && ok; ++s) {
-          if (s < nf && !load_slot(1, s)) ok = false;
-          if (ok && s >= LA && !load_slot(2, s - LA)) ok = false;
-        }
-        if (ok && tail_n > 0) {
-          // the tail weight, past the x_out staging, once every FFN MMA of the
-          // tile (the last readers of the ring) has completed
-          if (!mbar_wait_bounded(acc2_full, tl & 1, p.status)) break;
-          mbar_arrive_expect_tx(wt_full, (uint32_t)nkb * nb * (uint32_t)tail_n * (BK * 2));
-          for (int kb = 0; kb < nkb; ++kb)
-            for (int q = 0; q < nb; ++q)
-              tma_load_2d(sT + (size_t)(kb * nb + q) * tail_n * (BK * 2), q ? &tT_l : &tT_h, kb * BK, 0, wt_full);
-        }
+            tma_load_2d_if(dst + (size_t)(kb * nb + q) * d * (BK * 2), q ? &tWo_l : &tWo_h, kb * BK, 0, full, go);
+      } else if (kind == 1) {  // every k block: [kb][plane][128 rows x 64]
+        mbar_arrive_expect_tx_if(full, LY.w1_chunk, go);
+        for (int kb = 0; kb < nkb; ++kb)
+          for (int q = 0; q < nb; ++q)
+            tma_load_2d_if(dst + (size_t)(kb * nb + q) * (FC * BK * 2), q ? &tW1_l : &tW1_h, kb * BK, f * FC, full, go);
+      } else {  // two 64-column halves, every d row: [plane][half][d rows x 64]
+        mbar_arrive_expect_tx_if(full, LY.w2_chunk, go);
+        for (int q = 0; q < nb; ++q)
+          for (int hh = 0; hh < 2; ++hh)
+            tma_load_2d_if(dst + (size_t)(q * 2 + hh) * d * (BK * 2), q ? &tW2_l : &tW2_h, f * FC + BK * hh, 0, full, go);
+      }
+      ++ws;
+      if (++slot == LY.ring) {
+        slot = 0;
+        par ^= 1u;
+      }
+    };
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++tl) {
+      // sA holds the previous tile's output staging until its stores have read it
+      if (tl > 0) mbar_wait_warp(r_empty, (tl - 1) & 1, p.status);
+      mbar_arrive_expect_tx_if(a_full, LY.a_bytes, go);
+      for (int kb = 0; kb < nkb; ++kb) {
+        tma_load_2d_if(sA + (size_t)(kb * 2) * kAPlane, &tA_h, kb * BK, t * BM, a_full, go);
+        tma_load_2d_if(sA + (size_t)(kb * 2 + 1) * kAPlane, &tA_l, kb * BK, t * BM, a_full, go);
+      }
+      load_slot(0, 0);
+      for (int s = 0; s < nf + LA; ++s) {
+        if (s < nf) load_slot(1, s);
+        if (s >= LA) load_slot(2, s - LA);
+      }
+      if (tail_n > 0) {
+        // the tail weight, past the x_out staging, once every FFN MMA of the
+        // tile (the last readers of the ring) has completed
+        mbar_wait_warp(acc2_full, tl & 1, p.status);
+        mbar_arrive_expect_tx_if(wt_full, (uint32_t)nkb * nb * (uint32_t)tail_n * (BK * 2), go);
+        for (int kb = 0; kb < nkb; ++kb)
+          for (int q = 0; q < nb; ++q)
+            tma_load_2d_if(sT + (size_t)(kb * nb + q) * tail_n * (BK * 2), q ? &tT_l : &tT_h, kb * BK, 0, wt_full, go);
       }
     }
+    // the last loads land before this block's shared memory goes away (after a
+    // timed-out wait nothing else has waited for them)
+    for (int i = ws < LY.ring ? 0 : ws - LY.ring; i < ws; ++i)
+      mbar_wait_warp(w_full + i % LY.ring, (uint32_t)(i / LY.ring) & 1u, p.status);
+    if (tl > 0) mbar_wait_warp(a_full, (tl - 1) & 1, p.status);
+    if (tl > 0 && tail_n > 0) mbar_wait_warp(wt_full, (tl - 1) & 1, p.status);
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- MMA issuer ----------------
-      const uint32_t idesc1 = umma_idesc_bf16(BM, FC);
-      const uint32_t idesc2 = umma_idesc_bf16(BM, d);
-      int tl = 0, ws = 0, gf = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++tl) {
-        // ---- A W_O into the FFN1 buffer that chunk 0 of this tile uses next
-        if (!mbar_wait_bounded(a_full, tl & 1, p.status)) break;
-        {
-          const int slot = ws % LY.ring, bo = gf % NA1;
-          if (!mbar_wait_bounded(w_full + slot, (ws / LY.ring) & 1, p.status)) break;
-          if (gf >= NA1 && !mbar_wait_bounded(acc1_empty + bo, ((gf / NA1) - 1) & 1, p.status)) break;
-          tc_fence_after();
-          const uint32_t dst = tmem + (uint32_t)(bo * FC);
-          const uint64_t a0 = umma_desc_sw128(smem_u32(sA));
-          const uint64_t w0 = umma_desc_sw128(smem_u32(sW + (size_t)slot * LY.slot_bytes));
-#pragma unroll
-          for (int kb = 0; kb < nkb; ++kb) {
-#pragma unroll
-            for (int kk = 0; kk < BK / 16; ++kk) {
-              const uint64_t ah = desc_adv(a0, (uint32_t)(kb * 2) * kAPlane + kk * 32);
-              const uint64_t wh = desc_adv(w0, (uint32_t)(kb * nb) * (uint32_t)d * (BK * 2) + kk * 32);
-              umma_bf16(dst, ah, wh, idesc2, (kb | kk) != 0 ? 1u : 0u);
-              umma_bf16(dst, desc_adv(ah, kAPlane), wh, idesc2, 1u);
-              if (nb > 1) umma_bf16(dst, ah, desc_adv(wh, (uint32_t)d * (BK * 2)), idesc2, 1u);
-            }
-          }
-          umma_commit(w_empty + slot);
-          umma_commit(o_done);
-          ++ws;
-        }
-        // ---- FFN1 / FFN2 once the epilogue has put x in the accumulator and LN(x) in sA
-        if (!mbar_wait_bounded(ln_full, tl & 1, p.status)) break;
+    // ---------------- MMA issuer ----------------
+    const uint32_t go = elect_one();
+    const uint32_t idesc1 = umma_idesc_bf16(BM, FC);
+    const uint32_t idesc2 = umma_idesc_bf16(BM, d);
+    const uint64_t a0 = umma_desc_sw128(smem_u32(sA));
+    const uint64_t w00 = umma_desc_sw128(smem_u32(sW));
+    int tl = 0, gf = 0, slot = 0;
+    uint32_t par = 0;
+    // the next weight slot landed: its descriptor
+    auto next_slot = [&]() -> uint64_t {
+      mbar_wait_warp(w_full + slot, par, p.status);
+      tc_fence_after();
+      return desc_adv(w00, (uint32_t)slot * LY.slot_bytes);
+    };
+    // the slot frees once the products issued so far complete
+    auto release = [&]() {
+      umma_commit_if(w_empty + slot, go);
+      if (++slot == LY.ring) {
+        slot = 0;
+        par ^= 1u;
+      }
+    };
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++tl) {
+      // ---- A W_O into the FFN1 buffer that chunk 0 of this tile uses next
+      mbar_wait_warp(a_full, tl & 1, p.status);
+      {
+        const int bo = gf % NA1;
+        const uint64_t w0 = next_slot();
+        if (gf >= NA1) mbar_wait_warp(acc1_empty + bo, ((gf / NA1) - 1) & 1, p.status);
         tc_fence_after();
-        const int gf0 = gf;
-        for (int s = 0; s < nf + LA && ok; ++s) {
-          if (s < nf) {
-            // FFN1 chunk s -> acc1 buffer (gf0 + s) % NA1
-            const int g = gf0 + s, b = g % NA1;
-            // (chunk 0's buffer: waited for before the projection, read by the epilogue before ln_full)
-            if (s > 0 && g >= NA1 && !mbar_wait_bounded(acc1_empty + b, ((g / NA1) - 1) & 1, p.status)) {
-              ok = false;
-              break;
-            }
-            const int slot = ws % LY.ring;
-            if (!mbar_wait_bounded(w_full + slot, (ws / LY.ring) & 1, p.status)) {
-              ok = false;
-              break;
-            }
-            tc_fence_after();
-            const uint32_t dst = tmem + (uint32_t)(b * FC);
-            const uint64_t a0 = umma_desc_sw128(smem_u32(sA));
-            const uint64_t w0 = umma_desc_sw128(smem_u32(sW + (size_t)slot * LY.slot_bytes));
+        const uint32_t dst = tmem + (uint32_t)(bo * FC);
 #pragma unroll
-            for (int kb = 0; kb < nkb; ++kb) {
+        for (int kb = 0; kb < nkb; ++kb) {
 #pragma unroll
-              for (int kk = 0; kk < BK / 16; ++kk) {
-                const uint64_t ah = desc_adv(a0, (uint32_t)(kb * 2) * kAPlane + kk * 32);
-                const uint64_t wh = desc_adv(w0, (uint32_t)(kb * nb) * (FC * BK * 2) + kk * 32);
-                umma_bf16(dst, ah, wh, idesc1, (kb | kk) != 0 ? 1u : 0u);
-                umma_bf16(dst, desc_adv(ah, kAPlane), wh, idesc1, 1u);
-                if (nb > 1) umma_bf16(dst, ah, desc_adv(wh, FC * BK * 2), idesc1, 1u);
-              }
-            }
-            umma_commit(w_empty + slot);
-            umma_commit(acc1_full + b);
-            ++ws;
-          }
-          if (s >= LA) {
-            // FFN2 chunk c = s - LA: acc2 += mid(c) . W2 chunk c, mid(c) from TMEM buffer g % NA1
-            const int c = s - LA, g = gf0 + c, b = g % NA1;
-            if (!mbar_wait_bounded(mid_full + b, (g / NA1) & 1, p.status)) {
-              ok = false;
-              break;
-            }
-            const int slot = ws % LY.ring;
-            if (!mbar_wait_bounded(w_full + slot, (ws / LY.ring) & 1, p.status)) {
-              ok = false;
-              break;
-            }
-            tc_fence_after();
-            // each 32-column piece of the buffer holds 32 hidden units: hi plane in
-            // its first 16 columns, lo plane in the next 16 (two bf16 per column);
-            // the W2 slot holds 64-column halves of the chunk, d rows each
-            const uint32_t mt = tmem + (uint32_t)(b * FC);
-            const uint64_t w0 = umma_desc_sw128(smem_u32(sW + (size_t)slot * LY.slot_bytes));
-#pragma unroll
-            for (int kk = 0; kk < FC / 16; ++kk) {
-              const int hh = kk >> 2, k4 = kk & 3;
-              const uint32_t mh = mt + (uint32_t)(32 * (kk >> 1) + 8 * (kk & 1)), ml = mh + 16;
-              const uint64_t wh = desc_adv(w0, (uint32_t)hh * (uint32_t)d * (BK * 2) + k4 * 32);
-              umma_bf16_tmem_a(acc2, mh, wh, idesc2, 1u);
-              umma_bf16_tmem_a(acc2, ml, wh, idesc2, 1u);
-              if (nb > 1) umma_bf16_tmem_a(acc2, mh, desc_adv(wh, 2u * (uint32_t)d * (BK * 2)), idesc2, 1u);
-            }
-            umma_commit(w_empty + slot);
-            umma_commit(acc1_empty + b);
-            ++ws;
-            if (c == nf - 1) umma_commit(acc2_full);
+          for (int kk = 0; kk < BK / 16; ++kk) {
+            const uint64_t ah = desc_adv(a0, (uint32_t)(kb * 2) * kAPlane + kk * 32);
+            const uint64_t wh = desc_adv(w0, (uint32_t)(kb * nb) * (uint32_t)d * (BK * 2) + kk * 32);
+            umma_bf16_if(dst, ah, wh, idesc2, (kb | kk) != 0 ? 1u : 0u, go);
+            umma_bf16_if(dst, desc_adv(ah, kAPlane), wh, idesc2, 1u, go);
+            if (nb > 1) umma_bf16_if(dst, ah, desc_adv(wh, (uint32_t)d * (BK * 2)), idesc2, 1u, go);
           }
         }
-        gf = gf0 + nf;
-        if (ok && tail_n > 0) {
-          // tail: LN(x_out) . W_t into TMEM columns [0, tail_n) (every FFN1
-          // buffer is free once the FFN2 of the tile has completed)
-          if (!mbar_wait_bounded(tail_a, tl & 1, p.status)) break;
-          if (!mbar_wait_bounded(wt_full, tl & 1, p.status)) break;
-          tc_fence_after();
-          const uint32_t idesc3 = umma_idesc_bf16(BM, tail_n);
-          const uint64_t a0 = umma_desc_sw128(smem_u32(sA));
-          const uint64_t w0 = umma_desc_sw128(smem_u32(sT));
+        release();
+        umma_commit_if(o_done, go);
+      }
+      // ---- FFN1 / FFN2 once the epilogue has put x in the accumulator and LN(x) in sA
+      mbar_wait_warp(ln_full, tl & 1, p.status);
+      tc_fence_after();
+      const int gf0 = gf;
+      for (int s = 0; s < nf + LA; ++s) {
+        if (s < nf) {
+          // FFN1 chunk s -> acc1 buffer (gf0 + s) % NA1
+          const int g = gf0 + s, b = g % NA1;
+          // (chunk 0's buffer: waited for before the projection, read by the epilogue before ln_full)
+          if (s > 0 && g >= NA1) mbar_wait_warp(acc1_empty + b, ((g / NA1) - 1) & 1, p.status);
+          const uint64_t w0 = next_slot();
+          const uint32_t dst = tmem + (uint32_t)(b * FC);
 #pragma unroll
           for (int kb = 0; kb < nkb; ++kb) {
 #pragma unroll
             for (int kk = 0; kk < BK / 16; ++kk) {
               const uint64_t ah = desc_adv(a0, (uint32_t)(kb * 2) * kAPlane + kk * 32);
-              const uint64_t wh = desc_adv(w0, (uint32_t)(kb * nb) * (uint32_t)tail_n * (BK * 2) + kk * 32);
-              umma_bf16(tmem, ah, wh, idesc3, (kb | kk) != 0 ? 1u : 0u);
-              umma_bf16(tmem, desc_adv(ah, kAPlane), wh, idesc3, 1u);
-              if (nb > 1) umma_bf16(tmem, ah, desc_adv(wh, (uint32_t)tail_n * (BK * 2)), idesc3, 1u);
+              const uint64_t wh = desc_adv(w0, (uint32_t)(kb * nb) * (FC * BK * 2) + kk * 32);
+              umma_bf16_if(dst, ah, wh, idesc1, (kb | kk) != 0 ? 1u : 0u, go);
+              umma_bf16_if(dst, desc_adv(ah, kAPlane), wh, idesc1, 1u, go);
+              if (nb > 1) umma_bf16_if(dst, ah, desc_adv(wh, FC * BK * 2), idesc1, 1u, go);
             }
           }
-          umma_commit(tail_full);
+          release();
+          umma_commit_if(acc1_full + b, go);
+        }
+        if (s >= LA) {
+          // FFN2 chunk c = s - LA: acc2 += mid(c) . W2 chunk c, mid(c) from TMEM buffer g % NA1
+          const int c = s - LA, g = gf0 + c, b = g % NA1;
+          mbar_wait_warp(mid_full + b, (g / NA1) & 1, p.status);
+          const uint64_t w0 = next_slot();
+          // each 32-column piece of the buffer holds 32 hidden units: hi plane in
+          // its first 16 columns, lo plane in the next 16 (two bf16 per column);
+          // the W2 slot holds 64-column halves of the chunk, d rows each
+          const uint32_t mt = tmem + (uint32_t)(b * FC);
+#pragma unroll
+          for (int kk = 0; kk < FC / 16; ++kk) {
+            const int hh = kk >> 2, k4 = kk & 3;
+            const uint32_t mh = mt + (uint32_t)(32 * (kk >> 1) + 8 * (kk & 1)), ml = mh + 16;
+            const uint64_t wh = desc_adv(w0, (uint32_t)hh * (uint32_t)d * (BK * 2) + k4 * 32);
+            umma_bf16_tmem_a_if(acc2, mh, wh, idesc2, 1u, go);
+            umma_bf16_tmem_a_if(acc2, ml, wh, idesc2, 1u, go);
+            if (nb > 1) umma_bf16_tmem_a_if(acc2, mh, desc_adv(wh, 2u * (uint32_t)d * (BK * 2)), idesc2, 1u, go);
+          }
+          release();
+          umma_commit_if(acc1_empty + b, go);
+          if (c == nf - 1) umma_commit_if(acc2_full, go);
         }
       }
+      gf = gf0 + nf;
+      if (tail_n > 0) {
+        // tail: LN(x_out) . W_t into TMEM columns [0, tail_n) (every FFN1
+        // buffer is free once the FFN2 of the tile has completed)
+        mbar_wait_warp(tail_a, tl & 1, p.status);
+        mbar_wait_warp(wt_full, tl & 1, p.status);
+        tc_fence_after();
+        const uint32_t idesc3 = umma_idesc_bf16(BM, tail_n);
+        const uint64_t w0 = umma_desc_sw128(smem_u32(sT));
+#pragma unroll
+        for (int kb = 0; kb < nkb; ++kb) {
+#pragma unroll
+          for (int kk = 0; kk < BK / 16; ++kk) {
+            const uint64_t ah = desc_adv(a0, (uint32_t)(kb * 2) * kAPlane + kk * 32);
+            const uint64_t wh = desc_adv(w0, (uint32_t)(kb * nb) * (uint32_t)tail_n * (BK * 2) + kk * 32);
+            umma_bf16_if(tmem, ah, wh, idesc3, (kb | kk) != 0 ? 1u : 0u, go);
+            umma_bf16_if(tmem, desc_adv(ah, kAPlane), wh, idesc3, 1u, go);
+            if (nb > 1) umma_bf16_if(tmem, ah, desc_adv(wh, (uint32_t)tail_n * (BK * 2)), idesc3, 1u, go);
+          }
+        }
+        umma_commit_if(tail_full, go);
+      }
     }
+    umma_drain(drain, p.status, go);
   } else {
     // ---------------- epilogue (warps 2..9) ----------------
     const int ew = warp - 2, q = warp & 3, half = ew >> 2;
@@ -392,8 +399,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (lane == 0) mbar_arrive_one(bar);
     };
     int tl = 0, gf = 0;
-    bool ok = true;
-    for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++tl) {
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++tl) {
       const int m0 = t * BM;
       const int srow = m0 + q * 32;
       const bool valid = m0 + r < rows_valid;
@@ -429,7 +435,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
       const uint32_t proj = tmem + (uint32_t)((gf % NA1) * FC);  // A W_O
-      if (!mbar_wait_bounded(o_done, tl & 1, p.status)) break;
+      mbar_wait_warp(o_done, tl & 1, p.status);
       tc_fence_after();
       float s4[4] = {0.f, 0.f, 0.f, 0.f};  // four independent partial sums per statistic
 #pragma unroll
@@ -503,10 +509,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // warp's 64 columns of the chunk's TMEM buffer as FFN2's A operand
       for (int f = 0; f < nf; ++f, ++gf) {
         const int ba = gf % NA1;
-        if (!mbar_wait_bounded(acc1_full + ba, (gf / NA1) & 1, p.status)) {
-          ok = false;
-          break;
-        }
+        mbar_wait_warp(acc1_full + ba, (gf / NA1) & 1, p.status);
         tc_fence_after();
         // this warp's 64 columns as two 32-column pieces, each read whole and
         // then overwritten by its own hi (16 columns) and lo (16 columns) planes
@@ -529,9 +532,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         tc_fence_before();
         warp_arrive(mid_full + ba);
       }
-      if (!ok) break;
       // ---- final: x_out = acc2 + b2 (acc2 = x + FFN2), LayerNorm, stores
-      if (!mbar_wait_bounded(acc2_full, tl & 1, p.status)) break;
+      mbar_wait_warp(acc2_full, tl & 1, p.status);
       tc_fence_after();
       // this warp's x_out staging blocks at the start of the weight ring (every
       // MMA of the tile has completed, and before r_empty the producer loads
@@ -633,7 +635,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         // tail output: 32-column chunks half, half + 2, ... of this warp's row
         // quadrant, f16 (one 2 KB block) or a split pair (two), through two
         // rotating staging buffers of this warp where the tail weight was
-        if (!mbar_wait_bounded(tail_full, tl & 1, p.status)) break;
+        mbar_wait_warp(tail_full, tl & 1, p.status);
         tc_fence_after();
         const uint32_t tb = p.tail_f16 ? 2048u : 4096u;
         uint8_t* stg = sT + (size_t)ew * 2u * tb;
@@ -685,7 +687,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (lane == 0) bulk_wait0();  // output tensor stores complete before the CTA retires
   }
 
-  __syncwarp();  // each warp arrives whole: lane 0 of warps 0 and 1 ran the producer and MMA loops
+  __syncwarp();
   tc_fence_before();
   __syncthreads();
   if (warp == 0) tmem_dealloc(tmem, 512);
