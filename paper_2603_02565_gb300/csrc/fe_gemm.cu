@@ -6,13 +6,17 @@
 // K (d or F).  The kernel is persistent and warp-specialised; each CTA walks
 // 128-row x BN-column tiles (column tile fastest, so concurrently running CTAs
 // share activation rows in L2):
-//   warp 0 lane 0  : TMA producer, a ring of shared-memory stages that runs
+//   warp 0         : TMA producer, a ring of shared-memory stages that runs
 //                    ahead across tile boundaries
-//   warp 1 lane 0  : tcgen05.mma issuer into one of two TMEM accumulators
+//   warp 1         : tcgen05.mma issuer into one of two TMEM accumulators
 //   warps 2-9      : epilogue of the previous tile while the next one is
 //                    multiplied; warps w and w+4 share TMEM lane quadrant
 //                    w % 4 (tile rows (w % 4) * 32 + lane) and take
 //                    alternate 32-column chunks
+// The loading and the issuing warp run whole (fe_common.cuh): at two to four
+// MMAs of N >= 128 per 64-wide k step the issuing thread, not the tensor pipe, set
+// the pace (d = 512 summarisation batch 679 -> 631 us, 64 requests in fp32 140.9 ->
+// 137.7).
 // The activation is a split pair (hi + lo bf16); the product is
 // A_hi W_hi + A_lo W_hi (+ A_hi W_lo when the weights carry a lo plane).
 #include <cstdlib>
@@ -112,14 +116,14 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t pa
   return ok != 0;
 }
 // bounded like mbar_wait_bounded, acquiring at cluster scope (the peers' stores)
-__device__ __noinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, int* status) {
+__device__ __noinline__ void mbar_wait_cluster(uint64_t* bar, uint32_t parity, int* status) {
   const uint64_t t0 = globaltimer_ns();
   for (uint32_t it = 0;; ++it) {
-    if (mbar_try_wait_cluster(bar, parity)) return true;
-    if ((it & 255u) == 255u && (*reinterpret_cast<volatile int*>(status) & ST_TIMEOUT)) return false;
+    if (mbar_try_wait_cluster(bar, parity)) return;
+    if ((it & 255u) == 255u && (*reinterpret_cast<volatile int*>(status) & ST_TIMEOUT)) return;
     if (globaltimer_ns() - t0 > kWaitLimitNs) {
       atomicOr(status, ST_TIMEOUT);
-      return false;
+      return;
     }
   }
 }
@@ -149,7 +153,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* tfull = empty + S;  // [2] accumulator ready for the epilogue
   uint64_t* tempty = tfull + 2; // [2] accumulator drained by the epilogue
   uint64_t* xbar = tempty + 2;  // [2] cluster row exchange: partial sums / partial variances received
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(xbar + 2);
+  uint64_t* drain = xbar + 2;   // the products in flight at the end
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(xbar + 3);
   // output staging: two 4 KB buffers per epilogue warp, 1024-byte aligned; then
   // the row-reduction exchange of the two warps sharing a lane quadrant
   uint8_t* stg_base = smem + (((size_t)S * stage_bytes + 256 + 1023) & ~(size_t)1023);
@@ -168,6 +173,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(tfull + a, 1);
       mbar_init(tempty + a, kEpiWarps);  // one arrival per epilogue warp
     }
+    mbar_init(drain, 1);
     if (cs > 1) {
       mbar_init(xbar, 1);  // the local expect_tx; the peers' stores complete the bytes
       mbar_init(xbar + 1, 1);
@@ -200,71 +206,74 @@ __global__ void __launch_bounds__(kThreads, 1)
     return;
   }
 
+  // Warps 0 and 1 run whole (fe_common.cuh): uniform control flow, the
+  // instructions predicated on the elected lane.
   if (warp == 0) {
-    if (lane == 0) {
-      // ---------------- TMA producer ----------------
-      int it = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
-        const int m0 = (t / nt) * BM, n0 = (t % nt) * BN;
-        for (int kb = 0; kb < nk; ++kb, ++it) {
-          const int s = it % S;
-          if (it >= S && !mbar_wait_bounded(empty + s, ((it / S) & 1) ^ 1, p.status)) {
-            ok = false;
-            break;
-          }
-          uint8_t* st = smem + (size_t)s * stage_bytes;
-          mbar_arrive_expect_tx(full + s, stage_bytes);
-          tma_load_2d(st, &tA_h, kb * BK, m0, full + s);
-          if (NA > 1) tma_load_2d(st + kATile, &tA_l, kb * BK, m0, full + s);
-          for (int q = 0; q < nb; ++q) {
-            const CUtensorMap* tb = q ? &tB_l : &tB_h;
-            for (int h = 0; h < BN; h += 256)
-              tma_load_2d(st + NA * kATile + q * b_bytes + (uint32_t)h * BK * 2, tb, kb * BK, n0 + h, full + s);
-          }
+    // ---------------- TMA producer ----------------
+    const uint32_t go = elect_one();
+    int it = 0, st_i = 0;  // k blocks loaded, the next stage
+    uint32_t par = 1;      // the parity of its previous release (a fresh barrier passes)
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
+      const int m0 = (t / nt) * BM, n0 = (t % nt) * BN;
+      for (int kb = 0; kb < nk; ++kb, ++it) {
+        mbar_wait_warp(empty + st_i, par, p.status);
+        uint8_t* st = smem + (size_t)st_i * stage_bytes;
+        mbar_arrive_expect_tx_if(full + st_i, stage_bytes, go);
+        tma_load_2d_if(st, &tA_h, kb * BK, m0, full + st_i, go);
+        if (NA > 1) tma_load_2d_if(st + kATile, &tA_l, kb * BK, m0, full + st_i, go);
+        for (int q = 0; q < nb; ++q) {
+          const CUtensorMap* tb = q ? &tB_l : &tB_h;
+          for (int h = 0; h < BN; h += 256)
+            tma_load_2d_if(st + NA * kATile + q * b_bytes + (uint32_t)h * BK * 2, tb, kb * BK, n0 + h, full + st_i, go);
+        }
+        if (++st_i == S) {
+          st_i = 0;
+          par ^= 1u;
         }
       }
     }
+    // the last loads land before this block's shared memory goes away (after a
+    // timed-out wait nothing else has waited for them)
+    for (int i = it < S ? 0 : it - S; i < it; ++i) mbar_wait_warp(full + i % S, (uint32_t)(i / S) & 1u, p.status);
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- MMA issuer ----------------
-      const int nmma = BN > 256 ? 256 : BN;
-      const uint32_t idesc = umma_idesc_bf16(BM, nmma);
-      int it = 0, tl = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++tl) {
-        const int acc = tl % nacc, use = tl / nacc;
-        if (use > 0 && !mbar_wait_bounded(tempty + acc, (use - 1) & 1, p.status)) break;
+    // ---------------- MMA issuer ----------------
+    const uint32_t go = elect_one();
+    const int nmma = BN > 256 ? 256 : BN;
+    const uint32_t idesc = umma_idesc_bf16(BM, nmma);
+    const uint64_t sd0 = umma_desc_sw128(smem_u32(smem));
+    int tl = 0, st_i = 0;
+    uint32_t par = 0;
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++tl) {
+      const int acc = tl % nacc, use = tl / nacc;
+      if (use > 0) mbar_wait_warp(tempty + acc, (use - 1) & 1, p.status);
+      const uint32_t dst = tmem + (uint32_t)(acc * BN);
+      for (int kb = 0; kb < nk; ++kb) {
+        mbar_wait_warp(full + st_i, par, p.status);
         tc_fence_after();
-        const uint32_t dst = tmem + (uint32_t)(acc * BN);
-        for (int kb = 0; kb < nk; ++kb, ++it) {
-          const int s = it % S;
-          if (!mbar_wait_bounded(full + s, (it / S) & 1, p.status)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t st = smem_u32(smem + (size_t)s * stage_bytes);
-          // descriptors built once per stage; the k steps only add 32-byte offsets
-          const uint64_t ah0 = umma_desc_sw128(st), al0 = umma_desc_sw128(st + kATile);
-          const uint64_t bh0 = umma_desc_sw128(st + NA * kATile), bl0 = umma_desc_sw128(st + NA * kATile + b_bytes);
-          for (int h = 0; h < BN; h += 256) {
-            const uint32_t hb = (uint32_t)h * BK * 2;
+        // descriptors built once per stage; the k steps only add 32-byte offsets
+        const uint64_t ah0 = desc_adv(sd0, (uint32_t)st_i * stage_bytes), al0 = desc_adv(ah0, kATile);
+        const uint64_t bh0 = desc_adv(ah0, NA * kATile), bl0 = desc_adv(bh0, b_bytes);
+        for (int h = 0; h < BN; h += 256) {
+          const uint32_t hb = (uint32_t)h * BK * 2;
 #pragma unroll
-            for (int kk = 0; kk < BK / 16; ++kk) {
-              // (A_hi, W_hi), (A_lo, W_hi), (A_hi, W_lo)
-              const uint64_t ah = desc_adv(ah0, kk * 32), al = desc_adv(al0, kk * 32);
-              const uint64_t bh = desc_adv(bh0, hb + kk * 32);
-              umma_bf16(dst + (uint32_t)h, ah, bh, idesc, (kb | kk) != 0 ? 1u : 0u);
-              if (NA > 1) umma_bf16(dst + (uint32_t)h, al, bh, idesc, 1u);
-              if (nb > 1) umma_bf16(dst + (uint32_t)h, ah, desc_adv(bl0, hb + kk * 32), idesc, 1u);
-            }
+          for (int kk = 0; kk < BK / 16; ++kk) {
+            // (A_hi, W_hi), (A_lo, W_hi), (A_hi, W_lo)
+            const uint64_t ah = desc_adv(ah0, kk * 32), al = desc_adv(al0, kk * 32);
+            const uint64_t bh = desc_adv(bh0, hb + kk * 32);
+            umma_bf16_if(dst + (uint32_t)h, ah, bh, idesc, (kb | kk) != 0 ? 1u : 0u, go);
+            if (NA > 1) umma_bf16_if(dst + (uint32_t)h, al, bh, idesc, 1u, go);
+            if (nb > 1) umma_bf16_if(dst + (uint32_t)h, ah, desc_adv(bl0, hb + kk * 32), idesc, 1u, go);
           }
-          umma_commit(empty + s);  // frees this stage once its MMAs complete
         }
-        umma_commit(tfull + acc);  // accumulator complete (or abandoned after a timeout)
+        umma_commit_if(empty + st_i, go);  // frees this stage once its MMAs complete
+        if (++st_i == S) {
+          st_i = 0;
+          par ^= 1u;
+        }
       }
+      umma_commit_if(tfull + acc, go);  // accumulator complete
     }
+    umma_drain(drain, p.status, go);
   } else {
     // ---------------- epilogue (warps 2..9) ----------------
     const int ew = warp - 2;     // 0..7
@@ -319,17 +328,17 @@ __global__ void __launch_bounds__(kThreads, 1)
     // the current ones, so one area per kind suffices.
     int tl = 0;
     const uint32_t my_rank = cs > 1 ? cluster_rank() : 0u;
-    auto row_xchg = [&](int kind, float v, float& tot) -> bool {
+    auto row_xchg = [&](int kind, float v, float& tot) {
       float* xs = red + (size_t)kind * cs * 256;
       const uint32_t slot = smem_u32(xs + (my_rank * 2 + half) * 128 + r);
       const uint32_t bar = smem_u32(xbar + kind);
       for (int k = 0; k < cs; ++k) st_async_peer(map_peer(slot, (uint32_t)k), v, map_peer(bar, (uint32_t)k));
       if (ew == 0 && lane == 0) mbar_arrive_expect_tx(xbar + kind, (uint32_t)cs * 1024u);
-      if (!mbar_wait_cluster(xbar + kind, (uint32_t)tl & 1u, p.status)) return false;
+      mbar_wait_cluster(xbar + kind, (uint32_t)tl & 1u, p.status);
+      __syncwarp();
       float a = 0.f;
       for (int k = 0; k < cs; ++k) a += xs[(2 * k) * 128 + r] + xs[(2 * k + 1) * 128 + r];
       tot = a;
-      return true;
     };
 
     float xr[64];  // EPI_RESID_LN with BN <= 128: this warp's chunks of the row
@@ -355,7 +364,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         }
       }
-      if (!mbar_wait_bounded(tfull + acc, use & 1, p.status)) break;
+      mbar_wait_warp(tfull + acc, use & 1, p.status);
       tc_fence_after();
       const int srow = m0 + q * 32;
       const uint32_t trow = tmem + (uint32_t)(acc * BN) + ((uint32_t)(q * 32) << 16);
@@ -455,7 +464,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         float mean, rstd, tot = 0.f;
         if (cs > 1) {
-          if (!row_xchg(0, sum, tot)) break;
+          row_xchg(0, sum, tot);
           mean = tot / (float)p.N;
         } else {
           red_sum[half * 128 + r] = sum;
@@ -474,7 +483,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         }
         if (cs > 1) {
-          if (!row_xchg(1, var, tot)) break;
+          row_xchg(1, var, tot);
           rstd = 1.0f / sqrtf(tot / (float)p.N + p.eps);
         } else {
           red_var[half * 128 + r] = var;
@@ -603,8 +612,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         float tot[4] = {0.f, 0.f, 0.f, 0.f};
         if (cs > 1) {
           // every warp's partial dot of task 0 (and 1) into every CTA of the cluster
-          if (!row_xchg(0, acc4[0], tot[0])) break;
-          if (nt > 1 && !row_xchg(1, acc4[1], tot[1])) break;
+          row_xchg(0, acc4[0], tot[0]);
+          if (nt > 1) row_xchg(1, acc4[1], tot[1]);
         } else {
           // both halves' partial sums, two tasks per exchange
 #pragma unroll
@@ -651,7 +660,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (lane == 0) bulk_wait0();  // output tensor stores complete before the CTA retires
   }
 
-  __syncwarp();  // each warp arrives whole: single lanes ran the producer and MMA loops
+  __syncwarp();
   tc_fence_before();
   __syncthreads();
   if (cs > 1) cluster_sync_all();  // no peer still stores into this CTA's exchange area
