@@ -17,7 +17,7 @@
 // (128 columns each), then the tail product; the d-column accumulator of x
 // and FFN2 sits at [256, 512).  FFN1 of chunk f runs one chunk ahead of FFN2
 // of chunk f - 1, which reads its A operand (the split ReLU output) from TMEM.
-// Roles: warp 0 lane 0 loads (TMA), warp 1 lane 0 issues tcgen05.mma, warps
+// Roles: warp 0 loads (TMA), warp 1 issues tcgen05.mma, warps
 // 2-9 (two per TMEM lane quadrant, each owning 128 of a row's 256 columns)
 // run the epilogues: x0 + projection, LayerNorm statistics exchanged with the
 // partner warp, LN(x) as the split operand tile over the A tile, bias + ReLU
@@ -26,21 +26,26 @@
 // the A tile, stored by TMA).  Products take split bf16 activations
 // (hi + lo) times exact bf16 weights with fp32 accumulation; LayerNorm and
 // residuals are fp32.
+// What bounds it: the tensor pipe (a chunk is 64 MMAs of N = 128, 4096 cycles, on
+// both halves of its weights) and, per tile, the two LayerNorm phases.  With
+// warps 0 and 1 run whole (fe_common.cuh) the largest batch (295k rows, two element
+// layers and SeqEnc) went from 5495 to 5035 us and 45 requests from 269.5 to 235.5.
 #include "fe_common.cuh"
 #include "fe_kernels.h"
 
 namespace fe {
 
 namespace {
-// TMA 2D load with an L2 cache policy (createpolicy): evict_last for the weight
+// TMA 2D load (predicated on go) with an L2 cache policy (createpolicy): evict_last for the weight
 // boxes that every SM re-reads, evict_first for the activation tiles that
 // stream past them once.
-__device__ __forceinline__ void tma_load_2d_hint(void* smem_dst, const CUtensorMap* map, int x, int y,
-                                                 uint64_t* bar, uint64_t policy) {
+__device__ __forceinline__ void tma_load_2d_hint_if(void* smem_dst, const CUtensorMap* map, int x, int y,
+                                                 uint64_t* bar, uint64_t policy, uint32_t go) {
   asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
-      " [%0], [%1, {%3, %4}], [%2], %5;" ::"r"(smem_u32(smem_dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(x), "r"(y), "l"(policy)
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %6, 0;\n\t"
+      "@q cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+      " [%0], [%1, {%3, %4}], [%2], %5;\n\t}" ::"r"(smem_u32(smem_dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(x), "r"(y), "l"(policy), "r"(go)
       : "memory");
 }
 __device__ __forceinline__ uint64_t l2_policy_evict_last() {
@@ -90,14 +95,15 @@ __device__ __forceinline__ void arrive_one(uint64_t* bar) {
 // dst (+)= (k block of the split A tile: hi plane at sa, lo plane at sa + 16 KB)
 // . (weight box at w)^T, M = N = 128, K = 64: eight products.
 __device__ __noinline__ void mma_box(uint32_t dst, uint32_t sa, uint32_t w, uint32_t idesc, bool acc) {
+  const uint32_t go = elect_one();  // (the lane that the caller's commits elect)
   const uint64_t a0 = umma_desc_sw128(sa);
   const uint64_t w0 = umma_desc_sw128(w);
 #pragma unroll
   for (int kk = 0; kk < BK / 16; ++kk) {
     const uint64_t ah = desc_adv(a0, kk * 32);
     const uint64_t wh = desc_adv(w0, kk * 32);
-    umma_bf16(dst, ah, wh, idesc, (acc || kk != 0) ? 1u : 0u);
-    umma_bf16(dst, desc_adv(ah, kBox), wh, idesc, 1u);
+    umma_bf16_if(dst, ah, wh, idesc, (acc || kk != 0) ? 1u : 0u, go);
+    umma_bf16_if(dst, desc_adv(ah, kBox), wh, idesc, 1u, go);
   }
 }
 
@@ -148,6 +154,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* acc2_full = bars + 20;   // FFN2 of the tile complete
   uint64_t* tail_a = bars + 21;      // LN(x_out) in sA
   uint64_t* tail_full = bars + 22;   // the tail product complete
+  uint64_t* drain = bars + 23;       // the products in flight at the end
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 24);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -169,6 +176,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     mbar_init(acc2_full, 1);
     mbar_init(tail_a, kEpiWarps);
     mbar_init(tail_full, 1);
+    mbar_init(drain, 1);
     fence_mbar_init();
     prefetch_tmap(&tA_h);
     prefetch_tmap(&tWO);
@@ -193,148 +201,138 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (p.rows_dev) rows_valid = min(*p.rows_dev, p.rows);
   const int tiles = (rows_valid + BM - 1) / BM;
 
+  // Warps 0 and 1 run whole (fe_common.cuh): uniform control flow, the
+  // instructions predicated on the elected lane.
   if (warp == 0) {
-    if (lane == 0) {
-      // ---------------- TMA producer ----------------
-      int ws = 0, tl = 0;
-      bool ok = true;
-      // every CTA re-reads the same weight boxes while the activation tiles
-      // stream past once: keep the weights in L2, let the activations go first
-      const uint64_t keep = l2_policy_evict_last(), pass = l2_policy_evict_first();
-      auto load = [&](const CUtensorMap* m, int x, int y) -> bool {
-        const int slot = ws % kRing;
-        if (ws >= kRing && !mbar_wait_compact(w_empty + slot, ((ws / kRing) - 1) & 1, p.status)) return false;
-        mbar_arrive_expect_tx(w_full + slot, kBox);
-        tma_load_2d_hint(sR + (size_t)slot * kBox, m, x, y, w_full + slot, keep);
-        ++ws;
-        return true;
-      };
-      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++tl) {
-        // W_O boxes (kb, nh) in the MMA's order; the first four may load while
-        // the previous tile still uses sA
-        for (int i = 0; i < 2 * NKB && ok; ++i) {
-          if (i == kRing - 1) {
-            if (tl > 0 && !mbar_wait_compact(a_free, (tl - 1) & 1, p.status)) {
-              ok = false;
-              break;
-            }
-            mbar_arrive_expect_tx(a_full, kABytes);
-            for (int kb = 0; kb < NKB; ++kb) {
-              tma_load_2d_hint(sA + (size_t)(kb * 2) * kBox, &tA_h, kb * BK, t * BM, a_full, pass);
-              tma_load_2d_hint(sA + (size_t)(kb * 2 + 1) * kBox, &tA_l, kb * BK, t * BM, a_full, pass);
-            }
-          }
-          if (!load(&tWO, (i >> 1) * BK, (i & 1) * 128)) ok = false;
-        }
-        for (int s = 0; s <= nf && ok; ++s) {
-          if (s < nf)
-            for (int kb = 0; kb < NKB && ok; ++kb)
-              if (!load(&tW1, kb * BK, s * FC)) ok = false;
-          if (s >= 1)
-            for (int i = 0; i < 4 && ok; ++i)  // (nh, sub): sub fastest
-              if (!load(&tW2, (s - 1) * FC + (i & 1) * BK, (i >> 1) * 128)) ok = false;
-        }
-        if (p.tail)
-          for (int i = 0; i < 2 * NKB && ok; ++i)
-            if (!load(&tT, (i >> 1) * BK, (i & 1) * 128)) ok = false;
+    // ---------------- TMA producer ----------------
+    const uint32_t go = elect_one();
+    int ws = 0, slot = 0, tl = 0;
+    uint32_t par = 1;  // the parity of the slot's previous release (a fresh barrier passes)
+    // every CTA re-reads the same weight boxes while the activation tiles
+    // stream past once: keep the weights in L2, let the activations go first
+    const uint64_t keep = l2_policy_evict_last(), pass = l2_policy_evict_first();
+    auto load = [&](const CUtensorMap* m, int x, int y) {
+      mbar_wait_warp(w_empty + slot, par, p.status);
+      mbar_arrive_expect_tx_if(w_full + slot, kBox, go);
+      tma_load_2d_hint_if(sR + (size_t)slot * kBox, m, x, y, w_full + slot, keep, go);
+      ++ws;
+      if (++slot == kRing) {
+        slot = 0;
+        par ^= 1u;
       }
+    };
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++tl) {
+      // W_O boxes (kb, nh) in the MMA's order; the first four may load while
+      // the previous tile still uses sA
+      for (int i = 0; i < 2 * NKB; ++i) {
+        if (i == kRing - 1) {
+          if (tl > 0) mbar_wait_warp(a_free, (tl - 1) & 1, p.status);
+          mbar_arrive_expect_tx_if(a_full, kABytes, go);
+          for (int kb = 0; kb < NKB; ++kb) {
+            tma_load_2d_hint_if(sA + (size_t)(kb * 2) * kBox, &tA_h, kb * BK, t * BM, a_full, pass, go);
+            tma_load_2d_hint_if(sA + (size_t)(kb * 2 + 1) * kBox, &tA_l, kb * BK, t * BM, a_full, pass, go);
+          }
+        }
+        load(&tWO, (i >> 1) * BK, (i & 1) * 128);
+      }
+      for (int s = 0; s <= nf; ++s) {
+        if (s < nf)
+          for (int kb = 0; kb < NKB; ++kb) load(&tW1, kb * BK, s * FC);
+        if (s >= 1)
+          for (int i = 0; i < 4; ++i)  // (nh, sub): sub fastest
+            load(&tW2, (s - 1) * FC + (i & 1) * BK, (i >> 1) * 128);
+      }
+      if (p.tail)
+        for (int i = 0; i < 2 * NKB; ++i) load(&tT, (i >> 1) * BK, (i & 1) * 128);
     }
+    // the last loads land before this block's shared memory goes away (after a
+    // timed-out wait nothing else has waited for them)
+    for (int i = ws < kRing ? 0 : ws - kRing; i < ws; ++i)
+      mbar_wait_warp(w_full + i % kRing, (uint32_t)(i / kRing) & 1u, p.status);
+    if (tl > 0) mbar_wait_warp(a_full, (tl - 1) & 1, p.status);
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- MMA issuer ----------------
-      const uint32_t idesc = umma_idesc_bf16(BM, 128);
-      int ws = 0, tl = 0, gf = 0;
-      bool ok = true;
-      auto wait = [&](uint64_t* bar, uint32_t par) -> bool {
-        if (!mbar_wait_compact(bar, par, p.status)) ok = false;
-        return ok;
-      };
-      // the next weight box landed: its shared-memory address (0 on a timeout)
-      auto next_box = [&]() -> uint32_t {
-        const int slot = ws % kRing;
-        if (!wait(w_full + slot, (ws / kRing) & 1)) return 0u;
-        tc_fence_after();
-        return smem_u32(sR + (size_t)slot * kBox);
-      };
-      // the box's slot frees once the products issued so far complete
-      auto release = [&]() {
-        umma_commit(w_empty + ws % kRing);
-        ++ws;
-      };
-      // [0, 256) = LN-free product of the A tile in sA with a 256 x 256 weight
-      // (W_O or W_Q), box by box: k block kb, output half nh
-      auto mma_256 = [&]() -> bool {
-        for (int i = 0; i < 2 * NKB; ++i) {
-          const uint32_t w = next_box();
-          if (!w) return false;
-          const int kb = i >> 1, nh = i & 1;
-          mma_box(tmem + (uint32_t)(nh * 128), smem_u32(sA) + (uint32_t)(kb * 2) * kBox, w, idesc, kb != 0);
-          release();
-        }
-        return true;
-      };
-      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++tl) {
-        // ---- A W_O into [0, 256)
-        if (!wait(a_full, tl & 1)) break;
-        tc_fence_after();
-        if (!mma_256()) break;
-        umma_commit(o_done);
-        // ---- FFN1 chunk s one chunk ahead of FFN2 chunk s - 1
-        if (!wait(ln_full, tl & 1)) break;
-        tc_fence_after();
-        const int gf0 = gf;
-        for (int s = 0; s <= nf && ok; ++s) {
-          if (s < nf) {
-            const int g = gf0 + s, b = g & 1;
-            if (g >= 2 && !wait(acc1_empty + b, ((g >> 1) - 1) & 1)) break;
-            tc_fence_after();
-            for (int kb = 0; kb < NKB; ++kb) {
-              const uint32_t w = next_box();
-              if (!w) break;
-              mma_box(tmem + (uint32_t)(b * FC), smem_u32(sA) + (uint32_t)(kb * 2) * kBox, w, idesc, kb != 0);
-              release();
-            }
-            if (!ok) break;
-            umma_commit(acc1_full + b);
+    // ---------------- MMA issuer ----------------
+    const uint32_t go = elect_one();
+    const uint32_t idesc = umma_idesc_bf16(BM, 128);
+    int slot = 0, tl = 0, gf = 0;
+    uint32_t par = 0;
+    auto wait = [&](uint64_t* bar, uint32_t parity) {
+      mbar_wait_warp(bar, parity, p.status);
+      tc_fence_after();
+    };
+    // the next weight box landed: its shared-memory address
+    auto next_box = [&]() -> uint32_t {
+      wait(w_full + slot, par);
+      return smem_u32(sR + (size_t)slot * kBox);
+    };
+    // the box's slot frees once the products issued so far complete
+    auto release = [&]() {
+      umma_commit_if(w_empty + slot, go);
+      if (++slot == kRing) {
+        slot = 0;
+        par ^= 1u;
+      }
+    };
+    // [0, 256) = LN-free product of the A tile in sA with a 256 x 256 weight
+    // (W_O or W_Q), box by box: k block kb, output half nh
+    auto mma_256 = [&]() {
+      for (int i = 0; i < 2 * NKB; ++i) {
+        const uint32_t w = next_box();
+        const int kb = i >> 1, nh = i & 1;
+        mma_box(tmem + (uint32_t)(nh * 128), smem_u32(sA) + (uint32_t)(kb * 2) * kBox, w, idesc, kb != 0);
+        release();
+      }
+    };
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++tl) {
+      // ---- A W_O into [0, 256)
+      wait(a_full, tl & 1);
+      mma_256();
+      umma_commit_if(o_done, go);
+      // ---- FFN1 chunk s one chunk ahead of FFN2 chunk s - 1
+      wait(ln_full, tl & 1);
+      const int gf0 = gf;
+      for (int s = 0; s <= nf; ++s) {
+        if (s < nf) {
+          const int g = gf0 + s, b = g & 1;
+          if (g >= 2) wait(acc1_empty + b, ((g >> 1) - 1) & 1);
+          for (int kb = 0; kb < NKB; ++kb) {
+            const uint32_t w = next_box();
+            mma_box(tmem + (uint32_t)(b * FC), smem_u32(sA) + (uint32_t)(kb * 2) * kBox, w, idesc, kb != 0);
+            release();
           }
-          if (s >= 1) {
-            const int c = s - 1, g = gf0 + c, b = g & 1;
-            if (!wait(mid_full + b, (g >> 1) & 1)) break;
-            tc_fence_after();
-            // each 32-column piece of the buffer: 32 hidden units as the hi plane
-            // (16 columns of bf16 pairs) then the lo plane
-            const uint32_t mt = tmem + (uint32_t)(b * FC);
-            for (int i = 0; i < 4; ++i) {
-              const int nh = i >> 1, sub = i & 1;
-              const uint32_t w = next_box();
-              if (!w) break;
-              const uint64_t w0 = umma_desc_sw128(w);
+          umma_commit_if(acc1_full + b, go);
+        }
+        if (s >= 1) {
+          const int c = s - 1, g = gf0 + c, b = g & 1;
+          wait(mid_full + b, (g >> 1) & 1);
+          // each 32-column piece of the buffer: 32 hidden units as the hi plane
+          // (16 columns of bf16 pairs) then the lo plane
+          const uint32_t mt = tmem + (uint32_t)(b * FC);
+          for (int i = 0; i < 4; ++i) {
+            const int nh = i >> 1, sub = i & 1;
+            const uint64_t w0 = umma_desc_sw128(next_box());
 #pragma unroll
-              for (int k4 = 0; k4 < 4; ++k4) {
-                const int kk = 4 * sub + k4;
-                const uint32_t mh = mt + (uint32_t)(32 * (kk >> 1) + 8 * (kk & 1)), ml = mh + 16;
-                const uint64_t wh = desc_adv(w0, (uint32_t)k4 * 32);
-                umma_bf16_tmem_a(acc2 + (uint32_t)(nh * 128), mh, wh, idesc, 1u);
-                umma_bf16_tmem_a(acc2 + (uint32_t)(nh * 128), ml, wh, idesc, 1u);
-              }
-              release();
+            for (int k4 = 0; k4 < 4; ++k4) {
+              const uint32_t mh = mt + (uint32_t)(64 * sub + 32 * (k4 >> 1) + 8 * (k4 & 1)), ml = mh + 16;
+              const uint64_t wh = desc_adv(w0, (uint32_t)k4 * 32);
+              umma_bf16_tmem_a_if(acc2 + (uint32_t)(nh * 128), mh, wh, idesc, 1u, go);
+              umma_bf16_tmem_a_if(acc2 + (uint32_t)(nh * 128), ml, wh, idesc, 1u, go);
             }
-            if (!ok) break;
-            umma_commit(acc1_empty + b);
-            if (c == nf - 1) umma_commit(acc2_full);
+            release();
           }
-        }
-        if (!ok) break;
-        gf = gf0 + nf;
-        // ---- the tail LN(x_out) W_Q into [0, 256)
-        if (p.tail) {
-          if (!wait(tail_a, tl & 1)) break;
-          tc_fence_after();
-          if (!mma_256()) break;
-          umma_commit(tail_full);
+          umma_commit_if(acc1_empty + b, go);
+          if (c == nf - 1) umma_commit_if(acc2_full, go);
         }
       }
+      gf = gf0 + nf;
+      // ---- the tail LN(x_out) W_Q into [0, 256)
+      if (p.tail) {
+        wait(tail_a, tl & 1);
+        mma_256();
+        umma_commit_if(tail_full, go);
+      }
     }
+    umma_drain(drain, p.status, go);
   } else {
     // ---------------- epilogue (warps 2..9) ----------------
     // two warps per TMEM lane quadrant q; warp half hf owns columns
@@ -352,11 +350,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       __syncwarp();
       if (lane == 0) arrive_one(bar);
     };
-    bool ok = true;
-    auto wait = [&](uint64_t* bar, uint32_t par) -> bool {
-      if (!mbar_wait_compact(bar, par, p.status)) ok = false;
-      return ok;
-    };
+    auto wait = [&](uint64_t* bar, uint32_t par) { mbar_wait_warp(bar, par, p.status); };
     // the row statistics over both halves: sum -> mean, then sum of squares -> rstd
     auto pair_mean = [&](float s) {
       red_sum[hf * 128 + r] = s;
@@ -369,7 +363,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       return 1.0f / sqrtf((red_var[r] + red_var[128 + r]) * (1.f / (float)D) + p.eps);
     };
     int tl = 0, gf = 0;
-    for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++tl) {
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++tl) {
       const int m0 = t * BM;
       const bool valid = m0 + r < rows_valid;
       float* xrow = p.x + (size_t)(m0 + r) * p.ldx;
@@ -394,7 +388,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       // ---- x = x0 + A W_O back into the accumulator, LN(x) over the A tile
       // (the projection, the tile's only reader, is complete)
-      if (!wait(o_done, tl & 1)) break;
+      wait(o_done, tl & 1);
       tc_fence_after();
       float s4[4] = {0.f, 0.f, 0.f, 0.f};
       for (int i = 0; i < 4; ++i) {
@@ -437,7 +431,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // the chunk's TMEM buffer, FFN2's A operand
       for (int f = 0; f < nf; ++f, ++gf) {
         const int ba = gf & 1;
-        if (!wait(acc1_full + ba, (gf >> 1) & 1)) break;
+        wait(acc1_full + ba, (gf >> 1) & 1);
         tc_fence_after();
         for (int jp = 0; jp < 2; ++jp) {
           const uint32_t col = tmem + lane_off + (uint32_t)(ba * FC + 64 * hf + 32 * jp);
@@ -457,11 +451,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         tc_fence_before();
         warp_arrive(mid_full + ba);
       }
-      if (!ok) break;
       // ---- x_out = acc2 + b2 to memory, staged in this warp's 16 KB of sA (every
       // FFN1 has read LN(x) there) as four 32 x 32 blocks (128-byte swizzle)
       // and stored by TMA; then LN(x_out) over the A tile
-      if (!wait(acc2_full, tl & 1)) break;
+      wait(acc2_full, tl & 1);
       tc_fence_after();
       uint8_t* xst = sA + (size_t)ew * 16384u;
 #pragma unroll
@@ -533,7 +526,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // LN(x_out)): this thread's 128 columns of row r as 128-byte-swizzled
       // [kb][128 rows x 64] tiles, stored by TMA
       if (p.tail) {
-        if (!wait(tail_full, tl & 1)) break;
+        wait(tail_full, tl & 1);
         tc_fence_after();
         for (int i = 0; i < 4; ++i) {
           const int c = c0 + 32 * i;
@@ -564,7 +557,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (et == 0) bulk_wait0();  // output tensor stores complete before the CTA retires
   }
 
-  __syncwarp();  // each warp arrives whole: lane 0 of warps 0 and 1 ran the producer and MMA loops
+  __syncwarp();
   tc_fence_before();
   __syncthreads();
   if (warp == 0) tmem_dealloc(tmem, 512);
