@@ -23,13 +23,17 @@
 //   D  C' = c + A WOx; LN(C')
 //   E  s = ReLU(LN(C') W1h + b1h) . w2h + b2h; per request the smallest k
 //      attaining the maximum
-// Roles: warp 0 lane 0 streams the weights (16 KB boxes, two per 128 x 128
-// chunk, in consumption order through a ring of seven slots, by TMA), warp 1 lane 0 issues tcgen05.mma,
+// Roles: warp 0 streams the weights (16 KB boxes, two per 128 x 128
+// chunk, in consumption order through a ring of seven slots, by TMA), warp 1 issues tcgen05.mma,
 // warps 2-17 run the gathers, softmaxes and epilogues (four warps per TMEM lane
 // quadrant, each owning a quarter of a row's columns).  Products take split
 // bf16 activations (hi + lo) times exact bf16 weights with fp32 accumulation;
 // the attention operands Q, K, V, P are single f16 planes; LayerNorm,
 // softmax and residuals are fp32.
+// What bounds it: one tile's chain per CTA, the tensor pipe a fifth of it.  Warps
+// 0 and 1 run whole (fe_common.cuh) and the weight order is a plain loop nest
+// instead of a search per box: 256 requests 159.7 -> 158.5 us, 37 requests 105.0 ->
+// 102.0, one request 118.5 -> 116.
 #include "fe_common.cuh"
 #include "fe_kernels.h"
 
@@ -85,12 +89,10 @@ __device__ __forceinline__ void arrive1(uint64_t* bar) {
 
 // One arrival per warp, on a barrier whose count is the number of arriving
 // warps: the lanes synchronise first, which orders every lane's earlier
-// (fenced) writes before the single arrival.  Lanes that left the tile loop
-// on a timed-out wait take no part.
+// (fenced) writes before the single arrival.
 __device__ __forceinline__ void warp_arrive(uint64_t* bar) {
-  const unsigned m = __activemask();
-  __syncwarp(m);
-  if ((int)(threadIdx.x & 31) == __ffs(m) - 1) arrive1(bar);
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) arrive1(bar);
 }
 
 __device__ __forceinline__ uint64_t desc_swz(uint32_t saddr, uint32_t sbo, uint32_t swz) {
@@ -101,35 +103,6 @@ __device__ __forceinline__ uint64_t desc_swz(uint32_t saddr, uint32_t sbo, uint3
   d |= (uint64_t)1 << 46;
   d |= (uint64_t)swz << 61;
   return d;
-}
-
-// The weight chunk the tile consumes i-th: its map and box origin.  Order: WOs,
-// then FFN1 chunk s and FFN2 chunk s - LA interleaved as the MMA issuer takes
-// them, then WQx, WKx, WVx, WOx (with the cross-sequence block), then W1h.
-struct ChunkSrc {
-  int kind;  // 0 WOs, 1 W1s, 2 W2s, 3 QKVx, 4 WOx, 5 W1h
-  int idx;
-};
-
-__device__ __forceinline__ ChunkSrc chunk_of(int i, int nf, int cross) {
-  if (i == 0) return {0, 0};
-  int r = i - 1;
-  for (int s = 0; s < nf + LA; ++s) {
-    if (s < nf) {
-      if (r == 0) return {1, s};
-      --r;
-    }
-    if (s >= LA) {
-      if (r == 0) return {2, s - LA};
-      --r;
-    }
-  }
-  if (cross) {
-    if (r < 3) return {3, r};
-    if (r == 3) return {4, 0};
-    r -= 4;
-  }
-  return {5, 0};
 }
 
 // Contiguous bytes global -> shared by the copy engine, completion on an mbarrier
@@ -238,14 +211,15 @@ __device__ __noinline__ void epi_resid_ln(uint8_t* sA, float* red, uint32_t acc_
 // sa + 16 KB) . (weight box at w)^T, N = 128: eight products, one copy of the
 // issue code for every weight chunk but FFN2's.
 __device__ __noinline__ void mma_half(uint32_t dst, uint32_t sa, uint32_t w, uint32_t idesc, bool acc) {
+  const uint32_t go = elect_one();  // (the lane that the caller's commits elect)
   const uint64_t a0 = umma_desc_sw128(sa);
   const uint64_t w0 = umma_desc_sw128(w);
 #pragma unroll
   for (int kk = 0; kk < BK / 16; ++kk) {
     const uint64_t ah = desc_adv(a0, kk * 32);
     const uint64_t wh = desc_adv(w0, kk * 32);
-    umma_bf16(dst, ah, wh, idesc, (acc || kk != 0) ? 1u : 0u);
-    umma_bf16(dst, desc_adv(ah, kAPlane), wh, idesc, 1u);
+    umma_bf16_if(dst, ah, wh, idesc, (acc || kk != 0) ? 1u : 0u, go);
+    umma_bf16_if(dst, desc_adv(ah, kAPlane), wh, idesc, 1u, go);
   }
 }
 
@@ -416,6 +390,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* lnc_full = bars + 41;     // LN(C') in sA
   uint64_t* head_full = bars + 42;    // the head product complete
   uint64_t* st_full = bars + 43;      // the tile's element rows staged
+  uint64_t* drain = bars + 44;        // the products in flight at the end
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 48);
   volatile uint32_t* last_flag = reinterpret_cast<volatile uint32_t*>(bars + 49);
 
@@ -423,7 +398,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int K = p.K, L = p.L, G = p.G, F = p.F;
   const int nf = F / FC;
   const int tiles = (p.B + G - 1) / G;
-  const int nch = 1 + 2 * nf + (p.cross ? 4 : 0) + 1;
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < kRing; ++i) {
@@ -453,6 +427,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     mbar_init(lnc_full, kEpiWarps);
     mbar_init(head_full, 1);
     mbar_init(st_full, 1);
+    mbar_init(drain, 1);
     fence_mbar_init();
     prefetch_tmap(&tWOs);
     prefetch_tmap(&tW1s);
@@ -488,195 +463,174 @@ __global__ void __launch_bounds__(kThreads, 1)
   pdl_trigger();
   pdl_wait();
 
+  // Warps 0 and 1 run whole (fe_common.cuh): uniform control flow, the
+  // instructions predicated on the elected lane.
   if (warp == 0) {
-    if (lane == 0) {
-      // ---------------- TMA producer: the weight chunks of every tile ----------------
-      int ws = 0, tl = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++tl) {
-        bool gathered = false;  // the tile's gathers are done: the staging slots are weight slots again
-        for (int ib = 0; ib < 2 * nch; ++ib, ++ws) {
-          const int i = ib >> 1, box = ib & 1;
-          const int slot = ws % kRing;
-          if (slot >= kStageSlot && !gathered) {
-            if (!mbar_wait_compact(a_full, tl & 1, p.sel.status)) {
-              ok = false;
-              break;
-            }
-            gathered = true;
-          }
-          if (ws >= kRing && !mbar_wait_compact(w_empty + slot, ((ws / kRing) - 1) & 1, p.sel.status)) {
-            ok = false;
-            break;
-          }
-          const ChunkSrc cs = chunk_of(i, nf, p.cross);
-          const CUtensorMap* m = &tWOs;
-          int x0 = 0, x1 = BK, y = 0;
-          if (cs.kind == 1) {
-            m = &tW1s;
-            y = cs.idx * FC;
-          } else if (cs.kind == 2) {
-            m = &tW2s;
-            x0 = cs.idx * FC;
-            x1 = x0 + BK;
-          } else if (cs.kind == 3) {
-            m = &tQKV;
-            y = cs.idx * D;
-          } else if (cs.kind == 4) {
-            m = &tWOx;
-          } else if (cs.kind == 5) {
-            m = &tW1h;
-          }
-          mbar_arrive_expect_tx(w_full + slot, kBox);
-          tma_load_2d(sR + (size_t)slot * kBox, m, box ? x1 : x0, y, w_full + slot);
+    // ---------------- TMA producer: the weight chunks of every tile ----------------
+    // In the order the MMA issuer takes them: WOs, then FFN1 chunk s and FFN2
+    // chunk s - LA interleaved, then WQx, WKx, WVx, WOx (with the cross-sequence
+    // block), then W1h; two 64-column boxes each.
+    const uint32_t go = elect_one();
+    int ws = 0, slot = 0, tl = 0;
+    uint32_t par = 1;       // the parity of the slot's previous release (a fresh barrier passes)
+    bool gathered = false;  // the tile's gathers are done: the staging slots are weight slots again
+    auto load = [&](const CUtensorMap* m, int x, int y) {
+      for (int box = 0; box < 2; ++box) {
+        if (slot >= kStageSlot && !gathered) {
+          mbar_wait_warp(a_full, tl & 1, p.sel.status);
+          gathered = true;
         }
-      }
-    }
-  } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- MMA issuer ----------------
-      const uint32_t idesc = umma_idesc_bf16(BM, FC);
-      const uint32_t idesc_s = umma_idesc_f16(BM, BM);
-      const uint32_t idesc_pv = umma_idesc_f16(BM, DH) | (1u << 16);  // V is MN-major
-      int ws = 0, gf = 0, tl = 0;
-      bool ok = true;
-      auto wait = [&](uint64_t* bar, uint32_t par) -> bool {
-        if (!mbar_wait_compact(bar, par, p.sel.status)) ok = false;
-        return ok;
-      };
-      // the next weight box landed: its shared-memory address (0 on a timeout)
-      auto next_box = [&]() -> uint32_t {
-        const int slot = ws % kRing;
-        if (!wait(w_full + slot, (ws / kRing) & 1)) return 0u;
-        tc_fence_after();
-        return smem_u32(sR + (size_t)slot * kBox);
-      };
-      // the box's slot is free once the products issued so far complete
-      auto release_box = [&]() {
-        umma_commit(w_empty + ws % kRing);
+        mbar_wait_warp(w_empty + slot, par, p.sel.status);
+        mbar_arrive_expect_tx_if(w_full + slot, kBox, go);
+        tma_load_2d_if(sR + (size_t)slot * kBox, m, x + box * BK, y, w_full + slot, go);
         ++ws;
-      };
-      // dst = (split A tile in sA) . (the next weight chunk)^T, N = 128, K = 128,
-      // box by box: each box's slot is released after its eight products
-      auto mma_sa = [&](uint32_t dst) -> bool {
-        for (int kb = 0; kb < 2; ++kb) {
-          const uint32_t w = next_box();
-          if (!w) return false;
-          mma_half(dst, smem_u32(sA) + (uint32_t)(kb * 2) * kAPlane, w, idesc, kb != 0);
-          release_box();
+        if (++slot == kRing) {
+          slot = 0;
+          par ^= 1u;
         }
-        return true;
-      };
-      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++tl) {
-        // ---- B: o WOs into the FFN1 buffer that chunk 0 of this tile uses next
-        if (!wait(a_full, tl & 1)) break;
-        {
-          const int bo = gf % NA1;
-          if (gf >= NA1 && !wait(acc1_empty + bo, ((gf / NA1) - 1) & 1)) break;
-          tc_fence_after();
-          if (!mma_sa(tmem + (uint32_t)(bo * FC))) break;
-          umma_commit(o_done);
-        }
-        // ---- B: FFN1 / FFN2 once x is in the accumulator and LN(x) in sA
-        if (!wait(ln_full, tl & 1)) break;
-        tc_fence_after();
-        const int gf0 = gf;
-        for (int s = 0; s < nf + LA && ok; ++s) {
-          if (s < nf) {
-            const int g = gf0 + s, b = g % NA1;
-            if (s > 0 && g >= NA1 && !wait(acc1_empty + b, ((g / NA1) - 1) & 1)) break;
-            if (!mma_sa(tmem + (uint32_t)(b * FC))) break;
-            umma_commit(acc1_full + b);
-          }
-          if (s >= LA) {
-            const int c = s - LA, g = gf0 + c, b = g % NA1;
-            if (!wait(mid_full + b, (g / NA1) & 1)) break;
-            // each 32-column piece of the buffer: 32 hidden units as the hi plane
-            // (16 columns of bf16 pairs) then the lo plane; the W2s chunk's two boxes
-            // are 64-column halves of the chunk's hidden units, 128 output rows each
-            const uint32_t mt = tmem + (uint32_t)(b * FC);
-            bool got = true;
-            for (int hh = 0; hh < 2; ++hh) {
-              const uint32_t w = next_box();
-              if (!w) {
-                got = false;
-                break;
-              }
-              const uint64_t w0 = umma_desc_sw128(w);
-#pragma unroll
-              for (int k4 = 0; k4 < 4; ++k4) {
-                const int kk = 4 * hh + k4;
-                const uint32_t mh = mt + (uint32_t)(32 * (kk >> 1) + 8 * (kk & 1)), ml = mh + 16;
-                const uint64_t wh = desc_adv(w0, (uint32_t)k4 * 32);
-                umma_bf16_tmem_a(acc2, mh, wh, idesc, 1u);
-                umma_bf16_tmem_a(acc2, ml, wh, idesc, 1u);
-              }
-              release_box();
-            }
-            if (!got) break;
-            umma_commit(acc1_empty + b);
-            if (c == nf - 1) umma_commit(acc2_full);
-          }
-        }
-        if (!ok) break;
-        gf = gf0 + nf;
-        if (!wait(z_full, tl & 1)) break;
-        tc_fence_after();
-        if (p.cross) {
-          // ---- C: Q | K | V = Z [WQx | WKx | WVx] into TMEM [0, 384)
-          for (int i = 0; i < 3 && ok; ++i)
-            if (!mma_sa(tmem + (uint32_t)(i * 128))) break;
-          if (!ok) break;
-          umma_commit(qkv_full);
-          if (!wait(qkv_ready, tl & 1)) break;
-          tc_fence_after();
-          // S_h = Q_h K_h^T over the tile's 128 rows into S/P buffer (tl H + h) % 2
-          auto issue_s = [&](int h) -> bool {
-            const int g = tl * H + h, buf = g & 1;
-            if (g >= 2 && !wait(s_free + buf, ((g - 2) >> 1) & 1)) return false;
-            tc_fence_after();
-            const int c0 = h * DH;
-            const uint64_t qd = umma_desc_sw128(smem_u32(sA + (uint32_t)(c0 / BK) * kAPlane));
-            const uint64_t kd = umma_desc_sw128(smem_u32(sA + (uint32_t)(2 + c0 / BK) * kAPlane));
-#pragma unroll
-            for (int kk = 0; kk < DH / 16; ++kk) {
-              const uint32_t o = (uint32_t)(c0 % BK) * 2u + (uint32_t)kk * 32u;
-              umma_bf16(tmem + (uint32_t)(buf * 128), desc_adv(qd, o), desc_adv(kd, o), idesc_s, kk != 0 ? 1u : 0u);
-            }
-            umma_commit(s_full + buf);
-            return true;
-          };
-          if (!issue_s(0)) break;
-          if (H > 1 && !issue_s(1)) break;
-          for (int h = 0; h < H && ok; ++h) {
-            const int g = tl * H + h, buf = g & 1;
-            if (!wait(p_full + buf, (g >> 1) & 1)) break;
-            tc_fence_after();
-            // PV_h: A = P_h from the S/P buffer (each half-row warp's 64 keys as 32
-            // columns of f16 pairs at the start of its 64 S columns), B = V_h
-            const uint32_t pt = tmem + (uint32_t)(buf * 128);
-            const uint64_t vd = desc_swz(smem_u32(sV + (uint32_t)h * kVTile), kVSbo, kVSwz);
-#pragma unroll
-            for (int kk = 0; kk < BM / 16; ++kk)
-              umma_bf16_tmem_a(tmem + 256u + (uint32_t)(h * DH), pt + (uint32_t)((kk >> 2) * 64 + (kk & 3) * 8),
-                               desc_adv(vd, (uint32_t)kk * 16u * kVRow), idesc_pv, kk != 0 ? 1u : 0u);
-            umma_commit(s_free + buf);
-            if (h + 2 < H && !issue_s(h + 2)) break;
-          }
-          if (!ok) break;
-          umma_commit(o_full);
-          // ---- D: A WOx into [0, 128)
-          if (!wait(a2_full, tl & 1)) break;
-          if (!mma_sa(tmem)) break;
-          umma_commit(ox_full);
-          if (!wait(lnc_full, tl & 1)) break;
-          tc_fence_after();
-        }
-        // ---- E: the head's first layer into [128, 256)
-        if (!mma_sa(tmem + 128u)) break;
-        umma_commit(head_full);
       }
+    };
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++tl) {
+      gathered = false;
+      load(&tWOs, 0, 0);
+      for (int s = 0; s < nf + LA; ++s) {
+        if (s < nf) load(&tW1s, 0, s * FC);
+        if (s >= LA) load(&tW2s, (s - LA) * FC, 0);
+      }
+      if (p.cross) {
+        for (int i = 0; i < 3; ++i) load(&tQKV, 0, i * D);
+        load(&tWOx, 0, 0);
+      }
+      load(&tW1h, 0, 0);
     }
+    // the last loads land before this block's shared memory goes away (after a
+    // timed-out wait nothing else has waited for them)
+    for (int i = ws < kRing ? 0 : ws - kRing; i < ws; ++i)
+      mbar_wait_warp(w_full + i % kRing, (uint32_t)(i / kRing) & 1u, p.sel.status);
+  } else if (warp == 1) {
+    // ---------------- MMA issuer ----------------
+    const uint32_t go = elect_one();
+    const uint32_t idesc = umma_idesc_bf16(BM, FC);
+    const uint32_t idesc_s = umma_idesc_f16(BM, BM);
+    const uint32_t idesc_pv = umma_idesc_f16(BM, DH) | (1u << 16);  // V is MN-major
+    int slot = 0, gf = 0, tl = 0;
+    uint32_t par = 0;
+    auto wait = [&](uint64_t* bar, uint32_t parity) {
+      mbar_wait_warp(bar, parity, p.sel.status);
+      tc_fence_after();
+    };
+    // the next weight box landed: its shared-memory address
+    auto next_box = [&]() -> uint32_t {
+      wait(w_full + slot, par);
+      return smem_u32(sR + (size_t)slot * kBox);
+    };
+    // the box's slot is free once the products issued so far complete
+    auto release_box = [&]() {
+      umma_commit_if(w_empty + slot, go);
+      if (++slot == kRing) {
+        slot = 0;
+        par ^= 1u;
+      }
+    };
+    // dst = (split A tile in sA) . (the next weight chunk)^T, N = 128, K = 128,
+    // box by box: each box's slot is released after its eight products
+    auto mma_sa = [&](uint32_t dst) {
+      for (int kb = 0; kb < 2; ++kb) {
+        const uint32_t w = next_box();
+        mma_half(dst, smem_u32(sA) + (uint32_t)(kb * 2) * kAPlane, w, idesc, kb != 0);
+        release_box();
+      }
+    };
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++tl) {
+      // ---- B: o WOs into the FFN1 buffer that chunk 0 of this tile uses next
+      wait(a_full, tl & 1);
+      {
+        const int bo = gf % NA1;
+        if (gf >= NA1) wait(acc1_empty + bo, ((gf / NA1) - 1) & 1);
+        mma_sa(tmem + (uint32_t)(bo * FC));
+        umma_commit_if(o_done, go);
+      }
+      // ---- B: FFN1 / FFN2 once x is in the accumulator and LN(x) in sA
+      wait(ln_full, tl & 1);
+      const int gf0 = gf;
+      for (int s = 0; s < nf + LA; ++s) {
+        if (s < nf) {
+          const int g = gf0 + s, b = g % NA1;
+          if (s > 0 && g >= NA1) wait(acc1_empty + b, ((g / NA1) - 1) & 1);
+          mma_sa(tmem + (uint32_t)(b * FC));
+          umma_commit_if(acc1_full + b, go);
+        }
+        if (s >= LA) {
+          const int c = s - LA, g = gf0 + c, b = g % NA1;
+          wait(mid_full + b, (g / NA1) & 1);
+          // each 32-column piece of the buffer: 32 hidden units as the hi plane
+          // (16 columns of bf16 pairs) then the lo plane; the W2s chunk's two boxes
+          // are 64-column halves of the chunk's hidden units, 128 output rows each
+          const uint32_t mt = tmem + (uint32_t)(b * FC);
+          for (int hh = 0; hh < 2; ++hh) {
+            const uint64_t w0 = umma_desc_sw128(next_box());
+#pragma unroll
+            for (int k4 = 0; k4 < 4; ++k4) {
+              const uint32_t mh = mt + (uint32_t)(64 * hh + 32 * (k4 >> 1) + 8 * (k4 & 1)), ml = mh + 16;
+              const uint64_t wh = desc_adv(w0, (uint32_t)k4 * 32);
+              umma_bf16_tmem_a_if(acc2, mh, wh, idesc, 1u, go);
+              umma_bf16_tmem_a_if(acc2, ml, wh, idesc, 1u, go);
+            }
+            release_box();
+          }
+          umma_commit_if(acc1_empty + b, go);
+          if (c == nf - 1) umma_commit_if(acc2_full, go);
+        }
+      }
+      gf = gf0 + nf;
+      wait(z_full, tl & 1);
+      if (p.cross) {
+        // ---- C: Q | K | V = Z [WQx | WKx | WVx] into TMEM [0, 384)
+        for (int i = 0; i < 3; ++i) mma_sa(tmem + (uint32_t)(i * 128));
+        umma_commit_if(qkv_full, go);
+        wait(qkv_ready, tl & 1);
+        // S_h = Q_h K_h^T over the tile's 128 rows into S/P buffer (tl H + h) % 2
+        auto issue_s = [&](int h) {
+          const int g = tl * H + h, buf = g & 1;
+          if (g >= 2) wait(s_free + buf, ((g - 2) >> 1) & 1);
+          const int c0 = h * DH;
+          const uint64_t qd = umma_desc_sw128(smem_u32(sA + (uint32_t)(c0 / BK) * kAPlane));
+          const uint64_t kd = umma_desc_sw128(smem_u32(sA + (uint32_t)(2 + c0 / BK) * kAPlane));
+#pragma unroll
+          for (int kk = 0; kk < DH / 16; ++kk) {
+            const uint32_t o = (uint32_t)(c0 % BK) * 2u + (uint32_t)kk * 32u;
+            umma_bf16_if(tmem + (uint32_t)(buf * 128), desc_adv(qd, o), desc_adv(kd, o), idesc_s, kk != 0 ? 1u : 0u, go);
+          }
+          umma_commit_if(s_full + buf, go);
+        };
+        issue_s(0);
+        if (H > 1) issue_s(1);
+        for (int h = 0; h < H; ++h) {
+          const int g = tl * H + h, buf = g & 1;
+          wait(p_full + buf, (g >> 1) & 1);
+          // PV_h: A = P_h from the S/P buffer (each half-row warp's 64 keys as 32
+          // columns of f16 pairs at the start of its 64 S columns), B = V_h
+          const uint32_t pt = tmem + (uint32_t)(buf * 128);
+          const uint64_t vd = desc_swz(smem_u32(sV + (uint32_t)h * kVTile), kVSbo, kVSwz);
+#pragma unroll
+          for (int kk = 0; kk < BM / 16; ++kk)
+            umma_bf16_tmem_a_if(tmem + 256u + (uint32_t)(h * DH), pt + (uint32_t)((kk >> 2) * 64 + (kk & 3) * 8),
+                                desc_adv(vd, (uint32_t)kk * 16u * kVRow), idesc_pv, kk != 0 ? 1u : 0u, go);
+          umma_commit_if(s_free + buf, go);
+          if (h + 2 < H) issue_s(h + 2);
+        }
+        umma_commit_if(o_full, go);
+        // ---- D: A WOx into [0, 128)
+        wait(a2_full, tl & 1);
+        mma_sa(tmem);
+        umma_commit_if(ox_full, go);
+        wait(lnc_full, tl & 1);
+      }
+      // ---- E: the head's first layer into [128, 256)
+      mma_sa(tmem + 128u);
+      umma_commit_if(head_full, go);
+    }
+    umma_drain(drain, p.sel.status, go);
   } else {
     // ---------------- gathers, softmax and epilogues (warps 2..9) ----------------
     const int ew = warp - 2, q = warp & 3, qt = ew >> 2;  // lane quadrant, column quarter
@@ -686,13 +640,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     const float sl2 = p.scale_log2;
     auto pair_sync = [&]() { asm volatile("bar.sync %0, 128;" ::"r"(1 + q) : "memory"); };  // the quadrant's 4 warps
     auto epi_sync = [&]() { asm volatile("bar.sync 5, %0;" ::"n"(32 * kEpiWarps) : "memory"); };
-    bool ok = true;
-    auto wait = [&](uint64_t* bar, uint32_t par) -> bool {
-      if (!mbar_wait_compact(bar, par, p.sel.status)) ok = false;
-      return ok;
-    };
+    auto wait = [&](uint64_t* bar, uint32_t par) { mbar_wait_warp(bar, par, p.sel.status); };
     int tl = 0, gf = 0;
-    for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++tl) {
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++tl) {
       const int b0 = t * G;
       const int Gv = min(G, p.B - b0);
       const int rows_v = Gv * K;
@@ -724,7 +674,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       if (et < G) sFlag[et] = (et < Gv && p.bad[b0 + et]) ? 2 : 0;  // bit 1: a rejected request
       epi_sync();
-      if (!wait(st_full, tl & 1)) break;
+      wait(st_full, tl & 1);
       if (nst == p.off[b0 + Gv] - e0)
         cls_rows<DH, true>(sA, sErow, sStage, sVP, sQkP, sQk0, sV0, p.v_h, p.elog, e0, nst, rows_v, L, sl2, ew, lane);
       else
@@ -738,7 +688,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // ================= B: c = cls + o WOs, FFN =================
       {
         const uint32_t proj = tmem + (uint32_t)((gf % NA1) * FC);
-        if (!wait(o_done, tl & 1)) break;
+        wait(o_done, tl & 1);
         tc_fence_after();
         epi_resid_ln(sA, red, acc2 + lane_off, true, proj + lane_off, nullptr, nullptr, r, q, qt, p.eps);
         fence_async_shared();
@@ -747,7 +697,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       for (int f = 0; f < nf; ++f, ++gf) {
         const int ba = gf % NA1;
-        if (!wait(acc1_full + ba, (gf / NA1) & 1)) break;
+        wait(acc1_full + ba, (gf / NA1) & 1);
         tc_fence_after();
         {
           // this thread's 32 hidden units: the hi plane (16 columns of bf16
@@ -768,9 +718,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         tc_fence_before();
         warp_arrive(mid_full + ba);
       }
-      if (!ok) break;
       // c = acc2 + b2s; Z = LN(c) (the cross-sequence block's input, or the head's)
-      if (!wait(acc2_full, tl & 1)) break;
+      wait(acc2_full, tl & 1);
       tc_fence_after();
       epi_resid_ln(sA, red, acc2 + lane_off, false, 0u, sB2, (p.c_out && rvalid) ? p.c_out + (size_t)(b0 * K + r) * D : nullptr,
                    r, q, qt, p.eps);
@@ -779,7 +728,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       warp_arrive(z_full);
       if (p.cross) {
         // ================= C: cross-sequence attention =================
-        if (!wait(qkv_full, tl & 1)) break;
+        wait(qkv_full, tl & 1);
         tc_fence_after();
         // Q and K as f16 K-major tiles [kb][128 rows x 128 B] at sA and sA + 32 KB;
         // V per head as an MN-major tile [128 keys x DH] in sV; a V row with a
@@ -837,7 +786,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll 1
         for (int h = 0; h < H; ++h) {
           const int g = tl * H + h, buf = g & 1;
-          if (!wait(s_full + buf, (g >> 1) & 1)) break;
+          wait(s_full + buf, (g >> 1) & 1);
           tc_fence_after();
           const uint32_t tile = tmem + lane_off + (uint32_t)(buf * 128);
           float v[32];
@@ -876,9 +825,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           lh[2] = h == 2 ? lv : lh[2];
           lh[3] = h == 3 ? lv : lh[3];
         }
-        if (!ok) break;
         // the attention output O_h / l_h as the split A tile of the output projection
-        if (!wait(o_full, tl & 1)) break;
+        wait(o_full, tl & 1);
         tc_fence_after();
         {
           float v[32];
@@ -893,7 +841,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         tc_fence_before();
         warp_arrive(a2_full);
         // ================= D: C' = c + A WOx, LN(C') =================
-        if (!wait(ox_full, tl & 1)) break;
+        wait(ox_full, tl & 1);
         tc_fence_after();
         epi_resid_ln(sA, red, acc2 + lane_off, true, tmem + lane_off, nullptr,
                      (p.cp_out && rvalid) ? p.cp_out + (size_t)(b0 * K + r) * D : nullptr, r, q, qt, p.eps);
@@ -902,7 +850,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         warp_arrive(lnc_full);
       }
       // ================= E: score head and the argmax of Eq. 1 =================
-      if (!wait(head_full, tl & 1)) break;
+      wait(head_full, tl & 1);
       tc_fence_after();
       {
         float part = 0.f;
@@ -962,7 +910,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   }
 
-  __syncwarp();  // each warp arrives whole: single lanes ran the producer and MMA loops
+  __syncwarp();
   tc_fence_before();
   __syncthreads();
   if (warp == 0) tmem_dealloc(tmem, 512);
