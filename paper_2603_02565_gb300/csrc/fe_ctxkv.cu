@@ -140,6 +140,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* acc_empty = bars + 9;  // [2] accumulator drained
   uint64_t* st_full = bars + 11;   // state mode: the state product of the tile complete
   uint64_t* stats_full = bars + 12;  // [2] row statistics of the tile written
+  uint64_t* drain = bars + 14;     // the products in flight at the end
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 16);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -153,6 +154,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(acc_empty + i, kEpiWarps);
     }
     mbar_init(st_full, 1);
+    mbar_init(drain, 1);
     fence_mbar_init();
     prefetch_tmap(&tX);
     prefetch_tmap(&tW);
@@ -192,49 +194,52 @@ __global__ void __launch_bounds__(kThreads, 1)
     return;
   }
 
+  // Warps 0 and 1 run whole (fe_common.cuh): uniform control flow, the
+  // instructions predicated on the elected lane.
   if (warp == 0) {
-    if (lane == 0) {
-      // ---------------- TMA: raw context blocks ----------------
-      int it = 0;
-      for (int t = tile_at(it); t >= 0; t = tile_at(++it)) {
-        const int rb = it % NRAW;
-        if (it >= NRAW && !mbar_wait_bounded(raw_empty + rb, ((it / NRAW) - 1) & 1, p.status)) break;
-        mbar_arrive_expect_tx(raw_full + rb, LY.raw_bytes);
-        // context row of this block (one K/V per candidate sequence: rep > 1)
-        const int r0 = t * BM;
-        const int in_row = p.rep > 1 ? ((r0 / p.C) / p.rep) * p.C + r0 % p.C : r0;
-        for (int kb = 0; kb < NKB; ++kb)
-          tma_load_2d(sRaw + (size_t)rb * LY.raw_bytes + (size_t)kb * kPlane, &tX, kb * BK, in_row, raw_full + rb);
-      }
+    // ---------------- TMA: raw context blocks ----------------
+    const uint32_t go = elect_one();
+    int it = 0;
+    for (int t = tile_at(it); t >= 0; t = tile_at(++it)) {
+      const int rb = it % NRAW;
+      mbar_wait_warp(raw_empty + rb, ((it / NRAW) & 1) ^ 1, p.status);  // (a fresh barrier passes)
+      mbar_arrive_expect_tx_if(raw_full + rb, LY.raw_bytes, go);
+      // context row of this block (one K/V per candidate sequence: rep > 1)
+      const int r0 = t * BM;
+      const int in_row = p.rep > 1 ? ((r0 / p.C) / p.rep) * p.C + r0 % p.C : r0;
+      for (int kb = 0; kb < NKB; ++kb)
+        tma_load_2d_if(sRaw + (size_t)rb * LY.raw_bytes + (size_t)kb * kPlane, &tX, kb * BK, in_row, raw_full + rb, go);
     }
+    // the last loads land before this block's shared memory goes away (after a
+    // timed-out wait nothing else has waited for them)
+    for (int i = it < NRAW ? 0 : it - NRAW; i < it; ++i) mbar_wait_warp(raw_full + i % NRAW, (i / NRAW) & 1, p.status);
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- MMA issuer ----------------
-      const uint32_t idesc = umma_idesc_bf16(BM, Nh);
-      bool ok = mbar_wait_bounded(w_full, 0, p.status);
-      int it = 0;
-      for (int t = tile_at(it); t >= 0 && ok; t = tile_at(++it)) {
-        const int ab = it % NACC;
-        if (it >= NACC && !mbar_wait_bounded(acc_empty + ab, ((it / NACC) - 1) & 1, p.status)) break;
-        const int rb = it % NRAW;
-        if (!mbar_wait_bounded(raw_full + rb, (it / NRAW) & 1, p.status)) break;
-        tc_fence_after();
-        const uint32_t dst = tmem + (uint32_t)(256 * ab);
-        const uint64_t a0 = umma_desc_sw128(smem_u32(sRaw + (size_t)rb * LY.raw_bytes));
-        const uint64_t w0 = umma_desc_sw128(smem_u32(sW));
+    // ---------------- MMA issuer ----------------
+    const uint32_t go = elect_one();
+    const uint32_t idesc = umma_idesc_bf16(BM, Nh);
+    const uint64_t w0 = umma_desc_sw128(smem_u32(sW)), r0 = umma_desc_sw128(smem_u32(sRaw));
+    mbar_wait_warp(w_full, 0, p.status);
+    int it = 0;
+    for (int t = tile_at(it); t >= 0; t = tile_at(++it)) {
+      const int ab = it % NACC, rb = it % NRAW;
+      mbar_wait_warp(acc_empty + ab, ((it / NACC) & 1) ^ 1, p.status);  // (a fresh barrier passes)
+      mbar_wait_warp(raw_full + rb, (it / NRAW) & 1, p.status);
+      tc_fence_after();
+      const uint32_t dst = tmem + (uint32_t)(256 * ab);
+      const uint64_t a0 = desc_adv(r0, (uint32_t)rb * LY.raw_bytes);
 #pragma unroll
-        for (int kb = 0; kb < NKB; ++kb) {
+      for (int kb = 0; kb < NKB; ++kb) {
 #pragma unroll
-          for (int kk = 0; kk < BK / 16; ++kk) {
-            const uint64_t ah = desc_adv(a0, (uint32_t)kb * kPlane + kk * 32);
-            const uint64_t wh = desc_adv(w0, (uint32_t)kb * (uint32_t)Nh * (BK * 2) + kk * 32);
-            umma_bf16(dst, ah, wh, idesc, (kb | kk) != 0 ? 1u : 0u);
-          }
+        for (int kk = 0; kk < BK / 16; ++kk) {
+          const uint64_t ah = desc_adv(a0, (uint32_t)kb * kPlane + kk * 32);
+          const uint64_t wh = desc_adv(w0, (uint32_t)kb * (uint32_t)Nh * (BK * 2) + kk * 32);
+          umma_bf16_if(dst, ah, wh, idesc, (kb | kk) != 0 ? 1u : 0u, go);
         }
-        umma_commit(raw_empty + rb);  // the raw block frees once these MMAs (and the statistics) are done
-        umma_commit(acc_full + ab);
       }
+      umma_commit_if(raw_empty + rb, go);  // the raw block frees once these MMAs (and the statistics) are done
+      umma_commit_if(acc_full + ab, go);
     }
+    umma_drain(drain, p.status, go);
   } else if (warp < 2 + kLnWarps) {
     // ---------------- LayerNorm statistics: two threads per row ----------------
     // lanes l and l ^ 16 share row r; of each 64-column k block part 0 takes
@@ -244,7 +249,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     int it = 0;
     for (int t = tile_at(it); t >= 0; t = tile_at(++it)) {
       const int rb = it % NRAW;
-      if (!mbar_wait_bounded(raw_full + rb, (it / NRAW) & 1, p.status)) break;
+      mbar_wait_warp(raw_full + rb, (it / NRAW) & 1, p.status);
       const uint8_t* raw = sRaw + (size_t)rb * LY.raw_bytes;
       // piece j of this thread: global piece g, column 8 g, 128-byte-swizzled
       // within its 64-column block
@@ -280,7 +285,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const float rstd = 1.0f / sqrtf(q2 / (float)d + p.eps);
       // the statistics slot: the epilogue must be done with the tile it held
       const int sl = it % NACC;
-      if (it >= NACC && !mbar_wait_bounded(acc_empty + sl, ((it / NACC) - 1) & 1, p.status)) break;
+      mbar_wait_warp(acc_empty + sl, ((it / NACC) & 1) ^ 1, p.status);
       if (part == 0) stats[sl * 128 + r] = make_float2(rstd, -mean * rstd);
       arrive(stats_full + sl);
       arrive(raw_empty + rb);
@@ -314,14 +319,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       *reinterpret_cast<uint4*>(sPV + piece(d + 8)) = make_uint4(0x3C003C00u, 0x3C003C00u, 0x3C003C00u, 0x3C003C00u);
     }
     const uint32_t idesc = umma_idesc_f16(BM, d + 16) | (1u << 15) | (1u << 16);  // A and B MN-major
-    const bool wok = mbar_wait_bounded(w_full, 0, p.status);
-    if (wok && ew * 32 + lane < Nh) wsum[ew * 32 + lane] = weight_colsum(sW, Nh, NKB, ew * 32 + lane);
+    mbar_wait_warp(w_full, 0, p.status);
+    if (ew * 32 + lane < Nh) wsum[ew * 32 + lane] = weight_colsum(sW, Nh, NKB, ew * 32 + lane);
     epi_sync();
     int it = 0;
-    for (int t = tile_at(it); t >= 0 && wok; t = tile_at(++it)) {
+    for (int t = tile_at(it); t >= 0; t = tile_at(++it)) {
       const int pos = it % Ts;   // row block of the segment
-      if (!mbar_wait_bounded(acc_full, it & 1, p.status)) break;
-      if (!mbar_wait_bounded(stats_full, it & 1, p.status)) break;
+      mbar_wait_warp(acc_full, it & 1, p.status);
+      mbar_wait_warp(stats_full, it & 1, p.status);
       tc_fence_after();
       const float2 st = stats[r];  // rstd, -rstd mu of this thread's row
       for (int c = 32 * sub; c < 2 * d; c += 64) {
@@ -336,7 +341,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int i = 0; i < 32; ++i) v[i] = phi_elu1(v[i]);
         }
         // the previous row block's state product must be done reading the operand tiles
-        if (c < 64 && it > 0 && !mbar_wait_bounded(st_full, (it - 1) & 1, p.status)) break;
+        if (c < 64 && it > 0) mbar_wait_warp(st_full, (it - 1) & 1, p.status);
         uint8_t* buf = isk ? sPK : sPV;
 #pragma unroll
         for (int j = 0; j < 4; ++j)
@@ -362,7 +367,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (pos + 1 < Ts) continue;
       // the segment's last row block: its state, S of each head from the
       // diagonal blocks and z, stored (one segment per CTA pair: no atomics)
-      if (!mbar_wait_bounded(st_full, it & 1, p.status)) break;
+      mbar_wait_warp(st_full, it & 1, p.status);
       tc_fence_after();
       const int seg = (t * BM) / p.C;
       float* st_seg = p.states + ((size_t)seg * 2 + l) * H * SB;
@@ -393,15 +398,15 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t lane_off = (uint32_t)(q * 32) << 16;
     uint8_t* stg0 = sStg + (size_t)ew * kStgBufs * kStage;
     const int r = q * 32 + lane;  // this thread's row of the tile
-    const bool wok = mbar_wait_bounded(w_full, 0, p.status);
-    if (wok && ew * 32 + lane < Nh) wsum[ew * 32 + lane] = weight_colsum(sW, Nh, NKB, ew * 32 + lane);
+    mbar_wait_warp(w_full, 0, p.status);
+    if (ew * 32 + lane < Nh) wsum[ew * 32 + lane] = weight_colsum(sW, Nh, NKB, ew * 32 + lane);
     asm volatile("bar.sync 5, 256;" ::: "memory");  // the eight epilogue warps: column sums written
     int nstore = 0;
     int it = 0;
-    for (int t = tile_at(it); t >= 0 && wok; t = tile_at(++it)) {
+    for (int t = tile_at(it); t >= 0; t = tile_at(++it)) {
       const int ab = it & 1;
-      if (!mbar_wait_bounded(acc_full + ab, (it >> 1) & 1, p.status)) break;
-      if (!mbar_wait_bounded(stats_full + ab, (it >> 1) & 1, p.status)) break;
+      mbar_wait_warp(acc_full + ab, (it >> 1) & 1, p.status);
+      mbar_wait_warp(stats_full + ab, (it >> 1) & 1, p.status);
       tc_fence_after();
       const float2 st = stats[ab * 128 + r];  // rstd, -rstd mu of this thread's row
       const int srow = t * BM + q * 32;

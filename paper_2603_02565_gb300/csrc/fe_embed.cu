@@ -41,21 +41,8 @@ constexpr size_t kSmem = 1024 + kWBytes + kABytes + kStgBytes + 128 * 4 + 128 * 
 __device__ __forceinline__ void arrive1(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-// The eight gather / epilogue warps: a barrier, and one that also returns the
-// AND of their flags (so that they leave the tile loop together)
+// The eight gather / epilogue warps
 __device__ __forceinline__ void gather_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
-__device__ __forceinline__ bool gather_sync_and(bool v) {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\t"
-      "setp.ne.u32 p, %1, 0;\n\t"
-      "bar.red.and.pred q, 1, 256, p;\n\t"
-      "selp.u32 %0, 1, 0, q;\n\t}"
-      : "=r"(r)
-      : "r"((uint32_t)v)
-      : "memory");
-  return r != 0;
-}
 __device__ __forceinline__ float lo16(uint32_t v) { return __uint_as_float(v << 16); }
 __device__ __forceinline__ float hi16(uint32_t v) { return __uint_as_float(v & 0xFFFF0000u); }
 __device__ __forceinline__ float sum8(const uint4& q) {
@@ -81,6 +68,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* a_full = bars + 1;    // operand tile written
   uint64_t* acc_full = bars + 2;  // product complete in TMEM
   uint64_t* acc_empty = bars + 3; // product read by the epilogue
+  uint64_t* drain = bars + 5;     // the products in flight at the end
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 4);
   int* sOff = reinterpret_cast<int*>(bars + 32);  // [B + 1] request offsets (when B < kMaxOff)
 
@@ -90,6 +78,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     mbar_init(a_full, 32 * kGWarps);
     mbar_init(acc_full, 1);
     mbar_init(acc_empty, kGWarps);
+    mbar_init(drain, 1);
     fence_mbar_init();
     prefetch_tmap(&tW);
     prefetch_tmap(&tQ);
@@ -116,27 +105,27 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 
   if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- MMA issuer ----------------
-      const uint32_t idesc = umma_idesc_bf16(BM, d);
-      bool ok = mbar_wait_bounded(w_full, 0, p.status);
-      int tl = 0;
-      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++tl) {
-        if (tl > 0 && !mbar_wait_bounded(acc_empty, (tl - 1) & 1, p.status)) break;
-        if (!mbar_wait_bounded(a_full, tl & 1, p.status)) break;
-        tc_fence_after();
-        const uint64_t a0 = umma_desc_sw128(smem_u32(sA));
-        const uint64_t w0 = umma_desc_sw128(smem_u32(sW));
+    // ---------------- MMA issuer (whole warp: fe_common.cuh) ----------------
+    const uint32_t issue = elect_one();
+    const uint32_t idesc = umma_idesc_bf16(BM, d);
+    const uint64_t a0 = umma_desc_sw128(smem_u32(sA)), w0 = umma_desc_sw128(smem_u32(sW));
+    mbar_wait_warp(w_full, 0, p.status);
+    int tl = 0;
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++tl) {
+      if (tl > 0) mbar_wait_warp(acc_empty, (tl - 1) & 1, p.status);
+      mbar_wait_warp(a_full, tl & 1, p.status);
+      tc_fence_after();
 #pragma unroll
-        for (int kb = 0; kb < NKB; ++kb) {
+      for (int kb = 0; kb < NKB; ++kb) {
 #pragma unroll
-          for (int kk = 0; kk < BK / 16; ++kk)
-            umma_bf16(tmem, desc_adv(a0, (uint32_t)kb * kPlane + kk * 32),
-                      desc_adv(w0, (uint32_t)kb * (uint32_t)d * (BK * 2) + kk * 32), idesc, (kb | kk) != 0 ? 1u : 0u);
-        }
-        umma_commit(acc_full);
+        for (int kk = 0; kk < BK / 16; ++kk)
+          umma_bf16_if(tmem, desc_adv(a0, (uint32_t)kb * kPlane + kk * 32),
+                       desc_adv(w0, (uint32_t)kb * (uint32_t)d * (BK * 2) + kk * 32), idesc, (kb | kk) != 0 ? 1u : 0u,
+                       issue);
       }
+      umma_commit_if(acc_full, issue);
     }
+    umma_drain(drain, p.status, issue);
   } else if (warp >= 2) {
     // ---------------- gather + statistics, then epilogue (warps 2..9) ----------------
     const int gw = warp - 2;
@@ -156,10 +145,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     const bool off_staged = p.B < kMaxOff;
     if (off_staged)
       for (int i = gw * 32 + lane; i <= p.B; i += 32 * kGWarps) sOff[i] = p.off[i];
-    bool ok = mbar_wait_bounded(w_full, 0, p.status);
+    mbar_wait_warp(w_full, 0, p.status);
     {
       const int i = gw * 32 + lane;
-      if (ok && i < d) {
+      if (i < d) {
         float cs = 0.f;
         for (int kb = 0; kb < NKB; ++kb) {
           const uint8_t* wr = sW + ((size_t)kb * d + i) * (BK * 2);
@@ -169,16 +158,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         colsum[i] = cs;
       }
     }
-    bool go = gather_sync_and(ok);  // uniform over the eight warps
+    gather_sync();
     int nstore = 0, tl = 0;
-    for (int t = blockIdx.x; t < tiles && go; t += gridDim.x, ++tl) {
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++tl) {
       const int m0 = t * BM;
       // ---- gather (the previous tile's product, which read the operand tile,
       // is complete: every warp has waited for it; its statistics are read)
-      if (tl > 0) {
-        go = gather_sync_and(ok);
-        if (!go) break;
-      }
+      if (tl > 0) gather_sync();
       const int row = m0 + gr;
       const bool valid = row < rows_valid;
       uint4 pc[kPieces];
@@ -251,12 +237,11 @@ __global__ void __launch_bounds__(kThreads, 1)
       arrive1(a_full);
       gather_sync();  // every row's statistics written
       // ---- epilogue: Q = rstd acc - rstd mu colsum, f16, through the staging blocks
-      // (a wait that gives up skips it; the warps leave the loop together at the top)
-      ok = mbar_wait_bounded(acc_full, tl & 1, p.status);
+      mbar_wait_warp(acc_full, tl & 1, p.status);
       tc_fence_after();
       const float2 st = stats[er];
       const int srow = m0 + q * 32;
-      for (int c = 32 * half; c < d && ok; c += 64) {
+      for (int c = 32 * half; c < d; c += 64) {
         float v[32];
         tmem_ld32(tmem + lane_off + (uint32_t)c, v);
 #pragma unroll
@@ -286,7 +271,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (lane == 0) bulk_wait0();  // Q stores complete before the CTA retires
   }
 
-  __syncwarp();  // each warp arrives whole: single lanes ran the MMA loop
+  __syncwarp();
   tc_fence_before();
   __syncthreads();
   if (warp == 0) tmem_dealloc(tmem, 128);
