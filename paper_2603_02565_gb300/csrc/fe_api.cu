@@ -110,7 +110,7 @@ struct Planes {
   int rows = 0;
   CUtensorMap th{}, tl{};  // operand loads: 64 x 128 boxes, 128-byte swizzle
   CUtensorMap sh{}, sl{};  // epilogue stores: 32 x 32 boxes, 64-byte swizzle
-  CUtensorMap ah{}, al{};  // attention queries: d_h x 128 boxes
+  CUtensorMap ah{}, al{};  // attention queries: d_h x 32 boxes
   CUtensorMap kh{}, kl{};  // attention keys / values: d_h x (64 for d_h = 32, else 128) boxes
 };
 
@@ -233,7 +233,7 @@ int map_attn(Planes& p, int dh) {
   const int kv_rows = fe::attn_chunk_keys(dh);
   int rc = encode_map_t(&p.sh, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, p.h, p.ld, p.rows, 32, 32,
                         CU_TENSOR_MAP_SWIZZLE_64B);
-  if (rc == FE_OK) rc = encode_map_t(&p.ah, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, p.h, p.ld, p.rows, dh, 128, sw);
+  if (rc == FE_OK) rc = encode_map_t(&p.ah, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, p.h, p.ld, p.rows, dh, 32, sw);
   if (rc == FE_OK) rc = encode_map_t(&p.kh, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, p.h, p.ld, p.rows, dh, kv_rows, sw);
   return rc;
 }

@@ -271,13 +271,13 @@ cudaError_t ctxkv_launch(const CUtensorMap* x, const CUtensorMap* w, const CUten
 // own rows [q_off(b), q_off(b) + q_cnt(b)) (self-attention within segments).  Head h reads columns q_col + h*dh
 // of Q, k_col + h*dh of K, v_col + h*dh of V (each one f16 plane) and writes
 // columns o_col + h*dh of the bf16 hi/lo output planes.  The Q map has boxes
-// of dh x 128, the K/V maps dh x (64 for dh = 32, else 128), with the 64-byte
+// of dh x 32, the K/V maps dh x (64 for dh = 32, else 128), with the 64-byte
 // (dh = 32) or 128-byte (dh = 64) swizzle.
 // ---------------------------------------------------------------------------
 struct AttnParams {
   int n_segments, n_heads;
   int max_q;             // largest q_cnt of any segment (grid sizing)
-  int max_q_tiles;       // set by attn_launch
+  int sb, tp;            // segments and query tiles of a round (set by attn_launch)
   const int* q_off_dev;  // null: q_off = b * q_stride
   const int* q_cnt_dev;  // null: q_cnt = q_cnt_fixed
   int q_stride;
