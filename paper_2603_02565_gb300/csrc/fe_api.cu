@@ -838,7 +838,7 @@ int enqueue_batch(fe_ctx* c, const Shape& sh, const IoPtrs& io, cudaStream_t s) 
   if (c->cfg.linear_context_attn && !lin_fused) {
     Prof pf(c, "lin_state", sc);
     FE_CK(fe::lin_state_launch(c->KV.h, c->fused_ctxkv ? 1 : 0, c->KV.rows, c->KV.ld, fact ? B * K : B, C, d, c->dh,
-                               Ly, c->H, c->lin_states, sc));
+                               Ly, c->H, c->lin_states, c->status, sc));
   }
   if (fork) FE_CK(cudaEventRecord(c->kv_ev, sc));
   // (a2) distinct elements: gather + LN (+ the first layer's Q), then the cross-attention stack

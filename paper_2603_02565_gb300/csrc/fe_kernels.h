@@ -312,7 +312,7 @@ cudaError_t attn_launch(int dh, const CUtensorMap* q, const CUtensorMap* k, cons
 // ---------------------------------------------------------------------------
 cudaError_t linattn_prepare();
 cudaError_t lin_state_launch(const bf16* kv, int hm, int rows_alloc, int ld, int n_seg, int C, int d, int dh, int Ly,
-                             int H, float* states, cudaStream_t s);
+                             int H, float* states, int* status, cudaStream_t s);
 cudaError_t lin_attn_launch(const bf16* q, int ldq, const float* states, int n_seg, int Ly, int l, int H, int dh,
                             const int* off_dev, const int* cnt_dev, int stride, int cnt_fixed, bf16* o_h, bf16* o_l,
                             int ldo, cudaStream_t s);

@@ -11,12 +11,10 @@
 // instead of C key/value rows), and an element query q reads
 //     a = phi(q) S / (phi(q) . z).
 //
-//   lin_state_kernel : one CTA per (segment, layer x head); streams the
-//                      segment's C key/value rows through shared memory in
-//                      64-row chunks (16-byte loads of the next chunk in
-//                      flight while the current one is multiplied), every
-//                      thread owning a 2x2 (d_h = 32) or 4x4 (d_h = 64) tile
-//                      of S
+//   lin_state_kernel : one CTA per (segment, layer, group of up to 128
+//                      features); streams the segment's C key/value rows
+//                      through operand tiles of 64 rows, phi(K)^T [V | 1] on
+//                      the tensor core
 //   lin_attn_kernel  : one CTA per segment; the segment's states of one layer
 //                      (all heads) and phi(q) of 32-row blocks in shared
 //                      memory, one warp per (head, 16 rows), a lane per
@@ -41,29 +39,62 @@ __device__ __forceinline__ float warp_sum32(float v) {
   return v;
 }
 
-constexpr int kChunk = 64;  // context rows per shared-memory chunk
+constexpr int kChunk = 64;                // context rows per operand tile
+constexpr uint32_t kAtom = kChunk * 128;  // 64 features x kChunk rows, f16
+
+// MN-major operand descriptor, 128-byte swizzle: atoms of 64 features, kAtom apart, 8-row groups 1024 bytes apart
+__device__ __forceinline__ uint64_t desc_feat(uint32_t saddr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
+  d |= (uint64_t)(kAtom >> 4) << 16;
+  d |= (uint64_t)(1024 >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)2 << 61;
+  return d;
+}
+
+// operand tiles of a chunk: phi(K) hi and lo (128 features each), V and the ones columns
+template <int FG>
+struct StateCfg {
+  static constexpr uint32_t kA = 2 * kAtom;
+  static constexpr uint32_t kV = (FG == 128 ? 3 : FG == 64 ? 2 : 1) * kAtom;
+  static constexpr uint32_t kBuf = 2 * kA + kV;
+  static constexpr size_t kSmem = 2 * kBuf + 64;  // two buffers, barriers
+  // three accumulators: the hi products of even and of odd chunks, the lo products
+  static constexpr int kN = FG + 16;
+  static constexpr uint32_t kCols = 3 * kN <= 256 ? 256 : 512;
+};
 
 }  // namespace
 
 // Context states.  A CTA takes one segment, one layer and one group of FG
-// features (FG = min(d, 128): the heads [g FG / DH, (g + 1) FG / DH)); every
-// thread owns a TI x TJ tile of one head's S, so a context row costs it one
-// 16-byte load of phi(K) and TJ / 4 of V for TI * TJ multiply-adds.
+// features (FG = min(d, 128): the heads [g FG / DH, (g + 1) FG / DH)).  Per
+// 64 context rows its threads write phi(K), as a hi + lo pair of f16 tiles (22
+// bits), and V, an exact f16 tile followed by 16 columns of ones, and the tensor
+// core adds phi(K)^T [V | 1] to 128 x (FG + 16) accumulators in TMEM (z comes from
+// the ones columns; three accumulators, because the tensor core truncates each
+// addition); at the end each head's diagonal block and z are stored.  Two
+// operand buffers: the next chunk's rows are transformed and written
+// while the current one is multiplied, and the rows of two chunks are in flight.
+// What bounds it: the transform of K (an exponent, two conversions and a 16-byte
+// store per plane for 8 values); the products take 8 MMAs of N = FG + 16 a chunk.
+// 256 segments of 1000 rows, two layers of 64 columns: 107 us with fp32 products on the
+// CUDA cores, 60 us here with one chunk's rows in flight, 53 with two (131 MB of K/V, 20 us
+// at the copy rate); the 512 CTAs are 1.7 waves of two per SM.
 template <int DH, int FG>
-__global__ void __launch_bounds__(256) lin_state_kernel(const __half* __restrict__ kv, int hm, int rows_alloc, int ld,
-                                                        int C, int d, int H, float* __restrict__ states) {
+__global__ void __launch_bounds__(256, 2) lin_state_kernel(const __half* __restrict__ kv, int hm, int rows_alloc,
+                                                           int ld, int C, int d, int H, float* __restrict__ states,
+                                                           int* status) {
+  using Cfg = StateCfg<FG>;
   constexpr int HG = FG / DH;               // heads per group
-  constexpr int TI = 4;
-  constexpr int TJ = DH == 32 ? 4 : 8;
-  constexpr int TPH = DH * DH / (TI * TJ);  // threads per head (64 or 128); HG * TPH <= 256 are active
-  constexpr int NJT = DH / TJ;              // tiles along j
   constexpr int SB = DH * DH + DH;
-  constexpr int RC = 32;                    // context rows per chunk
-  constexpr int NP = RC * FG / 8;           // 16-byte pieces of a chunk, for K and for V
-  constexpr int P8 = (NP + 255) / 256;      // per thread
-  static_assert(HG * TPH <= 256, "tiling");
-  __shared__ __align__(16) float sK[RC][FG];  // phi(K) rows of the chunk
-  __shared__ __align__(16) float sV[RC][FG];
+  constexpr int NP = kChunk * FG / 8;       // 16-byte pieces of a chunk, for K and for V
+  constexpr int P8 = NP / 256;              // per thread
+  static_assert(NP % 256 == 0, "tiling");
+  extern __shared__ __align__(1024) uint8_t sm_state[];
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sm_state + 2 * Cfg::kBuf);
+  uint64_t* free_bar = bars;                // [2] the products of the chunk in this buffer are complete
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2);
   const int s = blockIdx.x, G = d / FG, l = blockIdx.y / G, g = blockIdx.y % G;
   const int kcol = 2 * l * d + g * FG, vcol = (2 * l + 1) * d + g * FG;
   const size_t row0 = (size_t)s * C;
@@ -71,24 +102,39 @@ __global__ void __launch_bounds__(256) lin_state_kernel(const __half* __restrict
   auto at = [&](size_t row, int col) -> size_t {
     return hm ? ((size_t)(col / DH) * rows_alloc + row) * DH + (col % DH) : row * ld + col;
   };
-  const int t = threadIdx.x, hh = t / TPH, tl = t % TPH;
-  const bool active = hh < HG;
-  const int fi = hh * DH + (tl / NJT) * TI;   // feature of S's first row in this tile
-  const int fj = hh * DH + (tl % NJT) * TJ;   // feature of its first column
-  const bool zrow = (tl % NJT) == 0;          // one column of tiles also sums phi(K) into z
-  float acc[TI][TJ];
-#pragma unroll
-  for (int x = 0; x < TI; ++x)
-#pragma unroll
-    for (int y = 0; y < TJ; ++y) acc[x][y] = 0.f;
-  float zacc[TI] = {0.f, 0.f, 0.f, 0.f};
-  uint4 kr[P8], vr[P8];
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  // the 16-byte piece of (row r, features m .. m + 7) in an operand tile
+  auto piece = [](int r, int m) {
+    return (uint32_t)(m >> 6) * kAtom + (uint32_t)r * 128u + ((((uint32_t)(m & 63) >> 3) ^ (uint32_t)(r & 7)) << 4);
+  };
+  if (t == 0) {
+    mbar_init(free_bar, 1);
+    mbar_init(free_bar + 1, 1);
+    fence_mbar_init();
+  }
+  if (warp == 0) tmem_alloc(tmem_slot, Cfg::kCols);
+  // features FG .. 127 of phi(K) are zeros, V's columns FG .. FG + 15 ones
+  for (int i = t; i < 2 * kChunk; i += 256) {
+    const int r = i % kChunk;
+    uint8_t* buf = sm_state + (size_t)(i / kChunk) * Cfg::kBuf;
+    for (int m = FG; m < 128; m += 8) {
+      *reinterpret_cast<uint4*>(buf + piece(r, m)) = make_uint4(0u, 0u, 0u, 0u);
+      *reinterpret_cast<uint4*>(buf + Cfg::kA + piece(r, m)) = make_uint4(0u, 0u, 0u, 0u);
+    }
+    const uint32_t one2 = 0x3C003C00u;
+    *reinterpret_cast<uint4*>(buf + 2 * Cfg::kA + piece(r, FG)) = make_uint4(one2, one2, one2, one2);
+    *reinterpret_cast<uint4*>(buf + 2 * Cfg::kA + piece(r, FG + 8)) = make_uint4(one2, one2, one2, one2);
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
   // the 16-byte pieces of a chunk this thread loads; rows past C read as zero
-  auto load = [&](int r0) {
+  auto load = [&](int r0, uint4* kr, uint4* vr) {
 #pragma unroll
     for (int q = 0; q < P8; ++q) {
       const int idx = t + 256 * q, r = idx / (FG / 8), c8 = (idx % (FG / 8)) * 8;
-      if (idx < NP && r0 + r < C) {
+      if (r0 + r < C) {
         kr[q] = *reinterpret_cast<const uint4*>(kv + at(row0 + r0 + r, kcol + c8));
         vr[q] = *reinterpret_cast<const uint4*>(kv + at(row0 + r0 + r, vcol + c8));
       } else {
@@ -97,75 +143,99 @@ __global__ void __launch_bounds__(256) lin_state_kernel(const __half* __restrict
       }
     }
   };
-  pdl_wait();
-  pdl_trigger();
-  load(0);
-  for (int r0 = 0; r0 < C; r0 += RC) {
-    const int nr = min(RC, C - r0);
-    __syncthreads();  // the previous chunk is consumed
+  const uint32_t go = elect_one();
+  const uint32_t idesc = umma_idesc_f16(128, Cfg::kN) | (1u << 15) | (1u << 16);  // A and B MN-major
+  // chunk it (its pieces in kr, vr; chunk it + 2's are then loaded into them) through operand buffer B
+  auto chunk = [&](auto bufc, int it, uint4* kr, uint4* vr) {
+    constexpr int B = decltype(bufc)::value;
+    const int r0 = it * kChunk;
+    uint8_t* buf = sm_state + (size_t)B * Cfg::kBuf;
+    if (it >= 2) mbar_wait_warp(free_bar + B, ((it >> 1) - 1) & 1, status);
 #pragma unroll
     for (int q = 0; q < P8; ++q) {
       const int idx = t + 256 * q, r = idx / (FG / 8), c8 = (idx % (FG / 8)) * 8;
-      if (idx >= NP) continue;
-      const __half* hk = reinterpret_cast<const __half*>(&kr[q]);
-      const __half* hv = reinterpret_cast<const __half*>(&vr[q]);
-      const bool valid = r < nr;
-      float4 k0, k1, v0, v1;
-      k0.x = valid ? phi(__half2float(hk[0])) : 0.f;  // a missing row adds nothing
-      k0.y = valid ? phi(__half2float(hk[1])) : 0.f;
-      k0.z = valid ? phi(__half2float(hk[2])) : 0.f;
-      k0.w = valid ? phi(__half2float(hk[3])) : 0.f;
-      k1.x = valid ? phi(__half2float(hk[4])) : 0.f;
-      k1.y = valid ? phi(__half2float(hk[5])) : 0.f;
-      k1.z = valid ? phi(__half2float(hk[6])) : 0.f;
-      k1.w = valid ? phi(__half2float(hk[7])) : 0.f;
-      v0 = make_float4(__half2float(hv[0]), __half2float(hv[1]), __half2float(hv[2]), __half2float(hv[3]));
-      v1 = make_float4(__half2float(hv[4]), __half2float(hv[5]), __half2float(hv[6]), __half2float(hv[7]));
-      *reinterpret_cast<float4*>(&sK[r][c8]) = k0;
-      *reinterpret_cast<float4*>(&sK[r][c8 + 4]) = k1;
-      *reinterpret_cast<float4*>(&sV[r][c8]) = v0;
-      *reinterpret_cast<float4*>(&sV[r][c8 + 4]) = v1;
+      const bool valid = r0 + r < C;  // a missing row adds nothing
+      const __half2* hk = reinterpret_cast<const __half2*>(&kr[q]);
+      uint32_t hi[4], lo[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float2 x = __half22float2(hk[e]);
+        const float f0 = valid ? phi(x.x) : 0.f, f1 = valid ? phi(x.y) : 0.f;
+        const __half2 h = __floats2half2_rn(f0, f1);
+        const float2 hf = __half22float2(h);
+        hi[e] = *reinterpret_cast<const uint32_t*>(&h);
+        lo[e] = pack_f16x2(f0 - hf.x, f1 - hf.y);
+      }
+      *reinterpret_cast<uint4*>(buf + piece(r, c8)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+      *reinterpret_cast<uint4*>(buf + Cfg::kA + piece(r, c8)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+      *reinterpret_cast<uint4*>(buf + 2 * Cfg::kA + piece(r, c8)) = vr[q];
     }
+    fence_async_shared();
+    tc_fence_before();
     __syncthreads();
-    if (r0 + RC < C) load(r0 + RC);  // in flight during the products below
-#pragma unroll 4
-    for (int r = 0; r < (active ? nr : 0); ++r) {
-      const float4 ka = *reinterpret_cast<const float4*>(&sK[r][fi]);
-      const float a[4] = {ka.x, ka.y, ka.z, ka.w};
-      float b[TJ];
+    if (r0 + 2 * kChunk < C) load(r0 + 2 * kChunk, kr, vr);  // in flight for a whole chunk (issued before the fence, it waited for them)
+    if (warp == 0) {
+      tc_fence_after();
+      const uint64_t ah = desc_feat(smem_u32(buf)), al = desc_feat(smem_u32(buf + Cfg::kA)),
+                     bd = desc_feat(smem_u32(buf + 2 * Cfg::kA));
 #pragma unroll
-      for (int y = 0; y < TJ; y += 4) {
-        const float4 vb = *reinterpret_cast<const float4*>(&sV[r][fj + y]);
-        b[y] = vb.x;
-        b[y + 1] = vb.y;
-        b[y + 2] = vb.z;
-        b[y + 3] = vb.w;
+      for (int kk = 0; kk < kChunk / 16; ++kk) {
+        const uint32_t o = (uint32_t)kk * 16u * 128u;
+        umma_bf16_if(tmem + (uint32_t)(B * Cfg::kN), desc_adv(ah, o), desc_adv(bd, o), idesc,
+                     (it > 1 || kk != 0) ? 1u : 0u, go);
+        umma_bf16_if(tmem + 2u * Cfg::kN, desc_adv(al, o), desc_adv(bd, o), idesc, (it | kk) != 0 ? 1u : 0u, go);
+      }
+      umma_commit_if(free_bar + B, go);
+    }
+  };
+  pdl_trigger();
+  pdl_wait();
+  uint4 k0[P8], v0[P8], k1[P8], v1[P8];
+  load(0, k0, v0);
+  load(kChunk, k1, v1);
+  const int it_end = (C + kChunk - 1) / kChunk;
+  for (int i = 0; i < it_end; i += 2) {
+    chunk(std::integral_constant<int, 0>{}, i, k0, v0);
+    if (i + 1 < it_end) chunk(std::integral_constant<int, 1>{}, i + 1, k1, v1);
+  }
+  // the last product (and so every earlier one) complete
+  mbar_wait_warp(free_bar + ((it_end - 1) & 1), ((it_end - 1) >> 1) & 1, status);
+  tc_fence_after();
+  // lane m of the accumulator: feature m of the group; its head's DH columns, and z in column FG
+  const int q = warp & 3, sub = warp >> 2, m = 32 * q + lane;
+  const int Ly = gridDim.y / G;
+  if (32 * q < FG) {
+    const int hh = m / DH, i = m % DH;
+    float* st = states + (((size_t)s * Ly + l) * H + g * HG + hh) * SB;  // S row-major, then z
+    const uint32_t row = tmem + ((uint32_t)(q * 32) << 16);
+    const bool odd = it_end > 1;  // (a single chunk leaves the second accumulator unwritten)
+    if (sub == 0 || DH == 64) {
+      const uint32_t col = row + (uint32_t)((32 * q) / DH * DH + 32 * sub);
+      float v[32], w[32];
+      tmem_ld32(col, v);
+      tmem_ld32(col + 2u * Cfg::kN, w);
+#pragma unroll
+      for (int j = 0; j < 32; ++j) v[j] += w[j];
+      if (odd) {
+        tmem_ld32(col + (uint32_t)Cfg::kN, w);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) v[j] += w[j];
       }
 #pragma unroll
-      for (int x = 0; x < TI; ++x)
-#pragma unroll
-        for (int y = 0; y < TJ; ++y) acc[x][y] = fmaf(a[x], b[y], acc[x][y]);
-      if (zrow) {
-#pragma unroll
-        for (int x = 0; x < TI; ++x) zacc[x] += a[x];
-      }
+      for (int j = 0; j < 32; j += 4)
+        *reinterpret_cast<float4*>(st + i * DH + 32 * sub + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+    }
+    if (sub == (DH == 64 ? 0 : 1)) {
+      uint32_t z[8], w[8], u[8];
+      tmem_ld8(row + (uint32_t)FG, z);
+      tmem_ld8(row + (uint32_t)(Cfg::kN + FG), u);
+      tmem_ld8(row + (uint32_t)(2 * Cfg::kN + FG), w);
+      st[DH * DH + i] = __uint_as_float(z[0]) + __uint_as_float(w[0]) + (odd ? __uint_as_float(u[0]) : 0.f);
     }
   }
-  if (!active) return;
-  const int h = g * HG + hh;
-  const int Ly = gridDim.y / G;
-  float* st = states + (((size_t)s * Ly + l) * H + h) * SB;  // S row-major, then z
-  const int i0 = fi - hh * DH, j0 = fj - hh * DH;
-#pragma unroll
-  for (int x = 0; x < TI; ++x)
-#pragma unroll
-    for (int y = 0; y < TJ; y += 4)
-      *reinterpret_cast<float4*>(st + (i0 + x) * DH + j0 + y) =
-          make_float4(acc[x][y], acc[x][y + 1], acc[x][y + 2], acc[x][y + 3]);
-  if (zrow) {
-#pragma unroll
-    for (int x = 0; x < TI; ++x) st[DH * DH + i0 + x] = zacc[x];
-  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) tmem_dealloc(tmem, Cfg::kCols);
 }
 
 namespace {
@@ -303,25 +373,31 @@ cudaError_t linattn_prepare() {
                                        kLinAttnSmemMax);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(lin_attn_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLinAttnSmemMax);
+  auto state = [&](const void* f, size_t smem) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  };
+  state((const void*)lin_state_kernel<32, 128>, StateCfg<128>::kSmem);
+  state((const void*)lin_state_kernel<32, 64>, StateCfg<64>::kSmem);
+  state((const void*)lin_state_kernel<64, 128>, StateCfg<128>::kSmem);
+  state((const void*)lin_state_kernel<64, 64>, StateCfg<64>::kSmem);
+  state((const void*)lin_state_kernel<32, 32>, StateCfg<32>::kSmem);
   return e;
 }
 
 cudaError_t lin_state_launch(const bf16* kv, int hm, int rows_alloc, int ld, int n_seg, int C, int d, int dh, int Ly,
-                             int H, float* states, cudaStream_t s) {
+                             int H, float* states, int* status, cudaStream_t s) {
   if (n_seg <= 0 || C <= 0) return cudaSuccess;
   const int FG = d < 128 ? d : 128;
   const dim3 grid((unsigned)n_seg, (unsigned)(Ly * (d / FG)));
   const __half* k = reinterpret_cast<const __half*>(kv);
-  if (dh == 32 && FG == 128)
-    return launch_k(lin_state_kernel<32, 128>, grid, dim3(256), 0, s, k, hm, rows_alloc, ld, C, d, H, states);
-  if (dh == 32 && FG == 64)
-    return launch_k(lin_state_kernel<32, 64>, grid, dim3(256), 0, s, k, hm, rows_alloc, ld, C, d, H, states);
-  if (dh == 64 && FG == 128)
-    return launch_k(lin_state_kernel<64, 128>, grid, dim3(256), 0, s, k, hm, rows_alloc, ld, C, d, H, states);
-  if (dh == 64 && FG == 64)
-    return launch_k(lin_state_kernel<64, 64>, grid, dim3(256), 0, s, k, hm, rows_alloc, ld, C, d, H, states);
-  if (dh == 32 && FG == 32)
-    return launch_k(lin_state_kernel<32, 32>, grid, dim3(256), 0, s, k, hm, rows_alloc, ld, C, d, H, states);
+  auto go = [&](auto kern, size_t smem) {
+    return launch_k(kern, grid, dim3(256), smem, s, k, hm, rows_alloc, ld, C, d, H, states, status);
+  };
+  if (dh == 32 && FG == 128) return go(lin_state_kernel<32, 128>, StateCfg<128>::kSmem);
+  if (dh == 32 && FG == 64) return go(lin_state_kernel<32, 64>, StateCfg<64>::kSmem);
+  if (dh == 64 && FG == 128) return go(lin_state_kernel<64, 128>, StateCfg<128>::kSmem);
+  if (dh == 64 && FG == 64) return go(lin_state_kernel<64, 64>, StateCfg<64>::kSmem);
+  if (dh == 32 && FG == 32) return go(lin_state_kernel<32, 32>, StateCfg<32>::kSmem);
   return cudaErrorInvalidValue;
 }
 
