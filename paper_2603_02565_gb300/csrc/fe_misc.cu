@@ -640,6 +640,108 @@ __global__ void __launch_bounds__(256) cls_attn_kernel(const ClsParams p, int W)
   }
 }
 
+// The same for launches of kRowsWarps warps and more at NS = 32 / H consecutive
+// sequences per warp, with L <= kRowsMaxL.  First lane (sequence q, head h)
+// runs that pair's softmax recurrence over the L keys and leaves each key's two
+// factors in shared memory (the row rescaling c = exp(m_old - m_new) and the weight
+// e = exp(s - m_new)); then, sequence by sequence, the lanes accumulate the value
+// rows, DPL columns each.  The kernel above has every lane repeat both exponentials
+// of its head for every key and waits for them between two gathers; here a key costs
+// its gathered row and the multiply-adds, and four rows are in flight.  Same
+// operations in the same order, so the same result.
+// What bounds it: the gathered rows from L2 (2.1 GB for 204800 sequences of 10 keys
+// at d = 256).  Measured against the kernel above: those 349 -> 262 us, 64000 of 10
+// at d = 128 90 -> 58.
+constexpr int kRowsMaxL = 32;
+constexpr long long kRowsWarps = 4000;
+
+template <int DPL, int DH>
+__global__ void __launch_bounds__(256) cls_rows_kernel(const ClsParams p) {
+  constexpr int d = 32 * DPL, H = d / DH, NS = 32 / H, NCH = DPL, CPH = DH / 32;
+  extern __shared__ float cls_sm[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int L = p.L, n = p.B * p.K;
+  const bool vp_smem = L * d <= kVpStage;
+  float* svp = cls_sm;  // P WVs, when staged
+  float2* ce0 = reinterpret_cast<float2*>(cls_sm + (vp_smem ? L * d : 0));
+  float2* ce = ce0 + warp * NS * H * L;                                        // [q][j][h]
+  int* ser = reinterpret_cast<int*>(ce0 + 8 * NS * H * L) + warp * NS * L;  // [q][j]: element row
+  // P WVs rows are parameters: staged before the programmatic wait
+  if (vp_smem) {
+    const float4* src = reinterpret_cast<const float4*>(p.vP);
+    for (int i = threadIdx.x; i < L * d / 4; i += blockDim.x) reinterpret_cast<float4*>(svp)[i] = src[i];
+  }
+  const float* vpb = vp_smem ? svp : p.vP;
+  pdl_wait();
+  pdl_trigger();
+  if (vp_smem) __syncthreads();
+  const int s0 = (blockIdx.x * 8 + warp) * NS;  // the warp's first sequence
+  if (s0 >= n) return;
+  const int ns = min(NS, n - s0);
+  for (int i = lane; i < ns * L; i += 32) {
+    const int b = (s0 + i / L) / p.K;
+    ser[i] = p.off[b] + p.slot_local[(size_t)s0 * L + i];
+  }
+  __syncwarp();
+  // ---- lane (q, h): the recurrence of sequence q's head h
+  float inv = 1.f;
+  int keys = 0;  // of this lane's sequence (none for a rejected request)
+  {
+    const int q = lane / H, h = lane % H;
+    if (q < ns) {
+      keys = p.bad[(s0 + q) / p.K] ? 0 : L;
+      float m = p.qk0[h] * p.scale, l = 1.f;  // token 0: [CLS]
+#pragma unroll 4
+      for (int j = 0; j < keys; ++j) {
+        const float* lg = p.elog + (size_t)ser[q * L + j] * NCH + h * CPH;
+        float s = lg[0];
+        if (CPH > 1) s += lg[1];
+        s = (s + p.qkP[j * H + h]) * p.scale;
+        const float mn = fmaxf(m, s);
+        const float c = expf(m - mn);
+        const float e = expf(s - mn);
+        l = l * c + e;
+        m = mn;
+        ce[(q * L + j) * H + h] = make_float2(c, e);
+      }
+      inv = 1.f / l;
+    }
+  }
+  __syncwarp();
+  // ---- the sequences' rows: this lane's DPL columns, of head hd
+  const int d0 = lane * DPL, hd = lane * DPL / DH;
+  for (int q = 0; q < ns; ++q) {
+    const int nk = __shfl_sync(0xffffffffu, keys, q * H);
+    const float iv = __shfl_sync(0xffffffffu, inv, q * H + hd);
+    float o[DPL];
+    load_vec<DPL>(p.v0 + d0, o);
+#pragma unroll 4
+    for (int j = 0; j < nk; ++j) {
+      const size_t er = (size_t)ser[q * L + j];
+      float vx[DPL], vp[DPL];
+      load_split<DPL>(p.kv_h + er * p.ldkv + d + d0, p.kv_l + er * p.ldkv + d + d0, vx);
+      load_vec<DPL>(vpb + (size_t)j * d + d0, vp);
+      const float2 f = ce[(q * L + j) * H + hd];
+      const float c = f.x, e = f.y;
+#pragma unroll
+      for (int t = 0; t < DPL; ++t) o[t] = o[t] * c + e * (vx[t] + vp[t]);
+    }
+#pragma unroll
+    for (int i = 0; i < DPL; ++i) o[i] *= iv;
+    const size_t seq = (size_t)(s0 + q);
+    store_split<DPL>(o, p.o_h + seq * p.ldo + d0, p.o_l + seq * p.ldo + d0);
+  }
+}
+
+template <int DPL, int DH>
+static cudaError_t cls_rows_launch(const ClsParams& p, cudaStream_t s) {
+  constexpr int H = 32 * DPL / DH, NS = 32 / H;
+  const long long n = (long long)p.B * p.K;
+  const unsigned g = (unsigned)((n + 8 * NS - 1) / (8 * NS));
+  const size_t smem = (p.L * p.d <= kVpStage ? (size_t)p.L * p.d * 4 : 0) + (size_t)8 * NS * p.L * (H * 8 + 4);
+  return launch_k(cls_rows_kernel<DPL, DH>, dim3(g), dim3(256), smem, s, p);
+}
+
 cudaError_t cls_attn_launch(const ClsParams& p, cudaStream_t s) {
   const int n = p.B * p.K;
   if (n <= 0) return cudaSuccess;
@@ -647,6 +749,19 @@ cudaError_t cls_attn_launch(const ClsParams& p, cudaStream_t s) {
   // the gathered rows, at least two keys per warp
   int W = 1;
   while (W < 8 && 2 * W <= p.L && (long long)n * W < 4096) W *= 2;
+  // With fewer warps of 32 / H sequences the recurrence's latency is not covered: a whole batch of 19200
+  // sequences at d = 128 (2400 warps) took 177.5 -> 184.5 us, of 32000 (4000) 234.5 -> 225.8, of 64000 400 -> 368;
+  // of 6400 at d = 256 (1600 warps) 264 -> 274, of 19200 (4800) 506.7 -> 501.0.
+  if ((long long)n * p.H >= 32 * kRowsWarps && p.L >= 1 && p.L <= kRowsMaxL) {
+    const int dh = p.d / p.H;
+    switch (p.d) {
+      case 64: return dh == 32 ? cls_rows_launch<2, 32>(p, s) : cls_rows_launch<2, 64>(p, s);
+      case 128: return dh == 32 ? cls_rows_launch<4, 32>(p, s) : cls_rows_launch<4, 64>(p, s);
+      case 256: return dh == 32 ? cls_rows_launch<8, 32>(p, s) : cls_rows_launch<8, 64>(p, s);
+      case 512: return dh == 32 ? cls_rows_launch<16, 32>(p, s) : cls_rows_launch<16, 64>(p, s);
+      default: break;
+    }
+  }
   const unsigned g = (unsigned)((n + 8 / W - 1) / (8 / W));
   const size_t smem = ((W > 1 ? (size_t)(8 * p.d + 512) : 0) + (p.L * p.d <= kVpStage ? (size_t)p.L * p.d : 0)) *
                       sizeof(float);
@@ -745,7 +860,15 @@ bool pdl_enabled() {
 }
 
 cudaError_t misc_prepare() {
-  return cudaFuncSetAttribute(compact_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 65536 + 1024);
+  cudaError_t e = cudaFuncSetAttribute(compact_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 65536 + 1024);
+  for (const void* f : {(const void*)cls_rows_kernel<2, 32>, (const void*)cls_rows_kernel<2, 64>,
+                        (const void*)cls_rows_kernel<4, 32>, (const void*)cls_rows_kernel<4, 64>,
+                        (const void*)cls_rows_kernel<8, 32>, (const void*)cls_rows_kernel<8, 64>,
+                        (const void*)cls_rows_kernel<16, 32>, (const void*)cls_rows_kernel<16, 64>})
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               kVpStage * 4 + 8 * kRowsMaxL * (32 * 8 + 32 * 4));
+  return e;
 }
 
 }  // namespace fe
