@@ -23,13 +23,23 @@
 // partner warp, LN(x) as the split operand tile over the A tile, bias + ReLU
 // + split per chunk, x_out + b2 (staged over the A tile and stored by TMA),
 // LN(x_out) over the A tile (stored by TMA), and the tail's f16 output (over
-// the A tile, stored by TMA).  Products take split bf16 activations
-// (hi + lo) times exact bf16 weights with fp32 accumulation; LayerNorm and
-// residuals are fp32.
+// the upper half of the A tile, stored by TMA).  A tile's A and x0 are prefetched
+// into L2 during the chunks of the tile before it, and each k block of the A tile
+// is loaded as soon as the store that last used its memory has read it, so that
+// A W_O starts while the rest is still on its way out or in.  Products take split
+// bf16 activations (hi + lo) times exact bf16 weights with fp32 accumulation;
+// LayerNorm and residuals are fp32.
 // What bounds it: the tensor pipe (a chunk is 64 MMAs of N = 128, 4096 cycles, on
 // both halves of its weights) and, per tile, the two LayerNorm phases.  With
 // warps 0 and 1 run whole (fe_common.cuh) the largest batch (295k rows, two element
 // layers and SeqEnc) went from 5495 to 5035 us and 45 requests from 269.5 to 235.5.
+// A tile's first k block came 8.5k cycles after the previous tile's end (its stores
+// drain at 32 bytes a cycle, then DRAM, on every SM at once).  The prefetch took the
+// largest batch from 4073 to 3952 us, rolled epilogue loops (127 registers, none
+// spilled, less code to fetch than unrolled by 4) to 3932 and 45 requests from 219.6 to
+// 216.3, the release by k blocks the largest to 3896.
+// Holding a thread's 128 columns in registers through both LayerNorm passes, the loops
+// unrolled, was slower (45 requests 226.5).
 #include "fe_common.cuh"
 #include "fe_kernels.h"
 
@@ -46,6 +56,16 @@ __device__ __forceinline__ void tma_load_2d_hint_if(void* smem_dst, const CUtens
       "@q cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
       " [%0], [%1, {%3, %4}], [%2], %5;\n\t}" ::"r"(smem_u32(smem_dst)),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(x), "r"(y), "l"(policy), "r"(go)
+      : "memory");
+}
+// all but the newest of this thread's bulk stores have read their source
+__device__ __forceinline__ void bulk_wait_read1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
+// TMA 2D box into L2 only (predicated on go)
+__device__ __forceinline__ void tma_prefetch_2d_if(const CUtensorMap* map, int x, int y, uint32_t go) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %3, 0;\n\t"
+      "@q cp.async.bulk.prefetch.tensor.2d.L2.global [%0, {%1, %2}];\n\t}" ::"l"(reinterpret_cast<uint64_t>(map)),
+      "r"(x), "r"(y), "r"(go)
       : "memory");
 }
 __device__ __forceinline__ uint64_t l2_policy_evict_last() {
@@ -144,8 +164,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* bars = reinterpret_cast<uint64_t*>(misc + kMiscBars);
   uint64_t* w_full = bars;           // [kRing]
   uint64_t* w_empty = bars + 5;      // [kRing]
-  uint64_t* a_full = bars + 10;      // A tile loaded
-  uint64_t* a_free = bars + 11;      // sA free for the next tile (LN(x_out) stored and read by the tail)
+  uint64_t* a_full = bars + 24;      // [NKB] k block of the A tile loaded
+  uint64_t* a_free = bars + 28;      // [NKB] k block of sA free for the next tile
   uint64_t* o_done = bars + 12;      // A W_O complete
   uint64_t* ln_full = bars + 13;     // x in the accumulator, LN(x) in sA
   uint64_t* acc1_full = bars + 14;   // [2]
@@ -155,7 +175,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* tail_a = bars + 21;      // LN(x_out) in sA
   uint64_t* tail_full = bars + 22;   // the tail product complete
   uint64_t* drain = bars + 23;       // the products in flight at the end
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 24);
+  uint64_t* q_read = bars + 10;      // the tail product read
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 32);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int F = p.F, nf = F / FC;
@@ -164,8 +185,11 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(w_full + i, 1);
       mbar_init(w_empty + i, 1);
     }
-    mbar_init(a_full, 1);
-    mbar_init(a_free, kEpiWarps);
+    for (int i = 0; i < NKB; ++i) {
+      mbar_init(a_full + i, 1);
+      mbar_init(a_free + i, 1);
+    }
+    mbar_init(q_read, kEpiWarps);
     mbar_init(o_done, 1);
     mbar_init(ln_full, kEpiWarps);
     for (int i = 0; i < 2; ++i) {
@@ -226,11 +250,11 @@ __global__ void __launch_bounds__(kThreads, 1)
       // the previous tile still uses sA
       for (int i = 0; i < 2 * NKB; ++i) {
         if (i == kRing - 1) {
-          if (tl > 0) mbar_wait_warp(a_free, (tl - 1) & 1, p.status);
-          mbar_arrive_expect_tx_if(a_full, kABytes, go);
           for (int kb = 0; kb < NKB; ++kb) {
-            tma_load_2d_hint_if(sA + (size_t)(kb * 2) * kBox, &tA_h, kb * BK, t * BM, a_full, pass, go);
-            tma_load_2d_hint_if(sA + (size_t)(kb * 2 + 1) * kBox, &tA_l, kb * BK, t * BM, a_full, pass, go);
+            if (tl > 0) mbar_wait_warp(a_free + kb, (tl - 1) & 1, p.status);
+            mbar_arrive_expect_tx_if(a_full + kb, 2 * kBox, go);
+            tma_load_2d_hint_if(sA + (size_t)(kb * 2) * kBox, &tA_h, kb * BK, t * BM, a_full + kb, pass, go);
+            tma_load_2d_hint_if(sA + (size_t)(kb * 2 + 1) * kBox, &tA_l, kb * BK, t * BM, a_full + kb, pass, go);
           }
         }
         load(&tWO, (i >> 1) * BK, (i & 1) * 128);
@@ -241,6 +265,15 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (s >= 1)
           for (int i = 0; i < 4; ++i)  // (nh, sub): sub fastest
             load(&tW2, (s - 1) * FC + (i & 1) * BK, (i >> 1) * 128);
+        // the next tile's A and x0 into L2 meanwhile
+        if (t + gridDim.x < tiles)
+          for (int kb = s; kb < NKB; kb += nf + 1) {
+            const int y = (t + gridDim.x) * BM;
+            tma_prefetch_2d_if(&tA_h, kb * BK, y, go);
+            tma_prefetch_2d_if(&tA_l, kb * BK, y, go);
+            if (!p.x0_row)
+              for (int i = 0; i < 8; ++i) tma_prefetch_2d_if(&tX, kb * BK + (i & 1) * 32, y + (i >> 1) * 32, go);
+          }
       }
       if (p.tail)
         for (int i = 0; i < 2 * NKB; ++i) load(&tT, (i >> 1) * BK, (i & 1) * 128);
@@ -249,7 +282,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     // timed-out wait nothing else has waited for them)
     for (int i = ws < kRing ? 0 : ws - kRing; i < ws; ++i)
       mbar_wait_warp(w_full + i % kRing, (uint32_t)(i / kRing) & 1u, p.status);
-    if (tl > 0) mbar_wait_warp(a_full, (tl - 1) & 1, p.status);
+    if (tl > 0)
+      for (int kb = 0; kb < NKB; ++kb) mbar_wait_warp(a_full + kb, (tl - 1) & 1, p.status);
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
     const uint32_t go = elect_one();
@@ -275,18 +309,20 @@ __global__ void __launch_bounds__(kThreads, 1)
     };
     // [0, 256) = LN-free product of the A tile in sA with a 256 x 256 weight
     // (W_O or W_Q), box by box: k block kb, output half nh
-    auto mma_256 = [&]() {
+    // `full`: the k blocks' barriers where the tile may still be landing
+    auto mma_256 = [&](uint64_t* full, uint32_t fpar) {
       for (int i = 0; i < 2 * NKB; ++i) {
-        const uint32_t w = next_box();
         const int kb = i >> 1, nh = i & 1;
+        if (full && nh == 0) wait(full + kb, fpar);
+        const uint32_t w = next_box();
         mma_box(tmem + (uint32_t)(nh * 128), smem_u32(sA) + (uint32_t)(kb * 2) * kBox, w, idesc, kb != 0);
         release();
       }
     };
     for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++tl) {
-      // ---- A W_O into [0, 256)
-      wait(a_full, tl & 1);
-      mma_256();
+      // ---- A W_O into [0, 256) (the previous tile's tail product read)
+      if (p.tail && tl > 0) wait(q_read, (tl - 1) & 1);
+      mma_256(a_full, tl & 1);
       umma_commit_if(o_done, go);
       // ---- FFN1 chunk s one chunk ahead of FFN2 chunk s - 1
       wait(ln_full, tl & 1);
@@ -328,7 +364,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // ---- the tail LN(x_out) W_Q into [0, 256)
       if (p.tail) {
         wait(tail_a, tl & 1);
-        mma_256();
+        mma_256(nullptr, 0);
         umma_commit_if(tail_full, go);
       }
     }
@@ -345,6 +381,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     float* red_sum = red;        // [half][row]
     float* red_var = red + 256;  // [half][row]
     auto pair_sync = [&]() { asm volatile("bar.sync %0, 64;" ::"r"(1 + q) : "memory"); };
+    auto half_sync = [&]() { asm volatile("bar.sync %0, 128;" ::"r"(6 + hf) : "memory"); };
+    const bool lead = (et & 127) == 0;  // issues its half's stores
     auto epi_sync = [&]() { asm volatile("bar.sync 5, %0;" ::"n"(32 * kEpiWarps) : "memory"); };
     auto warp_arrive = [&](uint64_t* bar) {
       __syncwarp();
@@ -369,6 +407,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       float* xrow = p.x + (size_t)(m0 + r) * p.ldx;
       // ---- x0 into the accumulator while the projection runs (x0 of rows past
       // the valid count is 0)
+#pragma unroll 1
       for (int i = 0; i < 4; ++i) {
         const int c = c0 + 32 * i;
         float v[32];
@@ -391,6 +430,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       wait(o_done, tl & 1);
       tc_fence_after();
       float s4[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
       for (int i = 0; i < 4; ++i) {
         const int c = c0 + 32 * i;
         float v[32], w[32];
@@ -406,6 +446,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const float mean0 = pair_mean((s4[0] + s4[1]) + (s4[2] + s4[3]));
 #pragma unroll
       for (int k = 0; k < 4; ++k) s4[k] = 0.f;
+#pragma unroll 1
       for (int i = 0; i < 4; ++i) {
         float v[32];
         tmem_ld32(acc2 + lane_off + (uint32_t)(c0 + 32 * i), v);
@@ -416,6 +457,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
       const float rstd0 = pair_rstd((s4[0] + s4[1]) + (s4[2] + s4[3]));
+#pragma unroll 1
       for (int i = 0; i < 4; ++i) {
         const int c = c0 + 32 * i;
         float v[32];
@@ -433,6 +475,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int ba = gf & 1;
         wait(acc1_full + ba, (gf >> 1) & 1);
         tc_fence_after();
+#pragma unroll 1
         for (int jp = 0; jp < 2; ++jp) {
           const uint32_t col = tmem + lane_off + (uint32_t)(ba * FC + 64 * hf + 32 * jp);
           const float* bias = sB1 + f * FC + 64 * hf + 32 * jp;
@@ -459,6 +502,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       uint8_t* xst = sA + (size_t)ew * 16384u;
 #pragma unroll
       for (int k = 0; k < 4; ++k) s4[k] = 0.f;
+#pragma unroll 1
       for (int i = 0; i < 4; ++i) {
         const int c = c0 + 32 * i;
         float v[32];
@@ -488,51 +532,78 @@ __global__ void __launch_bounds__(kThreads, 1)
       const float mean = pair_mean((s4[0] + s4[1]) + (s4[2] + s4[3]));
 #pragma unroll
       for (int k = 0; k < 4; ++k) s4[k] = 0.f;
+#pragma unroll 1
       for (int i = 0; i < 4; ++i) {
         const int c = c0 + 32 * i;
         float v[32];
         tmem_ld32(acc2 + lane_off + (uint32_t)c, v);
 #pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          const float dv = v[j] + sB2[c + j] - mean;
-          s4[j & 3] = fmaf(dv, dv, s4[j & 3]);
+        for (int j = 0; j < 32; j += 4) {
+          const float4 bb = *reinterpret_cast<const float4*>(sB2 + c + j);
+          const float d0 = v[j] + bb.x - mean, d1 = v[j + 1] + bb.y - mean;
+          const float d2 = v[j + 2] + bb.z - mean, d3 = v[j + 3] + bb.w - mean;
+          s4[0] = fmaf(d0, d0, s4[0]);
+          s4[1] = fmaf(d1, d1, s4[1]);
+          s4[2] = fmaf(d2, d2, s4[2]);
+          s4[3] = fmaf(d3, d3, s4[3]);
         }
       }
       const float rstd = pair_rstd((s4[0] + s4[1]) + (s4[2] + s4[3]));
       if (lane == 0) bulk_wait_read0();
       epi_sync();  // every warp's x_out staging read: sA takes LN(x_out)
+#pragma unroll 1
       for (int i = 0; i < 4; ++i) {
         const int c = c0 + 32 * i;
         float v[32];
         tmem_ld32(acc2 + lane_off + (uint32_t)c, v);
 #pragma unroll
-        for (int j = 0; j < 32; ++j) v[j] = (v[j] + sB2[c + j] - mean) * rstd;
+        for (int j = 0; j < 32; j += 4) {
+          const float4 bb = *reinterpret_cast<const float4*>(sB2 + c + j);
+          v[j] = (v[j] + bb.x - mean) * rstd;
+          v[j + 1] = (v[j + 1] + bb.y - mean) * rstd;
+          v[j + 2] = (v[j + 2] + bb.z - mean) * rstd;
+          v[j + 3] = (v[j + 3] + bb.w - mean) * rstd;
+        }
         store_split_cols(sA, r, c, v);
-      }
-      fence_async_shared();
-      tc_fence_before();
-      if (p.tail) warp_arrive(tail_a);
-      if (p.store_ln) {
-        epi_sync();  // every row of the tile written
-        if (et == 0) {
-          for (int kb = 0; kb < NKB; ++kb) {
-            tma_store_2d(&tO_h, sA + (size_t)(kb * 2) * kBox, kb * BK, m0);
-            tma_store_2d(&tO_l, sA + (size_t)(kb * 2 + 1) * kBox, kb * BK, m0);
+        if (i & 1) {
+          fence_async_shared();
+          if (p.store_ln) {
+            half_sync();  // every row of k block c / 64 written
+            if (lead) {
+              const int kb = c >> 6;
+              tma_store_2d(&tO_h, sA + (size_t)(kb * 2) * kBox, kb * BK, m0);
+              tma_store_2d(&tO_l, sA + (size_t)(kb * 2 + 1) * kBox, kb * BK, m0);
+              bulk_commit();
+            }
+            __syncwarp();
           }
-          bulk_commit();
         }
       }
-      // ---- the tail: Q = LN(x_out) W_Q as f16 over sA (the tail product has read
-      // LN(x_out)): this thread's 128 columns of row r as 128-byte-swizzled
-      // [kb][128 rows x 64] tiles, stored by TMA
+      tc_fence_before();
       if (p.tail) {
+        // ---- the tail: Q = LN(x_out) W_Q as f16 over the upper half of sA (the
+        // tail product has read LN(x_out), whose stores have read it too): this
+        // thread's 128 columns of row r as 128-byte-swizzled [kb][128 rows x 64]
+        // tiles, stored by TMA
+        warp_arrive(tail_a);
         wait(tail_full, tl & 1);
         tc_fence_after();
+        if (p.store_ln) {
+          if (lead) bulk_wait_read0();
+          epi_sync();
+        }
+        if (et == 0) {
+          arrive_one(a_free);
+          arrive_one(a_free + 1);
+        }
+        __syncwarp();
+        uint8_t* sQ = sA + (size_t)4 * kBox;
+#pragma unroll 1
         for (int i = 0; i < 4; ++i) {
           const int c = c0 + 32 * i;
           float v[32];
           tmem_ld32(tmem + lane_off + (uint32_t)c, v);
-          uint8_t* rowp = sA + (size_t)(c >> 6) * kBox + (size_t)r * 128u;
+          uint8_t* rowp = sQ + (size_t)(c >> 6) * kBox + (size_t)r * 128u;
           const int u0 = (c & 63) >> 3;
 #pragma unroll
           for (int j = 0; j < 4; ++j)
@@ -541,20 +612,29 @@ __global__ void __launch_bounds__(kThreads, 1)
                            pack_f16x2(v[8 * j + 4], v[8 * j + 5]), pack_f16x2(v[8 * j + 6], v[8 * j + 7]));
         }
         tc_fence_before();
+        warp_arrive(q_read);
         fence_async_shared();
-        epi_sync();  // every row of Q written
-        if (et == 0) {
-          for (int kb = 0; kb < NKB; ++kb) tma_store_2d(&tQ, sA + (size_t)kb * kBox, kb * BK, m0);
+        half_sync();  // every row of this half's Q written
+        if (lead) {
+          for (int kb = 2 * hf; kb < 2 * hf + 2; ++kb) tma_store_2d(&tQ, sQ + (size_t)kb * kBox, kb * BK, m0);
           bulk_commit();
+          bulk_wait_read0();
+          arrive_one(a_free + 2 + hf);
+        }
+      } else {
+        // ---- a k block may take the next tile's A once its store has read it
+        // (the TMEM columns [0, 256) were last read before the FFN2 products)
+        if (!p.store_ln) half_sync();
+        if (lead) {
+          bulk_wait_read1();
+          arrive_one(a_free + 2 * hf);
+          bulk_wait_read0();
+          arrive_one(a_free + 2 * hf + 1);
         }
       }
-      // ---- sA and the TMEM columns [0, 256) may take the next tile once the
-      // stores have read sA
-      if (et == 0) bulk_wait_read0();
-      epi_sync();
-      warp_arrive(a_free);
+      __syncwarp();
     }
-    if (et == 0) bulk_wait0();  // output tensor stores complete before the CTA retires
+    if (lane == 0) bulk_wait0();  // output tensor stores complete before the CTA retires
   }
 
   __syncwarp();
