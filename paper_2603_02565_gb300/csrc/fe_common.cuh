@@ -536,6 +536,13 @@ __device__ __forceinline__ void tmem_st16_nowait(uint32_t taddr, const uint32_t*
       : "memory");
 }
 
+__device__ __forceinline__ void tmem_st16_nowait(uint32_t taddr, const float* v) {
+  uint32_t r[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) r[i] = __float_as_uint(v[i]);
+  tmem_st16_nowait(taddr, r);
+}
+
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 }  // namespace fe

@@ -31,7 +31,10 @@
 // MMA cost its issuing thread up to 92 cycles where the pipe takes 64, and a
 // satisfied wait 100 or more; with the warps run whole the batch of 256 requests went
 // from 163.8 to 159.1 us, one request from 124.9 to 119.5, 64 requests in fp32
-// from 148.4 to 141.0.
+// from 148.4 to 141.0.  Most launches give a CTA one tile or two, so the epilogue's
+// code is fetched cold: its loops over a row's pieces stay rolled, 16 columns a turn
+// up to the first LayerNorm (256 requests 153.8 -> 150.6 -> 149.1 us, 64 in fp32 137.8
+// -> 135.8).
 #include "fe_common.cuh"
 #include "fe_kernels.h"
 
@@ -411,7 +414,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       auto load_x0 = [&](int c, float* x) {
         const float* src = p.x0_row ? nullptr : p.x0 + (size_t)(m0 + r) * p.ldx0 + c;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int j = 0; j < 4; ++j) {
           float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
           if (p.x0_row)
             v = *reinterpret_cast<const float4*>(sX0 + c + 4 * j);
@@ -425,48 +428,50 @@ __global__ void __launch_bounds__(kThreads, 1)
       };
       // x0 into the accumulator (this warp's lanes and columns, read by this
       // warp in the previous tile's final phase) while the projection runs
-#pragma unroll
-      for (int ci = 0; ci < 2; ++ci) {
-        const int c = 32 * half + 64 * ci;
+#pragma unroll 1
+      for (int pi = 0; pi < 4; ++pi) {
+        const int c = 32 * half + 64 * (pi >> 1) + 16 * (pi & 1);
         if (c < d) {
-          float xr[32];
+          float xr[16];
           load_x0(c, xr);
-          tmem_st32(acc2 + lane_off + (uint32_t)c, xr);
+          tmem_st16_nowait(acc2 + lane_off + (uint32_t)c, xr);
         }
       }
+      tmem_st_wait();
       const uint32_t proj = tmem + (uint32_t)((gf % NA1) * FC);  // A W_O
       mbar_wait_warp(o_done, tl & 1, p.status);
       tc_fence_after();
       float s4[4] = {0.f, 0.f, 0.f, 0.f};  // four independent partial sums per statistic
-#pragma unroll
-      for (int ci = 0; ci < 2; ++ci) {
-        const int c = 32 * half + 64 * ci;
+#pragma unroll 1
+      for (int pi = 0; pi < 4; ++pi) {
+        const int c = 32 * half + 64 * (pi >> 1) + 16 * (pi & 1);
         if (c < d) {
-          float v[32], w[32];
-          tmem_ld32(proj + lane_off + (uint32_t)c, v);
-          tmem_ld32(acc2 + lane_off + (uint32_t)c, w);
+          float v[16], w[16];
+          tmem_ld16(proj + lane_off + (uint32_t)c, v);
+          tmem_ld16(acc2 + lane_off + (uint32_t)c, w);
 #pragma unroll
-          for (int j = 0; j < 32; ++j) {
+          for (int j = 0; j < 16; ++j) {
             v[j] += w[j];
             s4[j & 3] += v[j];
           }
-          tmem_st32(acc2 + lane_off + (uint32_t)c, v);
+          tmem_st16_nowait(acc2 + lane_off + (uint32_t)c, v);
         }
       }
+      tmem_st_wait();
       red_sum[half * 128 + r] = (s4[0] + s4[1]) + (s4[2] + s4[3]);
       pair_sync();
       const float mean0 = (red_sum[r] + red_sum[128 + r]) / (float)d;
       // x is read back from the accumulator rather than kept in registers
 #pragma unroll
       for (int i = 0; i < 4; ++i) s4[i] = 0.f;
-#pragma unroll
-      for (int ci = 0; ci < 2; ++ci) {
-        const int c = 32 * half + 64 * ci;
+#pragma unroll 1
+      for (int pi = 0; pi < 4; ++pi) {
+        const int c = 32 * half + 64 * (pi >> 1) + 16 * (pi & 1);
         if (c < d) {
-          float v[32];
-          tmem_ld32(acc2 + lane_off + (uint32_t)c, v);
+          float v[16];
+          tmem_ld16(acc2 + lane_off + (uint32_t)c, v);
 #pragma unroll
-          for (int j = 0; j < 32; ++j) {
+          for (int j = 0; j < 16; ++j) {
             const float dv = v[j] - mean0;
             s4[j & 3] = fmaf(dv, dv, s4[j & 3]);
           }
@@ -477,7 +482,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const float rstd0 = 1.0f / sqrtf((red_var[r] + red_var[128 + r]) / (float)d + p.eps);
       // row r of planes (kb, hi) and (kb, lo), 128-byte swizzle: this warp's
       // four 16-byte pieces 4 half + jj; columns past d are zeros
-#pragma unroll
+#pragma unroll 1
       for (int ci = 0; ci < nkb; ++ci) {
         const int c = 32 * half + 64 * ci;
         uint32_t hi[16], lo[16];
@@ -513,7 +518,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         tc_fence_after();
         // this warp's 64 columns as two 32-column pieces, each read whole and
         // then overwritten by its own hi (16 columns) and lo (16 columns) planes
-#pragma unroll
+#pragma unroll 1
         for (int hp = 0; hp < 2; ++hp) {
           const uint32_t col = tmem + lane_off + (uint32_t)(ba * FC + 64 * half + 32 * hp);
           const float* bias = sB1 + f * FC + 64 * half + 32 * hp;
@@ -543,7 +548,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // row chunk of 32 fp32 in a block: 16-byte piece j of row `lane`, 128-byte swizzle
       auto xoff = [&](int j) { return (uint32_t)lane * 128u + ((uint32_t)(j ^ (lane & 7)) << 4); };
       float sum2 = 0.f;
-#pragma unroll
+#pragma unroll 1
       for (int ci = 0; ci < 2; ++ci) {
         const int c = 32 * half + 64 * ci;
         if (c < d) {
@@ -562,7 +567,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         }
       }
-#pragma unroll
+#pragma unroll 1
       for (int ci = 0; ci < 2; ++ci) {
         const int c = 32 * half + 64 * ci;
         if (c < d) issue(&tO_x, blk(ci), nullptr, nullptr, c, srow);
@@ -571,7 +576,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       pair_sync();
       const float mean = (red_sum[r] + red_sum[128 + r]) / (float)d;
       float v4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
+#pragma unroll 1
       for (int ci = 0; ci < 2; ++ci) {
         if (32 * half + 64 * ci < d) {
 #pragma unroll
@@ -591,7 +596,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // LN(x_out) as the split tile [kb][plane] in sA, 128-byte swizzle (every
       // FFN1 has read the LN(x) tile there): row r, this warp's four 16-byte
       // pieces 4 half + jj of each plane; columns past d are zeros
-#pragma unroll
+#pragma unroll 1
       for (int ci = 0; ci < nkb; ++ci) {
         const int c = 32 * half + 64 * ci;
         uint32_t hi[16], lo[16];
