@@ -598,7 +598,7 @@ void clear_graphs(fe_ctx* c) {
 }
 
 int gemm(fe_ctx* c, const char* site, int epi, const Planes& A, const Weight& W, int rows, const int* rows_dev,
-         fe::GemmParams p, const Planes* out, const F32Rows* xout, cudaStream_t s) {
+         fe::GemmParams p, const Planes* out, const F32Rows* xout, cudaStream_t s, const F32Rows* resid = nullptr) {
   if (rows <= 0) return FE_OK;
   Prof pf(c, site, s);
   p.rows = rows;
@@ -612,6 +612,10 @@ int gemm(fe_ctx* c, const char* site, int epi, const Planes& A, const Weight& W,
   p.cs = 1;
   p.status = c->status;
   p.eps = c->cfg.ln_eps;
+  if (resid) {
+    p.resid = resid->p;
+    p.ldr = resid->ld;
+  }
   const CUtensorMap *bh = &W.p.th, *bl = &W.p.tl;
   // stored products with fewer 128-column tiles than half the SMs (the sequence
   // side of wide shapes): 64-column tiles, twice the CTAs
@@ -649,7 +653,7 @@ int gemm(fe_ctx* c, const char* site, int epi, const Planes& A, const Weight& W,
     }
   }
   FE_CK(fe::gemm_launch(epi, &A.th, &A.tl, bh, bl, out ? &out->sh : nullptr, out ? &out->sl : nullptr,
-                        xout ? &xout->sx : nullptr, p, s));
+                        xout ? &xout->sx : nullptr, resid ? &resid->sx : nullptr, p, s));
   return FE_OK;
 }
 
@@ -891,10 +895,8 @@ int enqueue_batch(fe_ctx* c, const Shape& sh, const IoPtrs& io, cudaStream_t s) 
       Prof pf(c, "attn_elem_self", s);
       FE_CK(fe::attn_launch(c->dh, &c->eqkv.ah, &c->eqkv.kh, &c->eqkv.kh, ap, s));
     }
-    fe::GemmParams po{};
-    po.resid = c->h.p;
-    po.ldr = d;
-    FE_RC(gemm(c, "gemm_elem_o_ln", fe::EPI_RESID_LN, c->a, c->oe, R, sumU, po, &c->xln, &c->h, s));
+    FE_RC(gemm(c, "gemm_elem_o_ln", fe::EPI_RESID_LN, c->a, c->oe, R, sumU, fe::GemmParams{}, &c->xln, &c->h, s,
+               &c->h));
   }
   if (fork) FE_CK(cudaStreamWaitEvent(s, c->kv_ev, 0));  // the context K/V (or states) are complete
   for (int l = 0; l < Ly; ++l) {
@@ -955,10 +957,8 @@ int enqueue_batch(fe_ctx* c, const Shape& sh, const IoPtrs& io, cudaStream_t s) 
       FE_RC(ffn256(c, "ffn_item", c->a, c->wo[l], c->w1[l], c->w2[l], lw(c, l, T_B1), lw(c, l, T_B2), nullptr, c->h,
                    c->xln, R, sumU, s, last ? 1 : 0, last ? nullptr : &c->wq[l + 1], last ? nullptr : &c->q));
     } else {
-      fe::GemmParams po{};
-      po.resid = c->h.p;
-      po.ldr = d;
-      FE_RC(gemm(c, "gemm_item_o_ln", fe::EPI_RESID_LN, c->a, c->wo[l], R, sumU, po, &c->xln, &c->h, s));
+      FE_RC(gemm(c, "gemm_item_o_ln", fe::EPI_RESID_LN, c->a, c->wo[l], R, sumU, fe::GemmParams{}, &c->xln, &c->h, s,
+                 &c->h));
 
       fe::GemmParams p1{};
       p1.bias = lw(c, l, T_B1);
@@ -967,9 +967,8 @@ int enqueue_batch(fe_ctx* c, const Shape& sh, const IoPtrs& io, cudaStream_t s) 
 
       fe::GemmParams p2{};
       p2.bias = lw(c, l, T_B2);
-      p2.resid = c->h.p;
-      p2.ldr = d;
-      FE_RC(gemm(c, "gemm_item_ffn2_ln", fe::EPI_RESID_LN, c->mid, c->w2[l], R, sumU, p2, &c->xln, &c->h, s));
+      FE_RC(gemm(c, "gemm_item_ffn2_ln", fe::EPI_RESID_LN, c->mid, c->w2[l], R, sumU, p2, &c->xln, &c->h, s,
+                 &c->h));
     }
   }
   // element projections of SeqEnc: H WKs | H WVs (unless the last fused FFN did them)
@@ -1071,9 +1070,8 @@ int enqueue_batch(fe_ctx* c, const Shape& sh, const IoPtrs& io, cudaStream_t s) 
     {
       fe::GemmParams p{};
       p.bias = tw(c, T_B2S);
-      p.resid = c->c.p;
-      p.ldr = d;
-      FE_RC(gemm(c, "gemm_seq_ffn2_ln", fe::EPI_RESID_LN, c->mids, c->w2s, S, nullptr, p, &c->z, &c->c, s));
+      FE_RC(gemm(c, "gemm_seq_ffn2_ln", fe::EPI_RESID_LN, c->mids, c->w2s, S, nullptr, p, &c->z, &c->c, s,
+                 &c->c));
     }
   }
   // (a5) cross-sequence attention over the K sequence vectors of each request
@@ -1108,10 +1106,8 @@ int enqueue_batch(fe_ctx* c, const Shape& sh, const IoPtrs& io, cudaStream_t s) 
       Prof pf(c, "attn_cross_seq", s);
       FE_CK(fe::attn_launch(c->dh, &c->qkv.ah, &c->qkv.kh, &vseg, ap, s));
     }
-    fe::GemmParams po{};
-    po.resid = c->c.p;
-    po.ldr = d;
-    FE_RC(gemm(c, "gemm_cross_o_ln", fe::EPI_RESID_LN, c->ax, c->ox, S, nullptr, po, &c->lncp, &c->cp, s));
+    FE_RC(gemm(c, "gemm_cross_o_ln", fe::EPI_RESID_LN, c->ax, c->ox, S, nullptr, fe::GemmParams{}, &c->lncp, &c->cp, s,
+               &c->c));
   }
   // (a6) score heads (task heads and their fusion) and selection
   {

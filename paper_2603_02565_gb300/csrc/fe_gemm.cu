@@ -17,6 +17,12 @@
 // MMAs of N >= 128 per 64-wide k step the issuing thread, not the tensor pipe, set
 // the pace (d = 512 summarisation batch 679 -> 631 us, 64 requests in fp32 140.9 ->
 // 137.7).
+// The residual rows of a LayerNorm tile arrive by TMA in the staging buffers that x
+// leaves from: a thread's own 16-byte loads, one row per lane, took a line of the L1
+// that 220 KB of shared memory leaves for every one of them.  Rows of more than 128
+// columns have their own instantiation.  Both together: 64 requests of 1000 candidates
+// 367.2 -> 362.3 us, the d = 512 summarisation batch 625.4 -> 621.4, d = 256 largest
+// batch 3870 -> 3855.
 // The activation is a split pair (hi + lo bf16); the product is
 // A_hi W_hi + A_lo W_hi (+ A_hi W_lo when the weights carry a lo plane).
 #include <cstdlib>
@@ -36,6 +42,7 @@ __device__ __forceinline__ float relu_nan(float x) {
 }
 
 namespace {
+constexpr int kResidWide = 4;  // EPI_RESID_LN for tiles of more than 128 columns
 constexpr int BM = 128;
 constexpr int BK = 64;                               // one 128-byte swizzle row of bf16
 constexpr uint32_t kATile = BM * BK * 2;             // 16 KB per activation plane
@@ -61,7 +68,7 @@ __host__ __device__ inline uint32_t red_bytes(int cs) { return cs > 1 ? (uint32_
 constexpr int kMaxCluster = 8;
 int g_cluster_cap[2][kMaxCluster + 1] = {};  // resident clusters of size cs with one / two CTAs per SM
 int g_cluster_limit = -1;                 // FE_GEMM_CLUSTERS: 0 disables clusters, n > 0 caps clusters per launch
-bool g_two_per_sm[4][2] = {};             // [EPI][NB - 1]: two CTAs fit on an SM (registers) at half the shared memory
+bool g_two_per_sm[5][2] = {};             // [EPI][NB - 1]: two CTAs fit on an SM (registers) at half the shared memory
 }  // namespace
 
 size_t gemm_smem_bytes(int BN, int nb, int stages, int cs, int na) {
@@ -135,7 +142,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     gemm_kernel(const __grid_constant__ CUtensorMap tA_h, const __grid_constant__ CUtensorMap tA_l,
                 const __grid_constant__ CUtensorMap tB_h, const __grid_constant__ CUtensorMap tB_l,
                 const __grid_constant__ CUtensorMap tO_h, const __grid_constant__ CUtensorMap tO_l,
-                const __grid_constant__ CUtensorMap tO_x, const GemmParams p) {
+                const __grid_constant__ CUtensorMap tO_x, const __grid_constant__ CUtensorMap tR, const GemmParams p) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw_s = smem_u32(smem_raw);
   uint8_t* smem = smem_raw + ((1024u - (raw_s & 1023u)) & 1023u);
@@ -155,6 +162,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* xbar = tempty + 2;  // [2] cluster row exchange: partial sums / partial variances received
   uint64_t* drain = xbar + 2;   // the products in flight at the end
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(xbar + 3);
+  uint64_t* rbar = xbar + 4;    // [kEpiWarps] EPI_RESID_LN: the warp's residual blocks landed (the 256 bytes end here)
   // output staging: two 4 KB buffers per epilogue warp, 1024-byte aligned; then
   // the row-reduction exchange of the two warps sharing a lane quadrant
   uint8_t* stg_base = smem + (((size_t)S * stage_bytes + 256 + 1023) & ~(size_t)1023);
@@ -174,6 +182,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(tempty + a, kEpiWarps);  // one arrival per epilogue warp
     }
     mbar_init(drain, 1);
+    if (EPI == EPI_RESID_LN)
+      for (int i = 0; i < kEpiWarps; ++i) mbar_init(rbar + i, 1);
     if (cs > 1) {
       mbar_init(xbar, 1);  // the local expect_tx; the peers' stores complete the bytes
       mbar_init(xbar + 1, 1);
@@ -347,26 +357,20 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int m0 = (t / nt) * BM, n0 = (t % nt) * BN;
       const int grow = m0 + r;
       const bool valid = grow < rows_valid;
-      if (EPI == EPI_RESID_LN && BN <= 128) {
-        // residual rows, loaded while the MMAs of this tile run
-        const float* rrow = p.resid + (p.ldr ? (size_t)grow * p.ldr : (size_t)0);
-#pragma unroll
-        for (int ci = 0; ci < 2; ++ci) {
-          const int c = 32 * half + 64 * ci;
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            float4 qv = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (valid && c < BN) qv = reinterpret_cast<const float4*>(rrow + n0 + c)[j];
-            xr[32 * ci + 4 * j] = qv.x;
-            xr[32 * ci + 4 * j + 1] = qv.y;
-            xr[32 * ci + 4 * j + 2] = qv.z;
-            xr[32 * ci + 4 * j + 3] = qv.w;
-          }
+      const int srow = m0 + q * 32;
+      if (EPI == EPI_RESID_LN && p.ldr) {
+        // residual rows, loaded while the MMAs of this tile run: this warp's blocks (at most
+        // two) into its staging buffers, whose last stores have read them
+        if (lane == 0) {
+          bulk_wait_read0();
+          mbar_arrive_expect_tx(rbar + ew, (uint32_t)((BN - 32 * half + 63) / 64) * kStageOut);
+          for (int ci = 0, c = 32 * half; c < BN; ++ci, c += 64)
+            tma_load_2d(stg0 + (size_t)ci * kStageOut, &tR, n0 + c, srow, rbar + ew);
         }
+        __syncwarp();
       }
       mbar_wait_warp(tfull + acc, use & 1, p.status);
       tc_fence_after();
-      const int srow = m0 + q * 32;
       const uint32_t trow = tmem + (uint32_t)(acc * BN) + ((uint32_t)(q * 32) << 16);
       float* red_sum = red + (size_t)(tl & 1) * 512;  // [half][128]
       float* red_var = red_sum + 256;
@@ -424,10 +428,13 @@ __global__ void __launch_bounds__(kThreads, 1)
             stage_split(hi, lo, col, srow);
           }
         }
-      } else if (EPI == EPI_RESID_LN && BN <= 128) {
+      } else if (EPI == EPI_RESID_LN) {
         // rows of at most 128 columns: each warp holds its (at most two) chunks of
         // x = resid + acc + bias in registers; the residual was loaded before the
         // accumulator was ready, TMEM is read once
+        // (one row broadcast to every row is read where it lies)
+        if (p.ldr) mbar_wait_warp(rbar + ew, (uint32_t)tl & 1u, p.status);
+        const int sw = p.ldr ? lane & 7 : 0;
         float sum = 0.f;
 #pragma unroll
         for (int ci = 0; ci < 2; ++ci) {
@@ -436,7 +443,16 @@ __global__ void __launch_bounds__(kThreads, 1)
             float v[32];
             tmem_ld32(trow + (uint32_t)c, v);
 #pragma unroll
-            for (int i = 0; i < 32; ++i) xr[32 * ci + i] += v[i];
+            for (int j = 0; j < 8; ++j) {
+              const float* src = p.ldr ? reinterpret_cast<const float*>(stg0 + (size_t)ci * kStageOut) + lane * 32
+                                       : p.resid + n0 + c;
+              float4 qv = make_float4(0.f, 0.f, 0.f, 0.f);  // (rows past the valid count)
+              if (valid) qv = *reinterpret_cast<const float4*>(src + 4 * (j ^ sw));
+              xr[32 * ci + 4 * j] = qv.x + v[4 * j];
+              xr[32 * ci + 4 * j + 1] = qv.y + v[4 * j + 1];
+              xr[32 * ci + 4 * j + 2] = qv.z + v[4 * j + 2];
+              xr[32 * ci + 4 * j + 3] = qv.w + v[4 * j + 3];
+            }
             if (p.bias) {
               const float4* b4 = reinterpret_cast<const float4*>(p.bias + n0 + c);
 #pragma unroll
@@ -501,7 +517,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             stage_split(hi, lo, n0 + c, srow);
           }
         }
-      } else if (EPI == EPI_RESID_LN) {
+      } else if (EPI == kResidWide) {
         // wider rows: x kept in TMEM between the passes
         float sum = 0.f;
         const float* rrow = p.resid + (p.ldr ? (size_t)grow * p.ldr : (size_t)0);
@@ -671,7 +687,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 template <int EPI, int NB>
 static cudaError_t launch_t(const CUtensorMap* a_h, const CUtensorMap* a_l, const CUtensorMap* b_h,
                             const CUtensorMap* b_l, const CUtensorMap* o_h, const CUtensorMap* o_l,
-                            const CUtensorMap* o_x, const GemmParams& p0, cudaStream_t s) {
+                            const CUtensorMap* o_x, const CUtensorMap* r_x, const GemmParams& p0, cudaStream_t s) {
   GemmParams p = p0;
   const int cs = ((EPI == EPI_RESID_LN || EPI == EPI_HEAD) && p.cs > 1) ? p.cs : 1;
   p.cs = cs;
@@ -709,12 +725,12 @@ static cudaError_t launch_t(const CUtensorMap* a_h, const CUtensorMap* a_l, cons
     long long grid = nclu * cs;
     if (grid > tiles) grid = tiles;
     return launch_kc(gemm_kernel<EPI, NB>, dim3((unsigned)grid), dim3(kThreads), smem, s, cs, *a_h, *a_l, *b_h,
-                     *b_l, o_h ? *o_h : *a_h, o_l ? *o_l : *a_l, o_x ? *o_x : *a_h, p);
+                     *b_l, o_h ? *o_h : *a_h, o_l ? *o_l : *a_l, o_x ? *o_x : *a_h, r_x ? *r_x : *a_h, p);
   }
   long long grid = (long long)sms * per_sm;
   if (grid > tiles) grid = tiles;
   return launch_k(gemm_kernel<EPI, NB>, dim3((unsigned)grid), dim3(kThreads), smem, s, *a_h, *a_l, *b_h, *b_l,
-                  o_h ? *o_h : *a_h, o_l ? *o_l : *a_l, o_x ? *o_x : *a_h, p);
+                  o_h ? *o_h : *a_h, o_l ? *o_l : *a_l, o_x ? *o_x : *a_h, r_x ? *r_x : *a_h, p);
 }
 
 cudaError_t gemm_prepare() {
@@ -727,7 +743,9 @@ cudaError_t gemm_prepare() {
   attr((const void*)gemm_kernel<EPI_STORE, 1>);
   attr((const void*)gemm_kernel<EPI_STORE, 2>);
   attr((const void*)gemm_kernel<EPI_RESID_LN, 1>);
+  attr((const void*)gemm_kernel<kResidWide, 1>);
   attr((const void*)gemm_kernel<EPI_RESID_LN, 2>);
+  attr((const void*)gemm_kernel<kResidWide, 2>);
   attr((const void*)gemm_kernel<EPI_HEAD, 1>);
   attr((const void*)gemm_kernel<EPI_HEAD, 2>);
   attr((const void*)gemm_kernel<EPI_LN_FOLD, 1>);
@@ -740,7 +758,9 @@ cudaError_t gemm_prepare() {
   g_two_per_sm[EPI_STORE][0] = two_fit((const void*)gemm_kernel<EPI_STORE, 1>);
   g_two_per_sm[EPI_STORE][1] = two_fit((const void*)gemm_kernel<EPI_STORE, 2>);
   g_two_per_sm[EPI_RESID_LN][0] = two_fit((const void*)gemm_kernel<EPI_RESID_LN, 1>);
+  g_two_per_sm[kResidWide][0] = two_fit((const void*)gemm_kernel<kResidWide, 1>);
   g_two_per_sm[EPI_RESID_LN][1] = two_fit((const void*)gemm_kernel<EPI_RESID_LN, 2>);
+  g_two_per_sm[kResidWide][1] = two_fit((const void*)gemm_kernel<kResidWide, 2>);
   g_two_per_sm[EPI_HEAD][0] = two_fit((const void*)gemm_kernel<EPI_HEAD, 1>);
   g_two_per_sm[EPI_HEAD][1] = two_fit((const void*)gemm_kernel<EPI_HEAD, 2>);
   g_two_per_sm[EPI_LN_FOLD][0] = two_fit((const void*)gemm_kernel<EPI_LN_FOLD, 1>);
@@ -789,22 +809,26 @@ int gemm_cluster_capacity(int cs) {
 
 cudaError_t gemm_launch(int epi, const CUtensorMap* a_h, const CUtensorMap* a_l, const CUtensorMap* b_h,
                         const CUtensorMap* b_l, const CUtensorMap* o_h, const CUtensorMap* o_l,
-                        const CUtensorMap* o_x, const GemmParams& p, cudaStream_t s) {
+                        const CUtensorMap* o_x, const CUtensorMap* r_x, const GemmParams& p, cudaStream_t s) {
   if (p.rows <= 0) return cudaSuccess;
+  if (epi == EPI_RESID_LN && p.ldr && !r_x) return cudaErrorInvalidValue;
   const bool two = p.nb > 1;
   switch (epi) {
     case EPI_STORE:
-      return two ? launch_t<EPI_STORE, 2>(a_h, a_l, b_h, b_l, o_h, o_l, o_x, p, s)
-                 : launch_t<EPI_STORE, 1>(a_h, a_l, b_h, b_l, o_h, o_l, o_x, p, s);
+      return two ? launch_t<EPI_STORE, 2>(a_h, a_l, b_h, b_l, o_h, o_l, o_x, r_x, p, s)
+                 : launch_t<EPI_STORE, 1>(a_h, a_l, b_h, b_l, o_h, o_l, o_x, r_x, p, s);
     case EPI_RESID_LN:
-      return two ? launch_t<EPI_RESID_LN, 2>(a_h, a_l, b_h, b_l, o_h, o_l, o_x, p, s)
-                 : launch_t<EPI_RESID_LN, 1>(a_h, a_l, b_h, b_l, o_h, o_l, o_x, p, s);
+      if (p.BN > 128)
+        return two ? launch_t<kResidWide, 2>(a_h, a_l, b_h, b_l, o_h, o_l, o_x, r_x, p, s)
+                   : launch_t<kResidWide, 1>(a_h, a_l, b_h, b_l, o_h, o_l, o_x, r_x, p, s);
+      return two ? launch_t<EPI_RESID_LN, 2>(a_h, a_l, b_h, b_l, o_h, o_l, o_x, r_x, p, s)
+                 : launch_t<EPI_RESID_LN, 1>(a_h, a_l, b_h, b_l, o_h, o_l, o_x, r_x, p, s);
     case EPI_LN_FOLD:
-      return two ? launch_t<EPI_LN_FOLD, 2>(a_h, a_l, b_h, b_l, o_h, o_l, o_x, p, s)
-                 : launch_t<EPI_LN_FOLD, 1>(a_h, a_l, b_h, b_l, o_h, o_l, o_x, p, s);
+      return two ? launch_t<EPI_LN_FOLD, 2>(a_h, a_l, b_h, b_l, o_h, o_l, o_x, r_x, p, s)
+                 : launch_t<EPI_LN_FOLD, 1>(a_h, a_l, b_h, b_l, o_h, o_l, o_x, r_x, p, s);
     default:
-      return two ? launch_t<EPI_HEAD, 2>(a_h, a_l, b_h, b_l, o_h, o_l, o_x, p, s)
-                 : launch_t<EPI_HEAD, 1>(a_h, a_l, b_h, b_l, o_h, o_l, o_x, p, s);
+      return two ? launch_t<EPI_HEAD, 2>(a_h, a_l, b_h, b_l, o_h, o_l, o_x, r_x, p, s)
+                 : launch_t<EPI_HEAD, 1>(a_h, a_l, b_h, b_l, o_h, o_l, o_x, r_x, p, s);
   }
 }
 

@@ -137,10 +137,11 @@ int gemm_max_stages(int BN, int nb, int K_pad, int cs = 1, int na = 2);
 int gemm_cluster_capacity(int cs);
 // o_h / o_l: output bf16 planes (EPI_STORE: the product, EPI_RESID_LN: LN(x)), tensor maps with
 // 32 x 32 boxes and the 64-byte swizzle; o_x: the fp32 x_out rows of EPI_RESID_LN, 32 x 32 boxes,
-// 128-byte swizzle.  Unused maps may be null.
+// 128-byte swizzle; r_x: the residual rows of EPI_RESID_LN (ldr != 0), mapped like o_x.  Unused maps
+// may be null.
 cudaError_t gemm_launch(int epi, const CUtensorMap* a_h, const CUtensorMap* a_l, const CUtensorMap* b_h,
                         const CUtensorMap* b_l, const CUtensorMap* o_h, const CUtensorMap* o_l,
-                        const CUtensorMap* o_x, const GemmParams& p, cudaStream_t s);
+                        const CUtensorMap* o_x, const CUtensorMap* r_x, const GemmParams& p, cudaStream_t s);
 
 // ---------------------------------------------------------------------------
 // Attention output projection + FFN block for rows of width d <= 128 (fe_ffn.cu):
