@@ -425,6 +425,16 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// 32 bytes per thread, for a row per lane: each load takes a whole sector.  (16-byte
+// loads take every sector in two halves, and between them a line per lane of the
+// L1 that a kernel with 200 KB of shared memory leaves.)
+__device__ __forceinline__ void ld_sector(const float* p, float* x) {
+  asm volatile("ld.global.L1::no_allocate.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]), "=f"(x[4]), "=f"(x[5]), "=f"(x[6]), "=f"(x[7])
+               : "l"(p)
+               : "memory");
+}
+
 // 32 lanes x 64 columns -> 64 registers per thread, one load and one wait
 __device__ __forceinline__ void tmem_ld64(uint32_t taddr, float* v) {
   uint32_t r[64];

@@ -25,7 +25,9 @@
 // The MMA groups are 16 instructions of N >= 128 so that the tensor pipe has
 // queued work while the issuing warp polls its barriers; x0 is read by the
 // epilogue warps while the A tile is in flight, when they have nothing else to
-// do; the biases sit in shared memory.
+// do, a 32-byte sector a load (16 bytes a load took 256 requests 149.3 us in all
+// instead of 147.3, ragged ones 98.5 instead of 97.5; all of a row's loads at once
+// 153.7 and 102.2); the biases sit in shared memory.
 // What bounds it: a tile is one dependency chain of which the tensor pipe needs
 // 5 us (160 MMAs of N = 128 at d = 128, F = 512).  Behind `if (lane == 0)` an
 // MMA cost its issuing thread up to 92 cycles where the pipe takes 64, and a
@@ -414,16 +416,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       auto load_x0 = [&](int c, float* x) {
         const float* src = p.x0_row ? nullptr : p.x0 + (size_t)(m0 + r) * p.ldx0 + c;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (p.x0_row)
-            v = *reinterpret_cast<const float4*>(sX0 + c + 4 * j);
-          else if (valid)
-            v = *reinterpret_cast<const float4*>(src + 4 * j);
-          x[4 * j] = v.x;
-          x[4 * j + 1] = v.y;
-          x[4 * j + 2] = v.z;
-          x[4 * j + 3] = v.w;
+        for (int j = 0; j < 16; j += 8) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) x[j + i] = p.x0_row ? sX0[c + j + i] : 0.f;
+          if (!p.x0_row && valid) ld_sector(src + j, x + j);
         }
       };
       // x0 into the accumulator (this warp's lanes and columns, read by this
@@ -741,7 +737,7 @@ cudaError_t ffn_launch(const CUtensorMap* a_h, const CUtensorMap* a_l, const CUt
                        const CUtensorMap* t_l, const CUtensorMap* to_h, const CUtensorMap* to_l,
                        const FfnParams& p, cudaStream_t s) {
   if (p.rows <= 0) return cudaSuccess;
-  if (!p.x0_row && (!p.x0 || p.ldx0 < p.d || p.ldx0 % 4)) return cudaErrorInvalidValue;
+  if (!p.x0_row && (!p.x0 || p.ldx0 < p.d || p.ldx0 % 8 || (uintptr_t)p.x0 % 32)) return cudaErrorInvalidValue;
   if (p.tail_n > 0 && (!t_h || !to_h || (!p.tail_f16 && !to_l) ||
                        !ffn_tail_supported(p.d, p.d_pad, p.F, p.nb, p.tail_n, p.tail_f16)))
     return cudaErrorInvalidValue;

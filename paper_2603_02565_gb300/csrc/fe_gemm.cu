@@ -20,7 +20,8 @@
 // The residual rows of a LayerNorm tile arrive by TMA in the staging buffers that x
 // leaves from: a thread's own 16-byte loads, one row per lane, took a line of the L1
 // that 220 KB of shared memory leaves for every one of them.  Rows of more than 128
-// columns have their own instantiation.  Both together: 64 requests of 1000 candidates
+// columns have their own instantiation, whose threads load 32-byte sectors (largest
+// batch 3825 -> 3818).  Both together: 64 requests of 1000 candidates
 // 367.2 -> 362.3 us, the d = 512 summarisation batch 625.4 -> 621.4, d = 256 largest
 // batch 3870 -> 3855.
 // The activation is a split pair (hi + lo bf16); the product is
@@ -525,15 +526,11 @@ __global__ void __launch_bounds__(kThreads, 1)
           float v[32];
           tmem_ld32(trow + (uint32_t)c, v);
           if (valid) {
-            const float4* rr = reinterpret_cast<const float4*>(rrow + c);
+            float x[32];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              const float4 qv = rr[j];
-              v[4 * j + 0] += qv.x;
-              v[4 * j + 1] += qv.y;
-              v[4 * j + 2] += qv.z;
-              v[4 * j + 3] += qv.w;
-            }
+            for (int j = 0; j < 32; j += 8) ld_sector(rrow + c + j, x + j);
+#pragma unroll
+            for (int i = 0; i < 32; ++i) v[i] += x[i];
           }
           if (p.bias) {
 #pragma unroll
@@ -811,7 +808,7 @@ cudaError_t gemm_launch(int epi, const CUtensorMap* a_h, const CUtensorMap* a_l,
                         const CUtensorMap* b_l, const CUtensorMap* o_h, const CUtensorMap* o_l,
                         const CUtensorMap* o_x, const CUtensorMap* r_x, const GemmParams& p, cudaStream_t s) {
   if (p.rows <= 0) return cudaSuccess;
-  if (epi == EPI_RESID_LN && p.ldr && !r_x) return cudaErrorInvalidValue;
+  if (epi == EPI_RESID_LN && (p.ldr % 8 || (uintptr_t)p.resid % 32 || (p.ldr && !r_x))) return cudaErrorInvalidValue;
   const bool two = p.nb > 1;
   switch (epi) {
     case EPI_STORE:

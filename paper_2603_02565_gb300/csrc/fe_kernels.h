@@ -162,8 +162,8 @@ struct FfnParams {
   int d, d_pad, F, nb;
   const float* b1;      // [F]
   const float* b2;      // [d]
-  const float* x0;      // block input rows, unless x0_row is set
-  int ldx0;             // multiple of 4
+  const float* x0;      // block input rows (32-byte aligned), unless x0_row is set
+  int ldx0;             // multiple of 8
   const float* x0_row;  // [d], when set: the same input row for every row
   int tail_n;           // 0: no tail product
   int tail_f16;         // tail output as one f16 plane (else a split pair)
