@@ -34,9 +34,8 @@
 // satisfied wait 100 or more; with the warps run whole the batch of 256 requests went
 // from 163.8 to 159.1 us, one request from 124.9 to 119.5, 64 requests in fp32
 // from 148.4 to 141.0.  Most launches give a CTA one tile or two, so the epilogue's
-// code is fetched cold: its loops over a row's pieces stay rolled, 16 columns a turn
-// up to the first LayerNorm (256 requests 153.8 -> 150.6 -> 149.1 us, 64 in fp32 137.8
-// -> 135.8).
+// code is fetched cold: its loops over a row's pieces stay rolled (256 requests 153.8 -> 150.6
+// us, 64 in fp32 137.8 -> 136.3).
 #include "fe_common.cuh"
 #include "fe_kernels.h"
 
@@ -437,43 +436,35 @@ __global__ void __launch_bounds__(kThreads, 1)
       const uint32_t proj = tmem + (uint32_t)((gf % NA1) * FC);  // A W_O
       mbar_wait_warp(o_done, tl & 1, p.status);
       tc_fence_after();
-      float s4[4] = {0.f, 0.f, 0.f, 0.f};  // four independent partial sums per statistic
+      RowSum sum, var;
 #pragma unroll 1
-      for (int pi = 0; pi < 4; ++pi) {
-        const int c = 32 * half + 64 * (pi >> 1) + 16 * (pi & 1);
+      for (int ci = 0; ci < 2; ++ci) {
+        const int c = 32 * half + 64 * ci;
         if (c < d) {
-          float v[16], w[16];
-          tmem_ld16(proj + lane_off + (uint32_t)c, v);
-          tmem_ld16(acc2 + lane_off + (uint32_t)c, w);
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            v[j] += w[j];
-            s4[j & 3] += v[j];
-          }
+          float v[32], w[32];
+          tmem_ld32(proj + lane_off + (uint32_t)c, v);
+          tmem_ld32(acc2 + lane_off + (uint32_t)c, w);
+          row_plus<32>(v, w);
+          row_add<32>(sum, v);
           tmem_st16_nowait(acc2 + lane_off + (uint32_t)c, v);
+          tmem_st16_nowait(acc2 + lane_off + (uint32_t)c + 16u, v + 16);
         }
       }
       tmem_st_wait();
-      red_sum[half * 128 + r] = (s4[0] + s4[1]) + (s4[2] + s4[3]);
+      red_sum[half * 128 + r] = sum.total();
       pair_sync();
       const float mean0 = (red_sum[r] + red_sum[128 + r]) / (float)d;
       // x is read back from the accumulator rather than kept in registers
-#pragma unroll
-      for (int i = 0; i < 4; ++i) s4[i] = 0.f;
 #pragma unroll 1
-      for (int pi = 0; pi < 4; ++pi) {
-        const int c = 32 * half + 64 * (pi >> 1) + 16 * (pi & 1);
+      for (int ci = 0; ci < 2; ++ci) {
+        const int c = 32 * half + 64 * ci;
         if (c < d) {
-          float v[16];
-          tmem_ld16(acc2 + lane_off + (uint32_t)c, v);
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const float dv = v[j] - mean0;
-            s4[j & 3] = fmaf(dv, dv, s4[j & 3]);
-          }
+          float v[32];
+          tmem_ld32(acc2 + lane_off + (uint32_t)c, v);
+          row_add_sq<32>(var, v, mean0);
         }
       }
-      red_var[half * 128 + r] = (s4[0] + s4[1]) + (s4[2] + s4[3]);
+      red_var[half * 128 + r] = var.total();
       pair_sync();
       const float rstd0 = 1.0f / sqrtf((red_var[r] + red_var[128 + r]) / (float)d + p.eps);
       // row r of planes (kb, hi) and (kb, lo), 128-byte swizzle: this warp's
@@ -485,8 +476,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (c < d) {
           float v[32];
           tmem_ld32(acc2 + lane_off + (uint32_t)c, v);
+          row_norm<32>(v, mean0, rstd0);
 #pragma unroll
-          for (int j = 0; j < 16; ++j) split2((v[2 * j] - mean0) * rstd0, (v[2 * j + 1] - mean0) * rstd0, hi[j], lo[j]);
+          for (int j = 0; j < 16; ++j) split2(v[2 * j], v[2 * j + 1], hi[j], lo[j]);
         } else {
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
@@ -524,7 +516,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
             const float2 bb = *reinterpret_cast<const float2*>(bias + 2 * j);
-            split2_trunc(relu_nan(v[2 * j] + bb.x), relu_nan(v[2 * j + 1] + bb.y), hi[j], lo[j]);
+            const float b2[2] = {bb.x, bb.y};
+            row_plus<2>(v + 2 * j, b2);
+            split2_trunc(relu_nan(v[2 * j]), relu_nan(v[2 * j + 1]), hi[j], lo[j]);
           }
           tmem_st16_nowait(col, hi);
           tmem_st16_nowait(col + 16, lo);
@@ -571,22 +565,19 @@ __global__ void __launch_bounds__(kThreads, 1)
       red_sum[half * 128 + r] = sum2;
       pair_sync();
       const float mean = (red_sum[r] + red_sum[128 + r]) / (float)d;
-      float v4[4] = {0.f, 0.f, 0.f, 0.f};
+      RowSum var2;
 #pragma unroll 1
       for (int ci = 0; ci < 2; ++ci) {
         if (32 * half + 64 * ci < d) {
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
             const float4 x = *reinterpret_cast<const float4*>(blk(ci) + xoff(j));
-            const float d0 = x.x - mean, d1 = x.y - mean, d2 = x.z - mean, d3 = x.w - mean;
-            v4[0] = fmaf(d0, d0, v4[0]);
-            v4[1] = fmaf(d1, d1, v4[1]);
-            v4[2] = fmaf(d2, d2, v4[2]);
-            v4[3] = fmaf(d3, d3, v4[3]);
+            const float x4[4] = {x.x, x.y, x.z, x.w};
+            row_add_sq<4>(var2, x4, mean);
           }
         }
       }
-      red_var[half * 128 + r] = (v4[0] + v4[1]) + (v4[2] + v4[3]);
+      red_var[half * 128 + r] = var2.total();
       pair_sync();
       const float rstd = 1.0f / sqrtf((red_var[r] + red_var[128 + r]) / (float)d + p.eps);
       // LN(x_out) as the split tile [kb][plane] in sA, 128-byte swizzle (every
@@ -600,8 +591,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
             const float4 x = *reinterpret_cast<const float4*>(blk(ci) + xoff(j));
-            split2((x.x - mean) * rstd, (x.y - mean) * rstd, hi[2 * j], lo[2 * j]);
-            split2((x.z - mean) * rstd, (x.w - mean) * rstd, hi[2 * j + 1], lo[2 * j + 1]);
+            float x4[4] = {x.x, x.y, x.z, x.w};
+            row_norm<4>(x4, mean, rstd);
+            split2(x4[0], x4[1], hi[2 * j], lo[2 * j]);
+            split2(x4[2], x4[3], hi[2 * j + 1], lo[2 * j + 1]);
           }
         } else {
 #pragma unroll

@@ -424,41 +424,31 @@ __global__ void __launch_bounds__(kThreads, 1)
       // (the projection, the tile's only reader, is complete)
       wait(o_done, tl & 1);
       tc_fence_after();
-      float s4[4] = {0.f, 0.f, 0.f, 0.f};
+      RowSum sum0, var0;
 #pragma unroll 1
       for (int i = 0; i < 4; ++i) {
         const int c = c0 + 32 * i;
         float v[32], w[32];
         tmem_ld32(tmem + lane_off + (uint32_t)c, v);
         tmem_ld32(acc2 + lane_off + (uint32_t)c, w);
-#pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          v[j] += w[j];
-          s4[j & 3] += v[j];
-        }
+        row_plus<32>(v, w);
+        row_add<32>(sum0, v);
         tmem_st32(acc2 + lane_off + (uint32_t)c, v);
       }
-      const float mean0 = pair_mean((s4[0] + s4[1]) + (s4[2] + s4[3]));
-#pragma unroll
-      for (int k = 0; k < 4; ++k) s4[k] = 0.f;
+      const float mean0 = pair_mean(sum0.total());
 #pragma unroll 1
       for (int i = 0; i < 4; ++i) {
         float v[32];
         tmem_ld32(acc2 + lane_off + (uint32_t)(c0 + 32 * i), v);
-#pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          const float dv = v[j] - mean0;
-          s4[j & 3] = fmaf(dv, dv, s4[j & 3]);
-        }
+        row_add_sq<32>(var0, v, mean0);
       }
-      const float rstd0 = pair_rstd((s4[0] + s4[1]) + (s4[2] + s4[3]));
+      const float rstd0 = pair_rstd(var0.total());
 #pragma unroll 1
       for (int i = 0; i < 4; ++i) {
         const int c = c0 + 32 * i;
         float v[32];
         tmem_ld32(acc2 + lane_off + (uint32_t)c, v);
-#pragma unroll
-        for (int j = 0; j < 32; ++j) v[j] = (v[j] - mean0) * rstd0;
+        row_norm<32>(v, mean0, rstd0);
         store_split_cols(sA, r, c, v);
       }
       fence_async_shared();
@@ -480,7 +470,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
             const float2 bb = *reinterpret_cast<const float2*>(bias + 2 * j);
-            split2_trunc(relu_nan256(v[2 * j] + bb.x), relu_nan256(v[2 * j + 1] + bb.y), hi[j], lo[j]);
+            const float b2[2] = {bb.x, bb.y};
+            row_plus<2>(v + 2 * j, b2);
+            split2_trunc(relu_nan256(v[2 * j]), relu_nan256(v[2 * j + 1]), hi[j], lo[j]);
           }
           tmem_st16_nowait(col, hi);
           tmem_st16_nowait(col + 16u, lo);
@@ -495,8 +487,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       wait(acc2_full, tl & 1);
       tc_fence_after();
       uint8_t* xst = sA + (size_t)ew * 16384u;
-#pragma unroll
-      for (int k = 0; k < 4; ++k) s4[k] = 0.f;
+      RowSum sum, var;
 #pragma unroll 1
       for (int i = 0; i < 4; ++i) {
         const int c = c0 + 32 * i;
@@ -506,14 +497,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int j = 0; j < 32; j += 4) {
           const float4 bb = *reinterpret_cast<const float4*>(sB2 + c + j);
-          v[j] += bb.x;
-          v[j + 1] += bb.y;
-          v[j + 2] += bb.z;
-          v[j + 3] += bb.w;
-          s4[0] += v[j];
-          s4[1] += v[j + 1];
-          s4[2] += v[j + 2];
-          s4[3] += v[j + 3];
+          const float b4[4] = {bb.x, bb.y, bb.z, bb.w};
+          row_plus<4>(v + j, b4);
+          row_add<4>(sum, v + j);
           *reinterpret_cast<float4*>(blk + ((uint32_t)((j >> 2) ^ (lane & 7)) << 4)) =
               make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
         }
@@ -524,9 +510,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int i = 0; i < 4; ++i) tma_store_2d(&tX, xst + (size_t)i * 4096u, c0 + 32 * i, m0 + 32 * q);
         bulk_commit();
       }
-      const float mean = pair_mean((s4[0] + s4[1]) + (s4[2] + s4[3]));
-#pragma unroll
-      for (int k = 0; k < 4; ++k) s4[k] = 0.f;
+      const float mean = pair_mean(sum.total());
 #pragma unroll 1
       for (int i = 0; i < 4; ++i) {
         const int c = c0 + 32 * i;
@@ -535,15 +519,12 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int j = 0; j < 32; j += 4) {
           const float4 bb = *reinterpret_cast<const float4*>(sB2 + c + j);
-          const float d0 = v[j] + bb.x - mean, d1 = v[j + 1] + bb.y - mean;
-          const float d2 = v[j + 2] + bb.z - mean, d3 = v[j + 3] + bb.w - mean;
-          s4[0] = fmaf(d0, d0, s4[0]);
-          s4[1] = fmaf(d1, d1, s4[1]);
-          s4[2] = fmaf(d2, d2, s4[2]);
-          s4[3] = fmaf(d3, d3, s4[3]);
+          const float b4[4] = {bb.x, bb.y, bb.z, bb.w};
+          row_plus<4>(v + j, b4);
+          row_add_sq<4>(var, v + j, mean);
         }
       }
-      const float rstd = pair_rstd((s4[0] + s4[1]) + (s4[2] + s4[3]));
+      const float rstd = pair_rstd(var.total());
       if (lane == 0) bulk_wait_read0();
       epi_sync();  // every warp's x_out staging read: sA takes LN(x_out)
 #pragma unroll 1
@@ -554,10 +535,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int j = 0; j < 32; j += 4) {
           const float4 bb = *reinterpret_cast<const float4*>(sB2 + c + j);
-          v[j] = (v[j] + bb.x - mean) * rstd;
-          v[j + 1] = (v[j + 1] + bb.y - mean) * rstd;
-          v[j + 2] = (v[j + 2] + bb.z - mean) * rstd;
-          v[j + 3] = (v[j + 3] + bb.w - mean) * rstd;
+          const float b4[4] = {bb.x, bb.y, bb.z, bb.w};
+          row_plus<4>(v + j, b4);
+          row_norm<4>(v + j, mean, rstd);
         }
         store_split_cols(sA, r, c, v);
         if (i & 1) {

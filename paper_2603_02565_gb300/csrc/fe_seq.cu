@@ -164,17 +164,14 @@ __device__ __noinline__ void epi_resid_ln(uint8_t* sA, float* red, uint32_t acc_
   if (add) {
     float w[32];
     tmem_ld32(add_t + c, w);
-#pragma unroll
-    for (int j = 0; j < 32; ++j) v[j] += w[j];
+    row_plus<32>(v, w);
   }
   if (bias) {
 #pragma unroll
     for (int j = 0; j < 32; j += 4) {
       const float4 b = *reinterpret_cast<const float4*>(bias + c + j);
-      v[j] += b.x;
-      v[j + 1] += b.y;
-      v[j + 2] += b.z;
-      v[j + 3] += b.w;
+      const float bb[4] = {b.x, b.y, b.z, b.w};
+      row_plus<4>(v + j, bb);
     }
   }
   if (add || bias) tmem_st32_nw(acc_t + c, v);
@@ -184,25 +181,17 @@ __device__ __noinline__ void epi_resid_ln(uint8_t* sA, float* red, uint32_t acc_
       *reinterpret_cast<float4*>(out_row + c + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
   }
   // four independent partial sums per statistic (short dependency chains)
-  float s4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-  for (int j = 0; j < 32; ++j) s4[j & 3] += v[j];
-  red[qt * 128 + r] = (s4[0] + s4[1]) + (s4[2] + s4[3]);
+  RowSum sum, var;
+  row_add<32>(sum, v);
+  red[qt * 128 + r] = sum.total();
   asm volatile("bar.sync %0, 128;" ::"r"(1 + q) : "memory");
   const float mean = ((red[r] + red[128 + r]) + (red[256 + r] + red[384 + r])) * (1.f / (float)D);
-#pragma unroll
-  for (int i = 0; i < 4; ++i) s4[i] = 0.f;
-#pragma unroll
-  for (int j = 0; j < 32; ++j) {
-    const float dv = v[j] - mean;
-    s4[j & 3] = fmaf(dv, dv, s4[j & 3]);
-  }
-  red[512 + qt * 128 + r] = (s4[0] + s4[1]) + (s4[2] + s4[3]);
+  row_add_sq<32>(var, v, mean);
+  red[512 + qt * 128 + r] = var.total();
   asm volatile("bar.sync %0, 128;" ::"r"(1 + q) : "memory");
   const float rstd =
       1.0f / sqrtf(((red[512 + r] + red[640 + r]) + (red[768 + r] + red[896 + r])) * (1.f / (float)D) + eps);
-#pragma unroll
-  for (int j = 0; j < 32; ++j) v[j] = (v[j] - mean) * rstd;
+  row_norm<32>(v, mean, rstd);
   store_split32(sA, r, qt, v);
   if (add || bias) tmem_st_wait();
 }
@@ -274,12 +263,13 @@ __device__ __forceinline__ void cls_rows(uint8_t* sA, const int* sErow, const ui
     for (int k = 0; k < NR; ++k)
       if (live[k]) m[k] = fmaxf(m[k], (part(sErow[rrow[k] * 32 + j]) + qp) * sl2);
   }
-  float sum[NR], o[NR][16];
+  float sum[NR];
+  uint64_t o[NR][8];  // column pairs
 #pragma unroll
   for (int k = 0; k < NR; ++k) {
     sum[k] = 0.f;
 #pragma unroll
-    for (int i = 0; i < 16; ++i) o[k][i] = 0.f;
+    for (int i = 0; i < 8; ++i) o[k][i] = 0;  // (0.f, 0.f)
   }
 #pragma unroll 1
   for (int j = 0; j < L; ++j) {
@@ -298,35 +288,37 @@ __device__ __forceinline__ void cls_rows(uint8_t* sA, const int* sErow, const ui
       const float w = ex2_approx((part(e) + qp) * sl2 - m[k]);
       sum[k] += w;
       const uint32_t wv[8] = {a4.x, a4.y, a4.z, a4.w, b4.x, b4.y, b4.z, b4.w};
+      const uint64_t ww = f32x2_pack(w, w);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&wv[2 * i]));
-        const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&wv[2 * i + 1]));
-        o[k][4 * i] = fmaf(w, a.x + pp[i].x, o[k][4 * i]);
-        o[k][4 * i + 1] = fmaf(w, a.y + pp[i].y, o[k][4 * i + 1]);
-        o[k][4 * i + 2] = fmaf(w, b.x + pp[i].z, o[k][4 * i + 2]);
-        o[k][4 * i + 3] = fmaf(w, b.y + pp[i].w, o[k][4 * i + 3]);
+      for (int i = 0; i < 8; ++i) {
+        const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&wv[i]));
+        const float4 pv = pp[i >> 1];
+        o[k][i] = f32x2_fma(ww, f32x2_add(f32x2_pack(a.x, a.y), i & 1 ? f32x2_pack(pv.z, pv.w) : f32x2_pack(pv.x, pv.y)),
+                            o[k][i]);
       }
     }
   }
 #pragma unroll
   for (int k = 0; k < NR; ++k) {
     const int rr = rrow[k];
+    float ov[16];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) f32x2_unpack(o[k][i], ov[2 * i], ov[2 * i + 1]);
     if (live[k]) {
       const float pc = ex2_approx(s0 - m[k]);
       const float inv = 1.f / (sum[k] + pc);
 #pragma unroll
-      for (int i = 0; i < 16; ++i) o[k][i] = fmaf(pc, sV0[16 * li + ((i + 8 * rot) & 15)], o[k][i]) * inv;
+      for (int i = 0; i < 16; ++i) ov[i] = fmaf(pc, sV0[16 * li + ((i + 8 * rot) & 15)], ov[i]) * inv;
     } else if (rr < rows_v) {
       // a rejected request's scores become NaN; o = v0 keeps its rows finite
 #pragma unroll
-      for (int i = 0; i < 16; ++i) o[k][i] = sV0[16 * li + ((i + 8 * rot) & 15)];
+      for (int i = 0; i < 16; ++i) ov[i] = sV0[16 * li + ((i + 8 * rot) & 15)];
     }
     // o -> row rr of the split tile: registers 0-7 (columns 16 li + 8 rot ..) are
     // 16-byte piece 2 (li % 4) + rot of plane li / 4, registers 8-15 the other piece
     uint32_t hi[8], lo[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) split2(o[k][2 * i], o[k][2 * i + 1], hi[i], lo[i]);
+    for (int i = 0; i < 8; ++i) split2(ov[2 * i], ov[2 * i + 1], hi[i], lo[i]);
     uint8_t* rowp = sA + (size_t)((li >> 2) * 2) * kAPlane + (size_t)rr * 128u;
     const uint32_t o0 = (uint32_t)((2 * (li & 3) + rot) ^ (rr & 7)) << 4;
     const uint32_t o1 = (uint32_t)((2 * (li & 3) + (rot ^ 1)) ^ (rr & 7)) << 4;
@@ -708,9 +700,12 @@ __global__ void __launch_bounds__(kThreads, 1)
           tmem_ld32(col, v);
           uint32_t hi[16], lo[16];
 #pragma unroll
-          for (int j = 0; j < 16; ++j)
-            split2_trunc(relu_keep_nan(v[2 * j] + bias[2 * j]), relu_keep_nan(v[2 * j + 1] + bias[2 * j + 1]), hi[j],
-                         lo[j]);
+          for (int j = 0; j < 16; ++j) {
+            const float2 bb = *reinterpret_cast<const float2*>(bias + 2 * j);
+            const float b2[2] = {bb.x, bb.y};
+            row_plus<2>(v + 2 * j, b2);
+            split2_trunc(relu_keep_nan(v[2 * j]), relu_keep_nan(v[2 * j + 1]), hi[j], lo[j]);
+          }
           tmem_st16_nowait(col, hi);
           tmem_st16_nowait(col + 16u, lo);
         }
