@@ -15,10 +15,11 @@
 //                      features); streams the segment's C key/value rows
 //                      through operand tiles of 64 rows, phi(K)^T [V | 1] on
 //                      the tensor core
-//   lin_attn_kernel  : one CTA per segment; the segment's states of one layer
-//                      (all heads) and phi(q) of 32-row blocks in shared
-//                      memory, one warp per (head, 16 rows), a lane per
-//                      output column and 16 rows of accumulators in registers
+//   lin_attn_kernel  : one to eight CTAs per segment; the segment's states of
+//                      one layer (all heads) and phi(q) of 16- to 64-row
+//                      blocks in shared memory, one warp per (head, 8 rows), a
+//                      lane per output column and 8 rows of accumulators in
+//                      registers
 #include <cuda_fp16.h>
 
 #include "fe_common.cuh"
@@ -239,24 +240,28 @@ __global__ void __launch_bounds__(256, 2) lin_state_kernel(const __half* __restr
 }
 
 namespace {
-constexpr int kRowBlock = 32;  // element rows staged per block of lin_attn_kernel
-constexpr int kRowTask = 16;   // rows per warp task (a task: one head, kRowTask rows)
+constexpr int kRowBlock = 64;  // element rows staged per block of lin_attn_kernel, at most
+constexpr int kRowTask = 8;    // rows per warp task (a task: one head, kRowTask rows)
 }
 
 template <int DH>
 __global__ void __launch_bounds__(256) lin_attn_kernel(const __half* __restrict__ q, int ldq, int d,
                                                        const float* __restrict__ states, int Ly, int l, int H,
                                                        const int* __restrict__ off_dev, const int* __restrict__ cnt_dev,
-                                                       int stride, int cnt_fixed, bf16* o_h, bf16* o_l, int ldo) {
+                                                       int stride, int cnt_fixed, int row_block, bf16* o_h, bf16* o_l,
+                                                       int ldo) {
   constexpr int SB = DH * DH + DH;
   constexpr int NJ = DH / 32;           // output columns per lane
   extern __shared__ __align__(16) float sm[];
   float* sst = sm;                      // [H][SB]: layer l's states of this segment
-  float* sq = sm + H * SB;              // [kRowBlock][d + 4]: phi(q) of a block of rows (padded rows)
+  float* sq = sm + H * SB;              // [row_block][d + 4]: phi(q) of a block of rows (padded rows)
   const int ldq_s = d + 4;
   const int s = blockIdx.x;
   pdl_wait();
   pdl_trigger();
+  const int off = off_dev ? off_dev[s] : s * stride;
+  const int cnt = cnt_dev ? cnt_dev[s] : cnt_fixed;
+  if ((int)blockIdx.y * row_block >= cnt) return;
   // the states, four 16-byte loads in flight per thread at a time
   {
     const float4* src = reinterpret_cast<const float4*>(states + ((size_t)s * Ly + l) * H * SB);
@@ -272,12 +277,10 @@ __global__ void __launch_bounds__(256) lin_attn_kernel(const __half* __restrict_
         if (i0 + 256 * u < n4) dst[i0 + 256 * u] = v[u];
     }
   }
-  const int off = off_dev ? off_dev[s] : s * stride;
-  const int cnt = cnt_dev ? cnt_dev[s] : cnt_fixed;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int d8 = d / 8;
-  for (int rb = 0; rb < cnt; rb += kRowBlock) {
-    const int nr = min(kRowBlock, cnt - rb);
+  for (int rb = blockIdx.y * row_block; rb < cnt; rb += gridDim.y * row_block) {
+    const int nr = min(row_block, cnt - rb);
     __syncthreads();  // the previous block (and, the first time, the states) consumed / written
     for (int i0 = threadIdx.x; i0 < nr * d8; i0 += 1024) {
       uint4 raw[4];
@@ -364,8 +367,8 @@ __global__ void __launch_bounds__(256) lin_attn_kernel(const __half* __restrict_
 }
 
 namespace {
-// H <= 8 heads of d_h = 64, and a block of rows of width d <= 512
-constexpr int kLinAttnSmemMax = 8 * (64 * 64 + 64) * 4 + kRowBlock * (512 + 4) * 4;
+// H <= 8 heads of d_h = 64, and a block of rows of width d <= 512 (half a block there)
+constexpr int kLinAttnSmemMax = 8 * (64 * 64 + 64) * 4 + kRowBlock / 2 * (512 + 4) * 4;
 }
 
 cudaError_t linattn_prepare() {
@@ -406,15 +409,24 @@ cudaError_t lin_attn_launch(const bf16* q, int ldq, const float* states, int n_s
                             int ldo, cudaStream_t s) {
   if (n_seg <= 0) return cudaSuccess;
   const int d = H * dh;
-  const size_t smem = ((size_t)H * (dh * dh + dh) + (size_t)kRowBlock * (d + 4)) * sizeof(float);
+  // A CTA is a chain of two loads and a product per block of rows, so a segment's rows are dealt out to CTAs
+  // until there are about four per SM (in all for 256 segments of 60 rows, d = 64: one CTA each and blocks of 32
+  // rows, 16 per task, 190 us, blocks of 64 and 8 per task 186.4, two CTAs 178.1, more 178.0; for 64 segments
+  // 120.1, 113.2, 109.3 with eight), in smaller blocks the more of them there are (64 segments of 100 rows, d =
+  // 128: blocks of 32 190, of 16 185; 256 of 60, d = 64, with four CTAs: 178.0 and 180.5).
+  int ny = 4 * 152 / n_seg;
+  ny = ny < 1 ? 1 : ny > 8 ? 8 : ny;
+  const int row_block = ny >= 4 ? kRowBlock / 4 : ny > 1 || d > 256 ? kRowBlock / 2 : kRowBlock;
+  const size_t smem = ((size_t)H * (dh * dh + dh) + (size_t)row_block * (d + 4)) * sizeof(float);
   if (smem > (size_t)kLinAttnSmemMax) return cudaErrorInvalidValue;
   const __half* qh = reinterpret_cast<const __half*>(q);
+  const dim3 grid((unsigned)n_seg, (unsigned)ny);
   if (dh == 32)
-    return launch_k(lin_attn_kernel<32>, dim3((unsigned)n_seg), dim3(256), smem, s, qh, ldq, d, states, Ly, l, H, off_dev,
-                    cnt_dev, stride, cnt_fixed, o_h, o_l, ldo);
+    return launch_k(lin_attn_kernel<32>, grid, dim3(256), smem, s, qh, ldq, d, states, Ly, l, H, off_dev, cnt_dev, stride,
+                    cnt_fixed, row_block, o_h, o_l, ldo);
   if (dh == 64)
-    return launch_k(lin_attn_kernel<64>, dim3((unsigned)n_seg), dim3(256), smem, s, qh, ldq, d, states, Ly, l, H, off_dev,
-                    cnt_dev, stride, cnt_fixed, o_h, o_l, ldo);
+    return launch_k(lin_attn_kernel<64>, grid, dim3(256), smem, s, qh, ldq, d, states, Ly, l, H, off_dev, cnt_dev, stride,
+                    cnt_fixed, row_block, o_h, o_l, ldo);
   return cudaErrorInvalidValue;
 }
 
