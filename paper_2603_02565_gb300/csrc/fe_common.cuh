@@ -446,6 +446,13 @@ __device__ __forceinline__ void ld_sector(const float* p, float* x) {
                : "memory");
 }
 
+// the same for stores (32-byte aligned)
+__device__ __forceinline__ void st_sector(float* p, const float* x) {
+  asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "f"(x[0]), "f"(x[1]), "f"(x[2]), "f"(x[3]),
+               "f"(x[4]), "f"(x[5]), "f"(x[6]), "f"(x[7])
+               : "memory");
+}
+
 // 32 lanes x 64 columns -> 64 registers per thread, one load and one wait
 __device__ __forceinline__ void tmem_ld64(uint32_t taddr, float* v) {
   uint32_t r[64];

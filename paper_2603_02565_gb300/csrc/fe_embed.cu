@@ -227,9 +227,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                                   ((uint32_t)((g & 7) ^ (gr & 7)) << 4)) = pc[j];
         if (valid && 8 * g < d) {
           float* hr = p.h + (size_t)row * p.ldh + 8 * g;
-          *reinterpret_cast<float4*>(hr) = make_float4(lo16(pc[j].x), hi16(pc[j].x), lo16(pc[j].y), hi16(pc[j].y));
-          *reinterpret_cast<float4*>(hr + 4) =
-              make_float4(lo16(pc[j].z), hi16(pc[j].z), lo16(pc[j].w), hi16(pc[j].w));
+          const float x[8] = {lo16(pc[j].x), hi16(pc[j].x), lo16(pc[j].y), hi16(pc[j].y),
+                              lo16(pc[j].z), hi16(pc[j].z), lo16(pc[j].w), hi16(pc[j].w)};
+          st_sector(hr, x);  // (two 16-byte stores a thread: ragged requests 96.1 us in all instead of 95.0)
         }
       }
       if (part == 0) stats[gr] = valid ? make_float2(rstd, -mean * rstd) : make_float2(0.f, 0.f);
@@ -299,7 +299,8 @@ cudaError_t embed_q_prepare() {
 
 cudaError_t embed_q_launch(const CUtensorMap* w, const CUtensorMap* q_out, const EmbedParams& p, cudaStream_t s) {
   if (p.rows <= 0 || p.B <= 0) return cudaSuccess;
-  if (!embed_q_supported(p.d, p.d_pad, 1, 0) || !p.pool || !p.off || !p.list || !p.h || p.ldh < p.d || p.ldh % 4)
+  if (!embed_q_supported(p.d, p.d_pad, 1, 0) || !p.pool || !p.off || !p.list || !p.h || p.ldh < p.d || p.ldh % 8 ||
+      (uintptr_t)p.h % 32)
     return cudaErrorInvalidValue;
   const long long tiles = (p.rows + BM - 1) / BM;  // (the valid rows, read on the device, are fewer)
   long long grid = g_embed_sms > 0 ? g_embed_sms : 148;
