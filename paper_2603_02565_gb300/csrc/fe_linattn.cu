@@ -34,12 +34,6 @@ namespace {
 // of the keys and queries it is applied to
 __device__ __forceinline__ float phi(float x) { return x > 0.f ? x + 1.f : __expf(x); }
 
-__device__ __forceinline__ float warp_sum32(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-  return v;
-}
-
 constexpr int kChunk = 64;                // context rows per operand tile
 constexpr uint32_t kAtom = kChunk * 128;  // 64 features x kChunk rows, f16
 
