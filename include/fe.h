@@ -344,10 +344,13 @@ int fe_debug_alloc_hook(int fail_at, int64_t* live_out);
 
 /*
  * Test hook for the bounded device-side waits (no counterpart in the paper).
- * Enqueues on `stream` one thread that waits, through the batch kernels' own
- * bounded mbarrier wait, on a barrier that nothing arrives on, with a limit of
- * limit_us microseconds (1..1000000) instead of the batch kernels' one
- * second; no copy or tensor-core work is in flight.  The status word then
+ * Enqueues on `stream` one block whose warps wait, through each form of the
+ * batch kernels' own bounded mbarrier waits, on a barrier that nothing arrives
+ * on, with a limit of limit_us microseconds (1..1000000) instead of the batch
+ * kernels' one second; no copy or tensor-core work is in flight.  Half of the
+ * warps give up by that limit, the others because the status word is set; each
+ * then waits seven times more, a few polls each, and an epilogue warp's arrivals
+ * must not go through (FE_ERR_NUMERIC is returned otherwise).  The status then
  * reaches the host as a batch's does (copied to the page-locked word and
  * cleared), so the call waits and returns FE_ERR_TIMEOUT; the context stays
  * usable for the next batch.  Reserves a minimal workspace when the context

@@ -1725,7 +1725,7 @@ int fe_debug_wait_probe(fe_ctx* c, uint32_t limit_us, void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
   // the status word's way to the host is the batch's: copied to the
   // page-locked word, then cleared for the next batch
-  FE_CK(fe::wait_probe_launch(c->status, (uint64_t)limit_us * 1000ull, s));
+  FE_CK(fe::wait_probe_launch(c->status, limit_us, s));
   FE_CK(cudaMemcpyAsync(c->host_status, c->status, sizeof(int), cudaMemcpyDeviceToHost, s));
   FE_CK(cudaMemsetAsync(c->status, 0, sizeof(int), s));
   FE_CK(cudaEventRecord(c->done_ev, s));

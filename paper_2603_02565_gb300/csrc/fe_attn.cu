@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(AttnCfg<DH>::kThreads, 1)
     cur_first(p, b0, row0, lc);
     l_n = chunks(lc);
     auto load_next = [&]() {
-      mbar_wait_warp(kv_empty + ls, lpar, p.status);
+      mbar_wait_load(kv_empty + ls, kv_full + ls, lpar, p.status);
       uint8_t* kv = sKV + ls * Cfg::kKVBytes;
       const int row = kv_base(lc) + lj * CK;
       mbar_arrive_expect_tx_if(kv_full + ls, Cfg::kKVBytes, go);
@@ -280,9 +280,9 @@ __global__ void __launch_bounds__(AttnCfg<DH>::kThreads, 1)
       const uint64_t qd0 = desc_sw(smem_u32(sQ), Cfg::kSbo, Cfg::kSwz);
       const uint64_t kd0 = desc_sw(smem_u32(sKV), Cfg::kSbo, Cfg::kSwz);
       const uint64_t vd0 = desc_sw(smem_u32(sKV + Cfg::kKVTile), Cfg::kSbo, Cfg::kSwz);
-      // S: the next S's unit, chunk, chunk count, stage, Q buffer; units and S issued
+      // S: the next S's unit, chunk, chunk count, stage, Q buffer; S issued
       Cursor sc = lc;
-      int sj = 0, s_nch = l_n, ss = 0, sq = 0, su = 0, g_s = 0;
+      int sj = 0, s_nch = l_n, ss = 0, sq = 0, g_s = 0;
       uint32_t spar = 0, sqpar = 0;
       // request chunks up to number `last`, one at a call while the ring first fills, then two
       auto fill = [&](int last) {
@@ -292,9 +292,9 @@ __global__ void __launch_bounds__(AttnCfg<DH>::kThreads, 1)
       // S of the next chunk, once the softmax holds the previous one
       auto issue_s = [&]() {
         if (sc.b >= p.n_segments) return;
-        if (g_s > 0) mbar_wait_warp(s_read, (uint32_t)(g_s - 1) & 1u, p.status);
-        if (sj == 0) mbar_wait_warp(q_full + sq, sqpar, p.status);
-        mbar_wait_warp(kv_full + ss, spar, p.status);
+        if (g_s > 0) mbar_wait_role(s_read, (uint32_t)(g_s - 1) & 1u, p.status);
+        if (sj == 0) mbar_wait_role(q_full + sq, sqpar, p.status);
+        mbar_wait_role(kv_full + ss, spar, p.status);
         tc_fence_after();
         const uint64_t qd = qd0 + (uint64_t)((sq * Cfg::kQBytes) >> 4);
         const uint64_t kd = kd0 + (uint64_t)((ss * Cfg::kKVBytes) >> 4);
@@ -320,7 +320,6 @@ __global__ void __launch_bounds__(AttnCfg<DH>::kThreads, 1)
             sqpar ^= 1u;
           }
           sj = 0;
-          ++su;
           cur_next(p, row0, sc);
           s_nch = chunks(sc);
         }
@@ -333,7 +332,7 @@ __global__ void __launch_bounds__(AttnCfg<DH>::kThreads, 1)
         const bool next_first = sj == 0;  // S_{g+1} opens a unit
         fill(g - 1 + NS);                 // up to the stage of PV_{g-1}, complete before P_g may be written
         issue_s();                        // S_{g+1}
-        mbar_wait_warp(p_full, (uint32_t)g & 1u, p.status);
+        mbar_wait_role(p_full, (uint32_t)g & 1u, p.status);
         tc_fence_after();
         const uint64_t vd = vd0 + (uint64_t)((ps * Cfg::kKVBytes) >> 4);
 #pragma unroll
@@ -346,15 +345,12 @@ __global__ void __launch_bounds__(AttnCfg<DH>::kThreads, 1)
         first = next_first;
       }
       umma_drain(drain, p.status, go);
-      // the last loads land before this block's shared memory goes away (after a
-      // timed-out wait nothing else has waited for them)
-      for (int i = su < NQ ? 0 : su - NQ; i < su; ++i)
-        mbar_wait_warp(q_full + i % NQ, (uint32_t)(i / NQ) & 1u, p.status);
     } else if (load) {
       while (lc.b < p.n_segments) load_next();
     }
-    for (int i = lg < NS ? 0 : lg - NS; i < lg; ++i)
-      mbar_wait_warp(kv_full + i % NS, (uint32_t)(i / NS) & 1u, p.status);
+    // the last loads land before this block's shared memory goes away (after a
+    // timed-out wait nothing else has waited for them)
+    if (load) mbar_landed_ring(kv_full, ls, lpar, NS, p.status);
   } else {
     // ---------------- softmax / output ----------------
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(DH == 32 ? 104 : 208));
@@ -364,7 +360,7 @@ __global__ void __launch_bounds__(AttnCfg<DH>::kThreads, 1)
     const uint32_t t_p = t_s + (uint32_t)Cfg::kP, t_o = t_s + (uint32_t)Cfg::kO;
     const uint32_t go = elect_one();
     const uint32_t bb = smem_u32(bars);  // the group's barriers
-    int uq = 0;  // the unit's Q buffer; this warp's rows of it take the unit's output
+    int u = 0;  // the unit; its Q buffer is u % NQ, and this warp's rows of it take the unit's output
     constexpr uint32_t kKVE = 8u * (NQ + NS), kSFull = 8u * (NQ + 2 * NS);
     const float sc = p.scale_log2;
     int g = 0, ps = 0;         // chunk of the group's stream; the stage of chunk g - 1
@@ -372,8 +368,10 @@ __global__ void __launch_bounds__(AttnCfg<DH>::kThreads, 1)
     // This warp loads its own 32 rows of each unit's Q tile, one unit ahead:
     // row block k of the tile goes to lane quadrant (k - grp) mod 4.  The buffer's
     // previous unit is done with here (its S are complete, its output is stored).
-    auto load_q = [&](const Cursor& c, int buf) {
+    auto load_q = [&](const Cursor& c, int v) {
       if (c.b >= p.n_segments) return;
+      const int buf = v % NQ;
+      mbar_landed_at(bb + 8u * (uint32_t)buf, (uint32_t)(v / NQ - 1) & 1u, p.status);  // (a fresh barrier passes)
       const int blk = c.q0 + (r & ~31);
       if (blk < c.qcnt) {
         mbar_arrive_expect_tx_if(q_full + buf, Cfg::kQBlock, go);
@@ -388,7 +386,7 @@ __global__ void __launch_bounds__(AttnCfg<DH>::kThreads, 1)
     load_q(next, 0);
     for (c = next; c.b < p.n_segments; c = next) {
       cur_next(p, row0, next);
-      load_q(next, uq ^ 1);
+      load_q(next, u + 1);
       // the running maximum m that P is taken against moves only when a chunk's
       // maximum exceeds it by more than kSlack (log2 units; P <= 2^kSlack stays
       // far inside f16), and then the unit's output accumulator in TMEM is
@@ -510,7 +508,7 @@ __global__ void __launch_bounds__(AttnCfg<DH>::kThreads, 1)
           for (int i = 0; i < DH / 2; ++i) split2(o[2 * i] * inv, o[2 * i + 1] * inv, hi[i], lo[i]);
         }
         const size_t blk = (size_t)(c.qoff + c.q0 + (r & ~31)) * p.ldo + p.o_col + head * DH;
-        uint8_t* sOut = sQ + uq * Cfg::kQBytes + q4 * Cfg::kQBlock;
+        uint8_t* sOut = sQ + (u % NQ) * Cfg::kQBytes + q4 * Cfg::kQBlock;
         auto store = [&](bf16* dst, const uint32_t* w) {
 #pragma unroll
           for (int k = 0; k < NC; ++k)
@@ -531,8 +529,11 @@ __global__ void __launch_bounds__(AttnCfg<DH>::kThreads, 1)
         fence_async_shared();  // staging read before the next load into these rows
         __syncwarp();
       }
-      uq ^= 1;
+      ++u;
     }
+    // (after a timed-out wait, the Q rows still on their way)
+    for (int v = u < NQ ? 0 : u - NQ; v < u; ++v)
+      mbar_landed_at(bb + 8u * (uint32_t)(v % NQ), (uint32_t)(v / NQ) & 1u, p.status);
   }
 
   __syncwarp();

@@ -14,8 +14,8 @@
 
 namespace fe {
 
-// A bounded wait gives up after this many nanoseconds of %globaltimer.
-constexpr uint64_t kWaitLimitNs = 1000000000ull;
+// A bounded wait gives up after this many microseconds of %globaltimer.
+constexpr uint32_t kWaitLimitUs = 1000000;
 
 // ---------------------------------------------------------------------------
 // split bf16: x ~= hi + lo with hi = bf16(x), lo = bf16(x - hi)
@@ -106,62 +106,46 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 
-// Wait for the completion of the phase with the given parity.  Gives up after
-// limit_ns of %globaltimer, sets ST_TIMEOUT in *status and returns false.
-// Also gives up at once when another CTA of the batch has already timed out.
-__device__ __forceinline__ bool mbar_wait_bounded_ns(uint64_t* bar, uint32_t parity, int* status,
-                                                     uint64_t limit_ns) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = globaltimer_ns();
-  for (uint32_t it = 1;; ++it) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((it & 255u) == 0u && (*reinterpret_cast<volatile int*>(status) & ST_TIMEOUT)) return false;
-    if (globaltimer_ns() - t0 > limit_ns) {
-      atomicOr(status, ST_TIMEOUT);
-      return false;
-    }
-  }
-}
-
-// The batch kernels' wait: limit kWaitLimitNs.
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity, int* status) {
-  return mbar_wait_bounded_ns(bar, parity, status, kWaitLimitNs);
-}
-
-// The same wait with its loop out of line, for kernels with many wait sites
-// and registers to spare: one copy of the loop instead of one per site.
-static __device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity, int* status) {
-  const uint64_t t0 = globaltimer_ns();
-  for (uint32_t it = 1;; ++it) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((it & 255u) == 0u && (*reinterpret_cast<volatile int*>(status) & ST_TIMEOUT)) return false;
-    if (globaltimer_ns() - t0 > kWaitLimitNs) {
-      atomicOr(status, ST_TIMEOUT);
-      return false;
-    }
-  }
-}
-
 // ---------------------------------------------------------------------------
-// Whole-warp issue.  A role that only one thread performs (tcgen05.mma, its
-// commits, TMA) is run by its whole warp in step: every lane keeps the loop
-// state and polls the barriers, and the instructions themselves are predicated
-// on the lane that elect.sync picks (always the same one).  The control flow
-// stays uniform for the compiler; behind `if (lane == 0)` with a `break` on a
-// timed-out wait, two satisfied waits, two MMAs of N = 64 and a commit took 475
-// cycles of the issuing thread, this form 126 to 180 (eight MMAs and one wait: 739
-// and 385, the tensor pipe's own time).  So a wait returns nothing: after a
-// timeout the role runs on to its end without synchronisation, every later wait
-// giving up at once (the batch's results are invalid then; every address it
-// uses stays in bounds).  A wait ends with the warp converged: an elected lane
-// that ran ahead could advance a barrier by two phases under a lane still
-// polling it.
+// Whole-warp issue and bounded waits.  A role that only one thread performs
+// (tcgen05.mma, its commits, TMA) is run by its whole warp in step: every lane
+// keeps the loop state and polls the barriers, and the instructions themselves
+// are predicated on the lane that elect.sync picks (always the same one).  The
+// control flow stays uniform for the compiler; behind `if (lane == 0)` two
+// satisfied waits, two MMAs of N = 64 and a commit took 475 cycles of the issuing
+// thread, this form 126 to 180 (eight MMAs and one wait: 739 and 385, the tensor
+// pipe's own time).  The predicate has to be elect.sync's own result: combined
+// with a flag of the lane it costs as much as the branch (batch of 256 requests
+// 142.6 -> 168.0 us).
+//
+// Every wait is bounded: it gives up when its limit has passed or another thread of
+// the batch has set ST_TIMEOUT (looked up every eighth poll; a poll takes up to
+// 4 us).  The results of the batch are invalid then, and nothing may fault, hang
+// or outlive its block.  What could fault is a load's arrival on a barrier whose
+// previous load is still on its way: one too many for it.  (Arrivals on a barrier
+// without bytes cannot be too many.)  Two forms rule that out:
+//  * GEMM, context, embedding and d <= 128 FFN kernels: a warp does nothing more that
+//    others wait for.  A role warp leaves its loop (mbar_wait_ok).  An epilogue
+//    warp, whose partners meet it at named barriers, walks on to the end of its loop;
+//    a lane of it that has given up (go = 0) skips its waits, arrives no more and
+//    loads no more (mbar_wait_warp).
+//  * Attention, d = 256 FFN and sequence kernels: every role walks on, some 30 us a
+//    wait, on addresses that stay in bounds, and in front of each load waits for the
+//    previous one's bytes on that barrier, too (mbar_wait_load).  With a vote and an
+//    exit in their loops the d = 256 FFN was 2 to 3 % slower, the attention up to 6 %.
+// At its end each role waits for the copies and products that it has issued
+// (mbar_landed, umma_drain).
+// A wait ends with the warp converged: an issuing lane that ran ahead could
+// advance a barrier by two phases under a lane still polling it.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t elect_one() {
   uint32_t e;
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
   return e;
 }
+// State of an epilogue warp's lane: 1 for lane 0, which arrives for the warp, 2 for
+// the others, 0 after a wait of this lane has given up.
+__device__ __forceinline__ uint32_t lane0_go() { return (threadIdx.x & 31) == 0 ? 1u : 2u; }
 
 __device__ __forceinline__ bool mbar_try_wait_at(uint32_t bar, uint32_t parity) {
   uint32_t ok;
@@ -174,22 +158,36 @@ __device__ __forceinline__ bool mbar_try_wait_at(uint32_t bar, uint32_t parity) 
       : "memory");
   return ok != 0;
 }
-// The whole warp's wait.  Its loop is out of line: these kernels run much of their
-// code once per launch, so its size shows (the loop in line at every wait: serving
-// 156.7 -> 163.4 us, the wide ragged batch 221.2 -> 228.8).
-__device__ __forceinline__ void mbar_wait_warp(uint64_t* bar, uint32_t parity, int* status) {
-  if (!mbar_try_wait(bar, parity)) mbar_wait_slow(bar, parity, status);
+
+// The polling loop, out of line: false when it gives up.
+static __device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity, int* status, uint32_t limit_us) {
+  const uint64_t t0 = globaltimer_ns();
+  for (uint32_t it = 1;; ++it) {
+    if (mbar_try_wait(bar, parity)) return true;
+    if ((it & 7u) == 0u && (*reinterpret_cast<volatile int*>(status) & ST_TIMEOUT)) return false;
+    if (globaltimer_ns() - t0 > (uint64_t)limit_us * 1000u) {
+      atomicOr(status, ST_TIMEOUT);
+      return false;
+    }
+  }
+}
+// The wait of a warp that walks on.  Its loop is out of line: these kernels run much of their code
+// once per launch, so its size shows (the loop in line at every wait made a batch
+// of 256 requests 4 % slower).
+__device__ __forceinline__ void mbar_wait_role(uint64_t* bar, uint32_t parity, int* status,
+                                               uint32_t limit_us = kWaitLimitUs) {
+  if (!mbar_try_wait(bar, parity)) mbar_wait_slow(bar, parity, status, limit_us);
   __syncwarp();
 }
 // The same by shared-memory address and in line, where a call would spill the
-// values live across it.  It gives up after kWaitLimitNs (about; the timer's
-// upper bits) and, once any thread of the batch has, after 256 polls.
-__device__ __forceinline__ void mbar_wait_at(uint32_t bar, uint32_t parity, int* status) {
+// values live across it.  The limit counts in 65.5 us (the timer's upper bits).
+__device__ __forceinline__ void mbar_wait_at(uint32_t bar, uint32_t parity, int* status,
+                                             uint32_t limit_us = kWaitLimitUs) {
   if (!mbar_try_wait_at(bar, parity)) {
     const uint32_t t0 = (uint32_t)(globaltimer_ns() >> 16);
     for (uint32_t it = 1; !mbar_try_wait_at(bar, parity); ++it) {
-      if ((it & 255u) == 0u && (*reinterpret_cast<volatile int*>(status) & ST_TIMEOUT)) break;
-      if ((uint32_t)(globaltimer_ns() >> 16) - t0 > (uint32_t)(kWaitLimitNs >> 16)) {
+      if ((it & 7u) == 0u && (*reinterpret_cast<volatile int*>(status) & ST_TIMEOUT)) break;
+      if ((uint32_t)(globaltimer_ns() >> 16) - t0 > (uint32_t)((uint64_t)limit_us * 1000u >> 16)) {
         atomicOr(status, ST_TIMEOUT);
         break;
       }
@@ -197,12 +195,135 @@ __device__ __forceinline__ void mbar_wait_at(uint32_t bar, uint32_t parity, int*
   }
   __syncwarp();
 }
-__device__ __forceinline__ void mbar_arrive_if_at(uint32_t bar, uint32_t go) {
+// Whether a phase is complete, without the time that try_wait spends in an incomplete phase
+__device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+// The wait of a warp that leaves its loop: false, in every lane, if one has given up.
+__device__ __forceinline__ bool mbar_wait_ok(uint64_t* bar, uint32_t parity, int* status,
+                                             uint32_t limit_us = kWaitLimitUs) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  return __all_sync(0xffffffffu, mbar_wait_slow(bar, parity, status, limit_us));
+}
+// The wait for bytes or products on their way, which need nobody else's progress:
+// whatever the status says.
+static __device__ __noinline__ void mbar_landed_slow(uint64_t* bar, uint32_t parity, int* status, uint32_t limit_us) {
+  const uint64_t t0 = globaltimer_ns();
+  while (!mbar_try_wait(bar, parity)) {
+    if (globaltimer_ns() - t0 > (uint64_t)limit_us * 1000u) {
+      atomicOr(status, ST_TIMEOUT);
+      break;
+    }
+  }
+}
+__device__ __forceinline__ void mbar_landed(uint64_t* bar, uint32_t parity, int* status,
+                                            uint32_t limit_us = kWaitLimitUs) {
+  if (!mbar_try_wait(bar, parity)) mbar_landed_slow(bar, parity, status, limit_us);
+  __syncwarp();
+}
+// (in line, as mbar_wait_at)
+__device__ __forceinline__ void mbar_landed_at(uint32_t bar, uint32_t parity, int* status,
+                                               uint32_t limit_us = kWaitLimitUs) {
+  if (!mbar_try_wait_at(bar, parity)) {
+    const uint32_t t0 = (uint32_t)(globaltimer_ns() >> 16);
+    while (!mbar_try_wait_at(bar, parity)) {
+      if ((uint32_t)(globaltimer_ns() >> 16) - t0 > (uint32_t)((uint64_t)limit_us * 1000u >> 16)) {
+        atomicOr(status, ST_TIMEOUT);
+        break;
+      }
+    }
+  }
+  __syncwarp();
+}
+// The newest load on each of a ring's S barriers, the next load going to number `slot`
+// with the parity `par` of its wait (mbar_wait_load).  All are asked before one is
+// waited for: as a rule they landed long ago, and the kernel ends behind this.
+static __device__ __noinline__ void mbar_landed_ring_slow(uint64_t* full, int slot, uint32_t par, int S, int* status) {
+  for (int i = 0; i < S; ++i) mbar_landed_slow(full + i, i < slot ? par ^ 1u : par, status, kWaitLimitUs);
+}
+__device__ __forceinline__ void mbar_landed_ring(uint64_t* full, int slot, uint32_t par, int S, int* status) {
+  bool ok = true;
+#pragma unroll 4
+  for (int i = 0; i < S; ++i) ok &= mbar_test_wait(full + i, i < slot ? par ^ 1u : par);
+  if (!ok) mbar_landed_ring_slow(full, slot, par, S, status);
+  __syncwarp();
+}
+// The wait before the next load on barrier `full`: its previous load has landed (asked
+// first, off the path from the freed memory to its next load) and its memory is free.
+__device__ __forceinline__ void mbar_wait_load(uint64_t* empty, uint64_t* full, uint32_t parity, int* status) {
+  if (!mbar_try_wait(full, parity)) mbar_landed_slow(full, parity, status, kWaitLimitUs);
+  if (!mbar_try_wait(empty, parity)) mbar_wait_slow(empty, parity, status, kWaitLimitUs);
+  __syncwarp();
+}
+// An epilogue warp's wait (its loop in a function of its own, and `go` not asked in
+// front of the first poll: either made the d = 256 FFN 2 % slower).
+static __device__ __noinline__ uint32_t mbar_wait_slow_go(uint64_t* bar, uint32_t parity, int* status,
+                                                          uint32_t limit_us, uint32_t go) {
+  if (go == 0) return 0;
+  const uint64_t t0 = globaltimer_ns();
+  for (uint32_t it = 1;; ++it) {
+    if (mbar_try_wait(bar, parity)) return go;
+    if ((it & 7u) == 0u && (*reinterpret_cast<volatile int*>(status) & ST_TIMEOUT)) return 0;
+    if (globaltimer_ns() - t0 > (uint64_t)limit_us * 1000u) {
+      atomicOr(status, ST_TIMEOUT);
+      return 0;
+    }
+  }
+}
+__device__ __forceinline__ void mbar_wait_warp(uint64_t* bar, uint32_t parity, int* status, uint32_t& go,
+                                               uint32_t limit_us = kWaitLimitUs) {
+  if (!mbar_try_wait(bar, parity)) go = mbar_wait_slow_go(bar, parity, status, limit_us, go);
+  __syncwarp();
+}
+// The same with cluster-scope acquire (peers' stores into this CTA).
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+static __device__ __noinline__ bool mbar_wait_cluster_slow(uint64_t* bar, uint32_t parity, int* status,
+                                                           uint32_t limit_us) {
+  const uint64_t t0 = globaltimer_ns();
+  for (uint32_t it = 1;; ++it) {
+    if (mbar_try_wait_cluster(bar, parity)) return true;
+    if ((it & 7u) == 0u && (*reinterpret_cast<volatile int*>(status) & ST_TIMEOUT)) return false;
+    if (globaltimer_ns() - t0 > (uint64_t)limit_us * 1000u) {
+      atomicOr(status, ST_TIMEOUT);
+      return false;
+    }
+  }
+}
+__device__ __forceinline__ void mbar_wait_cluster(uint64_t* bar, uint32_t parity, int* status, uint32_t& go,
+                                                  uint32_t limit_us = kWaitLimitUs) {
+  if (go != 0 && !mbar_wait_cluster_slow(bar, parity, status, limit_us)) go = 0;
+  __syncwarp();
+}
+
+__device__ __forceinline__ void mbar_arrive_if_at(uint32_t bar, bool on) {
   asm volatile(
       "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
       "@q mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}" ::"r"(bar),
-      "r"(go)
+      "r"((uint32_t)on)
       : "memory");
+}
+// An epilogue warp's arrival: its lanes' earlier (fenced) writes come before it.
+__device__ __forceinline__ void mbar_arrive_warp(uint64_t* bar, uint32_t go) {
+  __syncwarp();
+  mbar_arrive_if_at(smem_u32(bar), go == 1);
 }
 
 __device__ __forceinline__ void mbar_arrive_expect_tx_if(uint64_t* bar, uint32_t bytes, uint32_t go) {
@@ -379,12 +500,11 @@ __device__ __forceinline__ void umma_commit_if(uint64_t* bar, uint32_t go) {
       : "memory");
 }
 
-// Every product issued so far is complete before the block may free its TMEM
-// (after a timed-out wait nothing else has waited for them).  drain: a barrier of
-// count 1 that nothing else uses.
+// Every product that this warp has issued is complete before the block frees its
+// TMEM.  drain: a barrier of count 1 that nothing else uses.
 __device__ __forceinline__ void umma_drain(uint64_t* drain, int* status, uint32_t go) {
   umma_commit_if(drain, go);
-  mbar_wait_warp(drain, 0u, status);
+  mbar_landed(drain, 0u, status);
 }
 
 // 32 lanes x 32 columns of 32-bit TMEM -> 32 registers per thread (row = lane).

@@ -92,6 +92,7 @@ __device__ __forceinline__ uint64_t desc_mn128(uint32_t saddr, uint32_t lbo) {
 // elu(x) + 1 (the linear-attention feature map)
 __device__ __forceinline__ float phi_elu1(float x) { return x > 0.f ? x + 1.f : __expf(x); }
 
+
 __device__ __forceinline__ void arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
@@ -140,7 +141,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* acc_empty = bars + 9;  // [2] accumulator drained
   uint64_t* st_full = bars + 11;   // state mode: the state product of the tile complete
   uint64_t* stats_full = bars + 12;  // [2] row statistics of the tile written
-  uint64_t* drain = bars + 14;     // the products in flight at the end
+  uint64_t* drain = bars + 14;     // the products in flight at the end, and the state products
+  uint64_t* st_drain = bars + 15;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 16);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -155,6 +157,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     mbar_init(st_full, 1);
     mbar_init(drain, 1);
+    mbar_init(st_drain, 1);
     fence_mbar_init();
     prefetch_tmap(&tX);
     prefetch_tmap(&tW);
@@ -202,7 +205,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     int it = 0;
     for (int t = tile_at(it); t >= 0; t = tile_at(++it)) {
       const int rb = it % NRAW;
-      mbar_wait_warp(raw_empty + rb, ((it / NRAW) & 1) ^ 1, p.status);  // (a fresh barrier passes)
+      if (!mbar_wait_ok(raw_empty + rb, ((it / NRAW) & 1) ^ 1, p.status)) break;  // (a fresh barrier passes)
       mbar_arrive_expect_tx_if(raw_full + rb, LY.raw_bytes, go);
       // context row of this block (one K/V per candidate sequence: rep > 1)
       const int r0 = t * BM;
@@ -212,18 +215,19 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     // the last loads land before this block's shared memory goes away (after a
     // timed-out wait nothing else has waited for them)
-    for (int i = it < NRAW ? 0 : it - NRAW; i < it; ++i) mbar_wait_warp(raw_full + i % NRAW, (i / NRAW) & 1, p.status);
+    mbar_landed(w_full, 0, p.status);
+    mbar_landed_ring(raw_full, it % NRAW, ((it / NRAW) & 1) ^ 1, NRAW, p.status);
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
     const uint32_t go = elect_one();
     const uint32_t idesc = umma_idesc_bf16(BM, Nh);
     const uint64_t w0 = umma_desc_sw128(smem_u32(sW)), r0 = umma_desc_sw128(smem_u32(sRaw));
-    mbar_wait_warp(w_full, 0, p.status);
+    const bool w_ok = mbar_wait_ok(w_full, 0, p.status);
     int it = 0;
-    for (int t = tile_at(it); t >= 0; t = tile_at(++it)) {
+    for (int t = tile_at(it); t >= 0 && w_ok; t = tile_at(++it)) {
       const int ab = it % NACC, rb = it % NRAW;
-      mbar_wait_warp(acc_empty + ab, ((it / NACC) & 1) ^ 1, p.status);  // (a fresh barrier passes)
-      mbar_wait_warp(raw_full + rb, (it / NRAW) & 1, p.status);
+      if (!mbar_wait_ok(acc_empty + ab, ((it / NACC) & 1) ^ 1, p.status)) break;  // (a fresh barrier passes)
+      if (!mbar_wait_ok(raw_full + rb, (it / NRAW) & 1, p.status)) break;
       tc_fence_after();
       const uint32_t dst = tmem + (uint32_t)(256 * ab);
       const uint64_t a0 = desc_adv(r0, (uint32_t)rb * LY.raw_bytes);
@@ -249,7 +253,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     int it = 0;
     for (int t = tile_at(it); t >= 0; t = tile_at(++it)) {
       const int rb = it % NRAW;
-      mbar_wait_warp(raw_full + rb, (it / NRAW) & 1, p.status);
+      if (!mbar_wait_ok(raw_full + rb, (it / NRAW) & 1, p.status)) break;
       const uint8_t* raw = sRaw + (size_t)rb * LY.raw_bytes;
       // piece j of this thread: global piece g, column 8 g, 128-byte-swizzled
       // within its 64-column block
@@ -285,7 +289,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const float rstd = 1.0f / sqrtf(q2 / (float)d + p.eps);
       // the statistics slot: the epilogue must be done with the tile it held
       const int sl = it % NACC;
-      mbar_wait_warp(acc_empty + sl, ((it / NACC) & 1) ^ 1, p.status);
+      if (!mbar_wait_ok(acc_empty + sl, ((it / NACC) & 1) ^ 1, p.status)) break;
       if (part == 0) stats[sl * 128 + r] = make_float2(rstd, -mean * rstd);
       arrive(stats_full + sl);
       arrive(raw_empty + rb);
@@ -318,15 +322,16 @@ __global__ void __launch_bounds__(kThreads, 1)
       *reinterpret_cast<uint4*>(sPV + piece(d)) = make_uint4(0x3C003C00u, 0x3C003C00u, 0x3C003C00u, 0x3C003C00u);
       *reinterpret_cast<uint4*>(sPV + piece(d + 8)) = make_uint4(0x3C003C00u, 0x3C003C00u, 0x3C003C00u, 0x3C003C00u);
     }
+    uint32_t go = lane0_go();
     const uint32_t idesc = umma_idesc_f16(BM, d + 16) | (1u << 15) | (1u << 16);  // A and B MN-major
-    mbar_wait_warp(w_full, 0, p.status);
+    mbar_wait_warp(w_full, 0, p.status, go);
     if (ew * 32 + lane < Nh) wsum[ew * 32 + lane] = weight_colsum(sW, Nh, NKB, ew * 32 + lane);
     epi_sync();
     int it = 0;
     for (int t = tile_at(it); t >= 0; t = tile_at(++it)) {
       const int pos = it % Ts;   // row block of the segment
-      mbar_wait_warp(acc_full, it & 1, p.status);
-      mbar_wait_warp(stats_full, it & 1, p.status);
+      mbar_wait_warp(acc_full, it & 1, p.status, go);
+      mbar_wait_warp(stats_full, it & 1, p.status, go);
       tc_fence_after();
       const float2 st = stats[r];  // rstd, -rstd mu of this thread's row
       for (int c = 32 * sub; c < 2 * d; c += 64) {
@@ -341,7 +346,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int i = 0; i < 32; ++i) v[i] = phi_elu1(v[i]);
         }
         // the previous row block's state product must be done reading the operand tiles
-        if (c < 64 && it > 0) mbar_wait_warp(st_full, (it - 1) & 1, p.status);
+        if (c < 64 && it > 0) mbar_wait_warp(st_full, (it - 1) & 1, p.status, go);
         uint8_t* buf = isk ? sPK : sPV;
 #pragma unroll
         for (int j = 0; j < 4; ++j)
@@ -352,10 +357,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       // the K/V accumulator is read: it may take the next tile
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) arrive(acc_empty);
+      mbar_arrive_if_at(smem_u32(acc_empty), go == 1);
       fence_async_shared();  // the operand tiles, visible to the tensor core
       epi_sync();
-      if (ew == 0 && lane == 0) {
+      if (ew == 0 && go == 1) {
         tc_fence_after();
         const uint64_t ad = desc_mn128(smem_u32(sPK), 16384u), bd = desc_mn128(smem_u32(sPV), 16384u);
 #pragma unroll
@@ -367,7 +372,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (pos + 1 < Ts) continue;
       // the segment's last row block: its state, S of each head from the
       // diagonal blocks and z, stored (one segment per CTA pair: no atomics)
-      mbar_wait_warp(st_full, it & 1, p.status);
+      mbar_wait_warp(st_full, it & 1, p.status, go);
       tc_fence_after();
       const int seg = (t * BM) / p.C;
       float* st_seg = p.states + ((size_t)seg * 2 + l) * H * SB;
@@ -390,6 +395,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       tc_fence_before();
       epi_sync();  // the state accumulator is read before the next segment's first product
     }
+    if (ew == 0) {  // the state products are complete
+      if (lane == 0) umma_commit(st_drain);
+      mbar_landed(st_drain, 0, p.status);
+    }
   } else {
     // ---------------- epilogue: TMEM -> f16 -> TMA stores ----------------
     const int ew = warp - 2 - kLnWarps;  // 0..7
@@ -398,15 +407,16 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t lane_off = (uint32_t)(q * 32) << 16;
     uint8_t* stg0 = sStg + (size_t)ew * kStgBufs * kStage;
     const int r = q * 32 + lane;  // this thread's row of the tile
-    mbar_wait_warp(w_full, 0, p.status);
+    uint32_t go = lane0_go();
+    mbar_wait_warp(w_full, 0, p.status, go);
     if (ew * 32 + lane < Nh) wsum[ew * 32 + lane] = weight_colsum(sW, Nh, NKB, ew * 32 + lane);
     asm volatile("bar.sync 5, 256;" ::: "memory");  // the eight epilogue warps: column sums written
     int nstore = 0;
     int it = 0;
     for (int t = tile_at(it); t >= 0; t = tile_at(++it)) {
       const int ab = it & 1;
-      mbar_wait_warp(acc_full + ab, (it >> 1) & 1, p.status);
-      mbar_wait_warp(stats_full + ab, (it >> 1) & 1, p.status);
+      mbar_wait_warp(acc_full + ab, (it >> 1) & 1, p.status, go);
+      mbar_wait_warp(stats_full + ab, (it >> 1) & 1, p.status, go);
       tc_fence_after();
       const float2 st = stats[ab * 128 + r];  // rstd, -rstd mu of this thread's row
       const int srow = t * BM + q * 32;
@@ -438,12 +448,12 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) arrive(acc_empty + ab);
+      mbar_arrive_if_at(smem_u32(acc_empty + ab), go == 1);
     }
     if (lane == 0) bulk_wait0();  // output stores complete before the CTA retires
   }
 
-  __syncwarp();  // each warp arrives whole: single lanes ran the producer and MMA loops
+  __syncwarp();
   tc_fence_before();
   __syncthreads();
   if (warp == 0) tmem_dealloc(tmem, 512);

@@ -98,22 +98,21 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int rows_valid = min(p.off[p.B], p.rows);  // off[B]: distinct elements of the batch
   const int tiles = (rows_valid + BM - 1) / BM;
   if ((int)blockIdx.x >= tiles) {
-    if (threadIdx.x == 0) mbar_wait_bounded(w_full, 0, p.status);  // no TMA write may land after the CTA
-    __syncwarp();
+    if (warp == 0) mbar_landed(w_full, 0, p.status);  // no TMA write may land after the CTA
     if (warp == 0) tmem_dealloc(tmem, 128);
     return;
   }
 
   if (warp == 1) {
     // ---------------- MMA issuer (whole warp: fe_common.cuh) ----------------
-    const uint32_t issue = elect_one();
+    const uint32_t go = elect_one();
     const uint32_t idesc = umma_idesc_bf16(BM, d);
     const uint64_t a0 = umma_desc_sw128(smem_u32(sA)), w0 = umma_desc_sw128(smem_u32(sW));
-    mbar_wait_warp(w_full, 0, p.status);
+    const bool w_ok = mbar_wait_ok(w_full, 0, p.status);
     int tl = 0;
-    for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++tl) {
-      if (tl > 0) mbar_wait_warp(acc_empty, (tl - 1) & 1, p.status);
-      mbar_wait_warp(a_full, tl & 1, p.status);
+    for (int t = blockIdx.x; t < tiles && w_ok; t += gridDim.x, ++tl) {
+      if (tl > 0 && !mbar_wait_ok(acc_empty, (tl - 1) & 1, p.status)) break;
+      if (!mbar_wait_ok(a_full, tl & 1, p.status)) break;
       tc_fence_after();
 #pragma unroll
       for (int kb = 0; kb < NKB; ++kb) {
@@ -121,14 +120,16 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int kk = 0; kk < BK / 16; ++kk)
           umma_bf16_if(tmem, desc_adv(a0, (uint32_t)kb * kPlane + kk * 32),
                        desc_adv(w0, (uint32_t)kb * (uint32_t)d * (BK * 2) + kk * 32), idesc, (kb | kk) != 0 ? 1u : 0u,
-                       issue);
+                       go);
       }
-      umma_commit_if(acc_full, issue);
+      umma_commit_if(acc_full, go);
     }
-    umma_drain(drain, p.status, issue);
+    umma_drain(drain, p.status, go);
+    mbar_landed(w_full, 0, p.status);
   } else if (warp >= 2) {
     // ---------------- gather + statistics, then epilogue (warps 2..9) ----------------
     const int gw = warp - 2;
+    uint32_t go = lane0_go();
     // gather: row gr of the tile, lanes l and l ^ 16 share it; of each 64-column
     // k block part 0 takes the first four 16-byte pieces, part 1 the last four
     const int gr = gw * 16 + (lane & 15), part = lane >> 4;
@@ -145,7 +146,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const bool off_staged = p.B < kMaxOff;
     if (off_staged)
       for (int i = gw * 32 + lane; i <= p.B; i += 32 * kGWarps) sOff[i] = p.off[i];
-    mbar_wait_warp(w_full, 0, p.status);
+    mbar_wait_warp(w_full, 0, p.status, go);
     {
       const int i = gw * 32 + lane;
       if (i < d) {
@@ -234,10 +235,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       if (part == 0) stats[gr] = valid ? make_float2(rstd, -mean * rstd) : make_float2(0.f, 0.f);
       fence_async_shared();
-      arrive1(a_full);
+      if (go) arrive1(a_full);  // (every lane arrives)
       gather_sync();  // every row's statistics written
       // ---- epilogue: Q = rstd acc - rstd mu colsum, f16, through the staging blocks
-      mbar_wait_warp(acc_full, tl & 1, p.status);
+      mbar_wait_warp(acc_full, tl & 1, p.status, go);
       tc_fence_after();
       const float2 st = stats[er];
       const int srow = m0 + q * 32;
@@ -266,7 +267,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) arrive1(acc_empty);
+      mbar_arrive_if_at(smem_u32(acc_empty), go == 1);
     }
     if (lane == 0) bulk_wait0();  // Q stores complete before the CTA retires
   }

@@ -86,9 +86,6 @@ __host__ __device__ inline FfnLayout ffn_layout(int d, int d_pad, int F, int nb)
   return L;
 }
 
-__device__ __forceinline__ void mbar_arrive_one(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
 }  // namespace
 
 // NKB: 64-wide k blocks of d (1 or 2); NB: weight planes (1 or 2).  Both are
@@ -196,11 +193,12 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp == 0) {
     // ---------------- TMA producer ----------------
     const uint32_t go = elect_one();
-    int tl = 0, ws = 0, slot = 0;  // tiles, weight slots loaded, the next ring slot
-    uint32_t par = 1;              // the parity of its previous release (a fresh barrier passes)
+    int slot = 0;          // the next ring slot
+    int n_a = 0, n_t = 0;  // A tiles and tail weights requested
+    uint32_t par = 1;      // the parity of its previous release (a fresh barrier passes)
     // kind 0: W_O; 1: W1 rows [f*128, f*128+128); 2: W2 columns [f*128, f*128+128)
-    auto load_slot = [&](int kind, int f) {
-      mbar_wait_warp(w_empty + slot, par, p.status);
+    auto load_slot = [&](int kind, int f) -> bool {
+      if (!mbar_wait_ok(w_empty + slot, par, p.status)) return false;
       uint8_t* dst = sW + (size_t)slot * LY.slot_bytes;
       uint64_t* full = w_full + slot;
       if (kind == 0) {  // every d row, every k block: [kb][plane][d rows x 64]
@@ -219,41 +217,44 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int hh = 0; hh < 2; ++hh)
             tma_load_2d_if(dst + (size_t)(q * 2 + hh) * d * (BK * 2), q ? &tW2_l : &tW2_h, f * FC + BK * hh, 0, full, go);
       }
-      ++ws;
       if (++slot == LY.ring) {
         slot = 0;
         par ^= 1u;
       }
+      return true;
     };
-    for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++tl) {
-      // sA holds the previous tile's output staging until its stores have read it
-      if (tl > 0) mbar_wait_warp(r_empty, (tl - 1) & 1, p.status);
-      mbar_arrive_expect_tx_if(a_full, LY.a_bytes, go);
-      for (int kb = 0; kb < nkb; ++kb) {
-        tma_load_2d_if(sA + (size_t)(kb * 2) * kAPlane, &tA_h, kb * BK, t * BM, a_full, go);
-        tma_load_2d_if(sA + (size_t)(kb * 2 + 1) * kAPlane, &tA_l, kb * BK, t * BM, a_full, go);
+    [&] {
+      for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
+        // sA holds the previous tile's output staging until its stores have read it
+        if (n_a > 0 && !mbar_wait_ok(r_empty, (n_a - 1) & 1, p.status)) return;
+        ++n_a;
+        mbar_arrive_expect_tx_if(a_full, LY.a_bytes, go);
+        for (int kb = 0; kb < nkb; ++kb) {
+          tma_load_2d_if(sA + (size_t)(kb * 2) * kAPlane, &tA_h, kb * BK, t * BM, a_full, go);
+          tma_load_2d_if(sA + (size_t)(kb * 2 + 1) * kAPlane, &tA_l, kb * BK, t * BM, a_full, go);
+        }
+        if (!load_slot(0, 0)) return;
+        for (int s = 0; s < nf + LA; ++s) {
+          if (s < nf && !load_slot(1, s)) return;
+          if (s >= LA && !load_slot(2, s - LA)) return;
+        }
+        if (tail_n > 0) {
+          // the tail weight, past the x_out staging, once every FFN MMA of the
+          // tile (the last readers of the ring) has completed
+          if (!mbar_wait_ok(acc2_full, n_t & 1, p.status)) return;
+          ++n_t;
+          mbar_arrive_expect_tx_if(wt_full, (uint32_t)nkb * nb * (uint32_t)tail_n * (BK * 2), go);
+          for (int kb = 0; kb < nkb; ++kb)
+            for (int q = 0; q < nb; ++q)
+              tma_load_2d_if(sT + (size_t)(kb * nb + q) * tail_n * (BK * 2), q ? &tT_l : &tT_h, kb * BK, 0, wt_full, go);
+        }
       }
-      load_slot(0, 0);
-      for (int s = 0; s < nf + LA; ++s) {
-        if (s < nf) load_slot(1, s);
-        if (s >= LA) load_slot(2, s - LA);
-      }
-      if (tail_n > 0) {
-        // the tail weight, past the x_out staging, once every FFN MMA of the
-        // tile (the last readers of the ring) has completed
-        mbar_wait_warp(acc2_full, tl & 1, p.status);
-        mbar_arrive_expect_tx_if(wt_full, (uint32_t)nkb * nb * (uint32_t)tail_n * (BK * 2), go);
-        for (int kb = 0; kb < nkb; ++kb)
-          for (int q = 0; q < nb; ++q)
-            tma_load_2d_if(sT + (size_t)(kb * nb + q) * tail_n * (BK * 2), q ? &tT_l : &tT_h, kb * BK, 0, wt_full, go);
-      }
-    }
+    }();
     // the last loads land before this block's shared memory goes away (after a
     // timed-out wait nothing else has waited for them)
-    for (int i = ws < LY.ring ? 0 : ws - LY.ring; i < ws; ++i)
-      mbar_wait_warp(w_full + i % LY.ring, (uint32_t)(i / LY.ring) & 1u, p.status);
-    if (tl > 0) mbar_wait_warp(a_full, (tl - 1) & 1, p.status);
-    if (tl > 0 && tail_n > 0) mbar_wait_warp(wt_full, (tl - 1) & 1, p.status);
+    mbar_landed_ring(w_full, slot, par, LY.ring, p.status);
+    mbar_landed(a_full, (n_a & 1) ^ 1, p.status);
+    if (tail_n > 0) mbar_landed(wt_full, (n_t & 1) ^ 1, p.status);
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
     const uint32_t go = elect_one();
@@ -263,12 +264,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint64_t w00 = umma_desc_sw128(smem_u32(sW));
     int tl = 0, gf = 0, slot = 0;
     uint32_t par = 0;
-    // the next weight slot landed: its descriptor
-    auto next_slot = [&]() -> uint64_t {
-      mbar_wait_warp(w_full + slot, par, p.status);
+    auto wait = [&](uint64_t* bar, uint32_t parity) -> bool {
+      const bool ok = mbar_wait_ok(bar, parity, p.status);
       tc_fence_after();
-      return desc_adv(w00, (uint32_t)slot * LY.slot_bytes);
+      return ok;
     };
+    // the next weight slot's descriptor
+    auto slot_desc = [&]() -> uint64_t { return desc_adv(w00, (uint32_t)slot * LY.slot_bytes); };
     // the slot frees once the products issued so far complete
     auto release = [&]() {
       umma_commit_if(w_empty + slot, go);
@@ -277,101 +279,103 @@ __global__ void __launch_bounds__(kThreads, 1)
         par ^= 1u;
       }
     };
-    for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++tl) {
-      // ---- A W_O into the FFN1 buffer that chunk 0 of this tile uses next
-      mbar_wait_warp(a_full, tl & 1, p.status);
-      {
-        const int bo = gf % NA1;
-        const uint64_t w0 = next_slot();
-        if (gf >= NA1) mbar_wait_warp(acc1_empty + bo, ((gf / NA1) - 1) & 1, p.status);
-        tc_fence_after();
-        const uint32_t dst = tmem + (uint32_t)(bo * FC);
-#pragma unroll
-        for (int kb = 0; kb < nkb; ++kb) {
-#pragma unroll
-          for (int kk = 0; kk < BK / 16; ++kk) {
-            const uint64_t ah = desc_adv(a0, (uint32_t)(kb * 2) * kAPlane + kk * 32);
-            const uint64_t wh = desc_adv(w0, (uint32_t)(kb * nb) * (uint32_t)d * (BK * 2) + kk * 32);
-            umma_bf16_if(dst, ah, wh, idesc2, (kb | kk) != 0 ? 1u : 0u, go);
-            umma_bf16_if(dst, desc_adv(ah, kAPlane), wh, idesc2, 1u, go);
-            if (nb > 1) umma_bf16_if(dst, ah, desc_adv(wh, (uint32_t)d * (BK * 2)), idesc2, 1u, go);
-          }
-        }
-        release();
-        umma_commit_if(o_done, go);
-      }
-      // ---- FFN1 / FFN2 once the epilogue has put x in the accumulator and LN(x) in sA
-      mbar_wait_warp(ln_full, tl & 1, p.status);
-      tc_fence_after();
-      const int gf0 = gf;
-      for (int s = 0; s < nf + LA; ++s) {
-        if (s < nf) {
-          // FFN1 chunk s -> acc1 buffer (gf0 + s) % NA1
-          const int g = gf0 + s, b = g % NA1;
-          // (chunk 0's buffer: waited for before the projection, read by the epilogue before ln_full)
-          if (s > 0 && g >= NA1) mbar_wait_warp(acc1_empty + b, ((g / NA1) - 1) & 1, p.status);
-          const uint64_t w0 = next_slot();
-          const uint32_t dst = tmem + (uint32_t)(b * FC);
+    [&] {
+      for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++tl) {
+        // ---- A W_O into the FFN1 buffer that chunk 0 of this tile uses next
+        if (!wait(a_full, tl & 1)) return;
+        {
+          const int bo = gf % NA1;
+          if (!wait(w_full + slot, par)) return;
+          const uint64_t w0 = slot_desc();
+          if (gf >= NA1 && !wait(acc1_empty + bo, ((gf / NA1) - 1) & 1)) return;
+          const uint32_t dst = tmem + (uint32_t)(bo * FC);
 #pragma unroll
           for (int kb = 0; kb < nkb; ++kb) {
 #pragma unroll
             for (int kk = 0; kk < BK / 16; ++kk) {
               const uint64_t ah = desc_adv(a0, (uint32_t)(kb * 2) * kAPlane + kk * 32);
-              const uint64_t wh = desc_adv(w0, (uint32_t)(kb * nb) * (FC * BK * 2) + kk * 32);
-              umma_bf16_if(dst, ah, wh, idesc1, (kb | kk) != 0 ? 1u : 0u, go);
-              umma_bf16_if(dst, desc_adv(ah, kAPlane), wh, idesc1, 1u, go);
-              if (nb > 1) umma_bf16_if(dst, ah, desc_adv(wh, FC * BK * 2), idesc1, 1u, go);
+              const uint64_t wh = desc_adv(w0, (uint32_t)(kb * nb) * (uint32_t)d * (BK * 2) + kk * 32);
+              umma_bf16_if(dst, ah, wh, idesc2, (kb | kk) != 0 ? 1u : 0u, go);
+              umma_bf16_if(dst, desc_adv(ah, kAPlane), wh, idesc2, 1u, go);
+              if (nb > 1) umma_bf16_if(dst, ah, desc_adv(wh, (uint32_t)d * (BK * 2)), idesc2, 1u, go);
             }
           }
           release();
-          umma_commit_if(acc1_full + b, go);
+          umma_commit_if(o_done, go);
         }
-        if (s >= LA) {
-          // FFN2 chunk c = s - LA: acc2 += mid(c) . W2 chunk c, mid(c) from TMEM buffer g % NA1
-          const int c = s - LA, g = gf0 + c, b = g % NA1;
-          mbar_wait_warp(mid_full + b, (g / NA1) & 1, p.status);
-          const uint64_t w0 = next_slot();
-          // each 32-column piece of the buffer holds 32 hidden units: hi plane in
-          // its first 16 columns, lo plane in the next 16 (two bf16 per column);
-          // the W2 slot holds 64-column halves of the chunk, d rows each
-          const uint32_t mt = tmem + (uint32_t)(b * FC);
+        // ---- FFN1 / FFN2 once the epilogue has put x in the accumulator and LN(x) in sA
+        if (!wait(ln_full, tl & 1)) return;
+        const int gf0 = gf;
+        for (int s = 0; s < nf + LA; ++s) {
+          if (s < nf) {
+            // FFN1 chunk s -> acc1 buffer (gf0 + s) % NA1
+            const int g = gf0 + s, b = g % NA1;
+            // (chunk 0's buffer: waited for before the projection, read by the epilogue before ln_full)
+            if (s > 0 && g >= NA1 && !wait(acc1_empty + b, ((g / NA1) - 1) & 1)) return;
+            if (!wait(w_full + slot, par)) return;
+            const uint64_t w0 = slot_desc();
+            const uint32_t dst = tmem + (uint32_t)(b * FC);
 #pragma unroll
-          for (int kk = 0; kk < FC / 16; ++kk) {
-            const int hh = kk >> 2, k4 = kk & 3;
-            const uint32_t mh = mt + (uint32_t)(32 * (kk >> 1) + 8 * (kk & 1)), ml = mh + 16;
-            const uint64_t wh = desc_adv(w0, (uint32_t)hh * (uint32_t)d * (BK * 2) + k4 * 32);
-            umma_bf16_tmem_a_if(acc2, mh, wh, idesc2, 1u, go);
-            umma_bf16_tmem_a_if(acc2, ml, wh, idesc2, 1u, go);
-            if (nb > 1) umma_bf16_tmem_a_if(acc2, mh, desc_adv(wh, 2u * (uint32_t)d * (BK * 2)), idesc2, 1u, go);
+            for (int kb = 0; kb < nkb; ++kb) {
+#pragma unroll
+              for (int kk = 0; kk < BK / 16; ++kk) {
+                const uint64_t ah = desc_adv(a0, (uint32_t)(kb * 2) * kAPlane + kk * 32);
+                const uint64_t wh = desc_adv(w0, (uint32_t)(kb * nb) * (FC * BK * 2) + kk * 32);
+                umma_bf16_if(dst, ah, wh, idesc1, (kb | kk) != 0 ? 1u : 0u, go);
+                umma_bf16_if(dst, desc_adv(ah, kAPlane), wh, idesc1, 1u, go);
+                if (nb > 1) umma_bf16_if(dst, ah, desc_adv(wh, FC * BK * 2), idesc1, 1u, go);
+              }
+            }
+            release();
+            umma_commit_if(acc1_full + b, go);
           }
-          release();
-          umma_commit_if(acc1_empty + b, go);
-          if (c == nf - 1) umma_commit_if(acc2_full, go);
+          if (s >= LA) {
+            // FFN2 chunk c = s - LA: acc2 += mid(c) . W2 chunk c, mid(c) from TMEM buffer g % NA1
+            const int c = s - LA, g = gf0 + c, b = g % NA1;
+            if (!wait(mid_full + b, (g / NA1) & 1)) return;
+            if (!wait(w_full + slot, par)) return;
+            const uint64_t w0 = slot_desc();
+            // each 32-column piece of the buffer holds 32 hidden units: hi plane in
+            // its first 16 columns, lo plane in the next 16 (two bf16 per column);
+            // the W2 slot holds 64-column halves of the chunk, d rows each
+            const uint32_t mt = tmem + (uint32_t)(b * FC);
+#pragma unroll
+            for (int kk = 0; kk < FC / 16; ++kk) {
+              const int hh = kk >> 2, k4 = kk & 3;
+              const uint32_t mh = mt + (uint32_t)(32 * (kk >> 1) + 8 * (kk & 1)), ml = mh + 16;
+              const uint64_t wh = desc_adv(w0, (uint32_t)hh * (uint32_t)d * (BK * 2) + k4 * 32);
+              umma_bf16_tmem_a_if(acc2, mh, wh, idesc2, 1u, go);
+              umma_bf16_tmem_a_if(acc2, ml, wh, idesc2, 1u, go);
+              if (nb > 1) umma_bf16_tmem_a_if(acc2, mh, desc_adv(wh, 2u * (uint32_t)d * (BK * 2)), idesc2, 1u, go);
+            }
+            release();
+            umma_commit_if(acc1_empty + b, go);
+            if (c == nf - 1) umma_commit_if(acc2_full, go);
+          }
+        }
+        gf = gf0 + nf;
+        if (tail_n > 0) {
+          // tail: LN(x_out) . W_t into TMEM columns [0, tail_n) (every FFN1
+          // buffer is free once the FFN2 of the tile has completed)
+          if (!wait(tail_a, tl & 1)) return;
+          if (!wait(wt_full, tl & 1)) return;
+          const uint32_t idesc3 = umma_idesc_bf16(BM, tail_n);
+          const uint64_t w0 = umma_desc_sw128(smem_u32(sT));
+#pragma unroll
+          for (int kb = 0; kb < nkb; ++kb) {
+#pragma unroll
+            for (int kk = 0; kk < BK / 16; ++kk) {
+              const uint64_t ah = desc_adv(a0, (uint32_t)(kb * 2) * kAPlane + kk * 32);
+              const uint64_t wh = desc_adv(w0, (uint32_t)(kb * nb) * (uint32_t)tail_n * (BK * 2) + kk * 32);
+              umma_bf16_if(tmem, ah, wh, idesc3, (kb | kk) != 0 ? 1u : 0u, go);
+              umma_bf16_if(tmem, desc_adv(ah, kAPlane), wh, idesc3, 1u, go);
+              if (nb > 1) umma_bf16_if(tmem, ah, desc_adv(wh, (uint32_t)tail_n * (BK * 2)), idesc3, 1u, go);
+            }
+          }
+          umma_commit_if(tail_full, go);
         }
       }
-      gf = gf0 + nf;
-      if (tail_n > 0) {
-        // tail: LN(x_out) . W_t into TMEM columns [0, tail_n) (every FFN1
-        // buffer is free once the FFN2 of the tile has completed)
-        mbar_wait_warp(tail_a, tl & 1, p.status);
-        mbar_wait_warp(wt_full, tl & 1, p.status);
-        tc_fence_after();
-        const uint32_t idesc3 = umma_idesc_bf16(BM, tail_n);
-        const uint64_t w0 = umma_desc_sw128(smem_u32(sT));
-#pragma unroll
-        for (int kb = 0; kb < nkb; ++kb) {
-#pragma unroll
-          for (int kk = 0; kk < BK / 16; ++kk) {
-            const uint64_t ah = desc_adv(a0, (uint32_t)(kb * 2) * kAPlane + kk * 32);
-            const uint64_t wh = desc_adv(w0, (uint32_t)(kb * nb) * (uint32_t)tail_n * (BK * 2) + kk * 32);
-            umma_bf16_if(tmem, ah, wh, idesc3, (kb | kk) != 0 ? 1u : 0u, go);
-            umma_bf16_if(tmem, desc_adv(ah, kAPlane), wh, idesc3, 1u, go);
-            if (nb > 1) umma_bf16_if(tmem, ah, desc_adv(wh, (uint32_t)tail_n * (BK * 2)), idesc3, 1u, go);
-          }
-        }
-        umma_commit_if(tail_full, go);
-      }
-    }
+    }();
     umma_drain(drain, p.status, go);
   } else {
     // ---------------- epilogue (warps 2..9) ----------------
@@ -398,10 +402,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       __syncwarp();
     };
     // one arrival per warp on barriers counted in warps (the lanes synchronise first)
-    auto warp_arrive = [&](uint64_t* bar) {
-      __syncwarp();
-      if (lane == 0) mbar_arrive_one(bar);
-    };
+    uint32_t go = lane0_go();
+    auto warp_arrive = [&](uint64_t* bar) { mbar_arrive_warp(bar, go); };
     int tl = 0, gf = 0;
     for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++tl) {
       const int m0 = t * BM;
@@ -434,7 +436,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       tmem_st_wait();
       const uint32_t proj = tmem + (uint32_t)((gf % NA1) * FC);  // A W_O
-      mbar_wait_warp(o_done, tl & 1, p.status);
+      mbar_wait_warp(o_done, tl & 1, p.status, go);
       tc_fence_after();
       RowSum sum, var;
 #pragma unroll 1
@@ -502,7 +504,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // warp's 64 columns of the chunk's TMEM buffer as FFN2's A operand
       for (int f = 0; f < nf; ++f, ++gf) {
         const int ba = gf % NA1;
-        mbar_wait_warp(acc1_full + ba, (gf / NA1) & 1, p.status);
+        mbar_wait_warp(acc1_full + ba, (gf / NA1) & 1, p.status, go);
         tc_fence_after();
         // this warp's 64 columns as two 32-column pieces, each read whole and
         // then overwritten by its own hi (16 columns) and lo (16 columns) planes
@@ -528,7 +530,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         warp_arrive(mid_full + ba);
       }
       // ---- final: x_out = acc2 + b2 (acc2 = x + FFN2), LayerNorm, stores
-      mbar_wait_warp(acc2_full, tl & 1, p.status);
+      mbar_wait_warp(acc2_full, tl & 1, p.status, go);
       tc_fence_after();
       // this warp's x_out staging blocks at the start of the weight ring (every
       // MMA of the tile has completed, and before r_empty the producer loads
@@ -629,7 +631,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         // tail output: 32-column chunks half, half + 2, ... of this warp's row
         // quadrant, f16 (one 2 KB block) or a split pair (two), through two
         // rotating staging buffers of this warp where the tail weight was
-        mbar_wait_warp(tail_full, tl & 1, p.status);
+        mbar_wait_warp(tail_full, tl & 1, p.status, go);
         tc_fence_after();
         const uint32_t tb = p.tail_f16 ? 2048u : 4096u;
         uint8_t* stg = sT + (size_t)ew * 2u * tb;
@@ -676,7 +678,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         tc_fence_before();  // TMEM read before r_empty lets the next tile's projection in
       }
       stores_read();
-      if (lane == 0) mbar_arrive_one(r_empty);  // sA and the ring may take the next tile's loads
+      mbar_arrive_if_at(smem_u32(r_empty), go == 1);  // sA and the ring may take the next tile's loads
     }
     if (lane == 0) bulk_wait0();  // output tensor stores complete before the CTA retires
   }

@@ -231,16 +231,15 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp == 0) {
     // ---------------- TMA producer ----------------
     const uint32_t go = elect_one();
-    int ws = 0, slot = 0, tl = 0;
+    int slot = 0, tl = 0;
     uint32_t par = 1;  // the parity of the slot's previous release (a fresh barrier passes)
     // every CTA re-reads the same weight boxes while the activation tiles
     // stream past once: keep the weights in L2, let the activations go first
     const uint64_t keep = l2_policy_evict_last(), pass = l2_policy_evict_first();
     auto load = [&](const CUtensorMap* m, int x, int y) {
-      mbar_wait_warp(w_empty + slot, par, p.status);
+      mbar_wait_load(w_empty + slot, w_full + slot, par, p.status);
       mbar_arrive_expect_tx_if(w_full + slot, kBox, go);
       tma_load_2d_hint_if(sR + (size_t)slot * kBox, m, x, y, w_full + slot, keep, go);
-      ++ws;
       if (++slot == kRing) {
         slot = 0;
         par ^= 1u;
@@ -252,7 +251,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int i = 0; i < 2 * NKB; ++i) {
         if (i == kRing - 1) {
           for (int kb = 0; kb < NKB; ++kb) {
-            if (tl > 0) mbar_wait_warp(a_free + kb, (tl - 1) & 1, p.status);
+            if (tl > 0) mbar_wait_load(a_free + kb, a_full + kb, (tl - 1) & 1, p.status);
             mbar_arrive_expect_tx_if(a_full + kb, 2 * kBox, go);
             tma_load_2d_hint_if(sA + (size_t)(kb * 2) * kBox, &tA_h, kb * BK, t * BM, a_full + kb, pass, go);
             tma_load_2d_hint_if(sA + (size_t)(kb * 2 + 1) * kBox, &tA_l, kb * BK, t * BM, a_full + kb, pass, go);
@@ -281,10 +280,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     // the last loads land before this block's shared memory goes away (after a
     // timed-out wait nothing else has waited for them)
-    for (int i = ws < kRing ? 0 : ws - kRing; i < ws; ++i)
-      mbar_wait_warp(w_full + i % kRing, (uint32_t)(i / kRing) & 1u, p.status);
-    if (tl > 0)
-      for (int kb = 0; kb < NKB; ++kb) mbar_wait_warp(a_full + kb, (tl - 1) & 1, p.status);
+    mbar_landed_ring(w_full, slot, par, kRing, p.status);
+    mbar_landed_ring(a_full, 0, (tl & 1) ^ 1, NKB, p.status);
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
     const uint32_t go = elect_one();
@@ -292,7 +289,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     int slot = 0, tl = 0, gf = 0;
     uint32_t par = 0;
     auto wait = [&](uint64_t* bar, uint32_t parity) {
-      mbar_wait_warp(bar, parity, p.status);
+      mbar_wait_role(bar, parity, p.status);
       tc_fence_after();
     };
     // the next weight box landed: its shared-memory address
@@ -389,7 +386,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       __syncwarp();
       if (lane == 0) arrive_one(bar);
     };
-    auto wait = [&](uint64_t* bar, uint32_t par) { mbar_wait_warp(bar, par, p.status); };
+    auto wait = [&](uint64_t* bar, uint32_t par) { mbar_wait_role(bar, par, p.status); };
     // the row statistics over both halves: sum -> mean, then sum of squares -> rstd
     auto pair_mean = [&](float s) {
       red_sum[hf * 128 + r] = s;

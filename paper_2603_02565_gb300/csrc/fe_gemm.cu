@@ -85,10 +85,6 @@ int gemm_max_stages(int BN, int nb, int K_pad, int cs, int na) {
   return s < 1 ? 1 : s;
 }
 
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
 // ---- thread-block cluster helpers (the RESID_LN row exchange) ----
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
@@ -112,30 +108,6 @@ __device__ __forceinline__ void st_async_peer(uint32_t addr, float v, uint32_t b
                "r"(__float_as_uint(v)), "r"(bar)
                : "memory");
 }
-__device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// bounded like mbar_wait_bounded, acquiring at cluster scope (the peers' stores)
-__device__ __noinline__ void mbar_wait_cluster(uint64_t* bar, uint32_t parity, int* status) {
-  const uint64_t t0 = globaltimer_ns();
-  for (uint32_t it = 0;; ++it) {
-    if (mbar_try_wait_cluster(bar, parity)) return;
-    if ((it & 255u) == 255u && (*reinterpret_cast<volatile int*>(status) & ST_TIMEOUT)) return;
-    if (globaltimer_ns() - t0 > kWaitLimitNs) {
-      atomicOr(status, ST_TIMEOUT);
-      return;
-    }
-  }
-}
-
 // NB: weight planes (1 when the weights are exact in bf16, else 2); a
 // compile-time constant so that the MMA issue sequence has no branches
 template <int EPI, int NB>
@@ -222,12 +194,13 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp == 0) {
     // ---------------- TMA producer ----------------
     const uint32_t go = elect_one();
-    int it = 0, st_i = 0;  // k blocks loaded, the next stage
-    uint32_t par = 1;      // the parity of its previous release (a fresh barrier passes)
-    for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
+    int st_i = 0;      // the next stage
+    uint32_t par = 1;  // the parity of its previous release (a fresh barrier passes)
+    bool ok = true;
+    for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
       const int m0 = (t / nt) * BM, n0 = (t % nt) * BN;
-      for (int kb = 0; kb < nk; ++kb, ++it) {
-        mbar_wait_warp(empty + st_i, par, p.status);
+      for (int kb = 0; kb < nk; ++kb) {
+        if (!(ok = mbar_wait_ok(empty + st_i, par, p.status))) break;
         uint8_t* st = smem + (size_t)st_i * stage_bytes;
         mbar_arrive_expect_tx_if(full + st_i, stage_bytes, go);
         tma_load_2d_if(st, &tA_h, kb * BK, m0, full + st_i, go);
@@ -245,7 +218,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     // the last loads land before this block's shared memory goes away (after a
     // timed-out wait nothing else has waited for them)
-    for (int i = it < S ? 0 : it - S; i < it; ++i) mbar_wait_warp(full + i % S, (uint32_t)(i / S) & 1u, p.status);
+    mbar_landed_ring(full, st_i, par, S, p.status);
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
     const uint32_t go = elect_one();
@@ -254,12 +227,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint64_t sd0 = umma_desc_sw128(smem_u32(smem));
     int tl = 0, st_i = 0;
     uint32_t par = 0;
-    for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++tl) {
+    bool ok = true;
+    for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++tl) {
       const int acc = tl % nacc, use = tl / nacc;
-      if (use > 0) mbar_wait_warp(tempty + acc, (use - 1) & 1, p.status);
+      if (use > 0 && !mbar_wait_ok(tempty + acc, (use - 1) & 1, p.status)) break;
       const uint32_t dst = tmem + (uint32_t)(acc * BN);
       for (int kb = 0; kb < nk; ++kb) {
-        mbar_wait_warp(full + st_i, par, p.status);
+        if (!(ok = mbar_wait_ok(full + st_i, par, p.status))) break;
         tc_fence_after();
         // descriptors built once per stage; the k steps only add 32-byte offsets
         const uint64_t ah0 = desc_adv(sd0, (uint32_t)st_i * stage_bytes), al0 = desc_adv(ah0, kATile);
@@ -282,7 +256,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           par ^= 1u;
         }
       }
-      umma_commit_if(tfull + acc, go);  // accumulator complete
+      if (ok) umma_commit_if(tfull + acc, go);  // accumulator complete
     }
     umma_drain(drain, p.status, go);
   } else {
@@ -291,6 +265,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int q = warp & 3;      // TMEM lane quadrant this warp may access
     const int half = ew >> 2;    // which alternate 32-column chunks
     const int r = q * 32 + lane;
+    uint32_t go = lane0_go();
     uint8_t* stg0 = stg_base + (size_t)ew * 2 * kStageOut;
     int nstore = 0;              // bulk-store groups issued by this warp (selects the staging buffer)
     // the two warps of a lane quadrant meet at named barrier 1 + q (64 threads)
@@ -343,15 +318,16 @@ __global__ void __launch_bounds__(kThreads, 1)
       float* xs = red + (size_t)kind * cs * 256;
       const uint32_t slot = smem_u32(xs + (my_rank * 2 + half) * 128 + r);
       const uint32_t bar = smem_u32(xbar + kind);
-      for (int k = 0; k < cs; ++k) st_async_peer(map_peer(slot, (uint32_t)k), v, map_peer(bar, (uint32_t)k));
-      if (ew == 0 && lane == 0) mbar_arrive_expect_tx(xbar + kind, (uint32_t)cs * 1024u);
-      mbar_wait_cluster(xbar + kind, (uint32_t)tl & 1u, p.status);
-      __syncwarp();
+      if (go)
+        for (int k = 0; k < cs; ++k) st_async_peer(map_peer(slot, (uint32_t)k), v, map_peer(bar, (uint32_t)k));
+      if (ew == 0 && go == 1) mbar_arrive_expect_tx(xbar + kind, (uint32_t)cs * 1024u);
+      mbar_wait_cluster(xbar + kind, (uint32_t)tl & 1u, p.status, go);
       float a = 0.f;
       for (int k = 0; k < cs; ++k) a += xs[(2 * k) * 128 + r] + xs[(2 * k + 1) * 128 + r];
       tot = a;
     };
 
+    uint32_t rpar = 1;  // the parity of the newest residual tile requested (a fresh barrier passes)
     float xr[64];  // EPI_RESID_LN with BN <= 128: this warp's chunks of the row
     for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++tl) {
       const int acc = tl % nacc, use = tl / nacc;
@@ -362,7 +338,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (EPI == EPI_RESID_LN && p.ldr) {
         // residual rows, loaded while the MMAs of this tile run: this warp's blocks (at most
         // two) into its staging buffers, whose last stores have read them
-        if (lane == 0) {
+        if (go == 1) {
+          rpar ^= 1u;
           bulk_wait_read0();
           mbar_arrive_expect_tx(rbar + ew, (uint32_t)((BN - 32 * half + 63) / 64) * kStageOut);
           for (int ci = 0, c = 32 * half; c < BN; ++ci, c += 64)
@@ -370,7 +347,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         __syncwarp();
       }
-      mbar_wait_warp(tfull + acc, use & 1, p.status);
+      mbar_wait_warp(tfull + acc, use & 1, p.status, go);
       tc_fence_after();
       const uint32_t trow = tmem + (uint32_t)(acc * BN) + ((uint32_t)(q * 32) << 16);
       float* red_sum = red + (size_t)(tl & 1) * 512;  // [half][128]
@@ -434,7 +411,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         // x = resid + acc + bias in registers; the residual was loaded before the
         // accumulator was ready, TMEM is read once
         // (one row broadcast to every row is read where it lies)
-        if (p.ldr) mbar_wait_warp(rbar + ew, (uint32_t)tl & 1u, p.status);
+        if (p.ldr) mbar_wait_warp(rbar + ew, (uint32_t)tl & 1u, p.status, go);
         const int sw = p.ldr ? lane & 7 : 0;
         float sum = 0.f;
 #pragma unroll
@@ -668,9 +645,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       // every TMEM read of this accumulator has completed (tcgen05.wait::ld)
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(tempty + acc);
+      mbar_arrive_if_at(smem_u32(tempty + acc), go == 1);
     }
     if (lane == 0) bulk_wait0();  // output tensor stores complete before the CTA retires
+    if (EPI == EPI_RESID_LN) mbar_landed(rbar + ew, __shfl_sync(0xffffffffu, rpar, 0), p.status);
   }
 
   __syncwarp();

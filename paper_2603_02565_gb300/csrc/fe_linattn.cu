@@ -89,7 +89,8 @@ __global__ void __launch_bounds__(256, 2) lin_state_kernel(const __half* __restr
   extern __shared__ __align__(1024) uint8_t sm_state[];
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm_state + 2 * Cfg::kBuf);
   uint64_t* free_bar = bars;                // [2] the products of the chunk in this buffer are complete
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2);
+  uint64_t* drain = bars + 2;               // the products in flight at the end
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 3);
   const int s = blockIdx.x, G = d / FG, l = blockIdx.y / G, g = blockIdx.y % G;
   const int kcol = 2 * l * d + g * FG, vcol = (2 * l + 1) * d + g * FG;
   const size_t row0 = (size_t)s * C;
@@ -105,6 +106,7 @@ __global__ void __launch_bounds__(256, 2) lin_state_kernel(const __half* __restr
   if (t == 0) {
     mbar_init(free_bar, 1);
     mbar_init(free_bar + 1, 1);
+    mbar_init(drain, 1);
     fence_mbar_init();
   }
   if (warp == 0) tmem_alloc(tmem_slot, Cfg::kCols);
@@ -145,7 +147,7 @@ __global__ void __launch_bounds__(256, 2) lin_state_kernel(const __half* __restr
     constexpr int B = decltype(bufc)::value;
     const int r0 = it * kChunk;
     uint8_t* buf = sm_state + (size_t)B * Cfg::kBuf;
-    if (it >= 2) mbar_wait_warp(free_bar + B, ((it >> 1) - 1) & 1, status);
+    if (it >= 2) mbar_wait_role(free_bar + B, ((it >> 1) - 1) & 1, status);
 #pragma unroll
     for (int q = 0; q < P8; ++q) {
       const int idx = t + 256 * q, r = idx / (FG / 8), c8 = (idx % (FG / 8)) * 8;
@@ -194,7 +196,7 @@ __global__ void __launch_bounds__(256, 2) lin_state_kernel(const __half* __restr
     if (i + 1 < it_end) chunk(std::integral_constant<int, 1>{}, i + 1, k1, v1);
   }
   // the last product (and so every earlier one) complete
-  mbar_wait_warp(free_bar + ((it_end - 1) & 1), ((it_end - 1) >> 1) & 1, status);
+  mbar_wait_role(free_bar + ((it_end - 1) & 1), ((it_end - 1) >> 1) & 1, status);
   tc_fence_after();
   // lane m of the accumulator: feature m of the group; its head's DH columns, and z in column FG
   const int q = warp & 3, sub = warp >> 2, m = 32 * q + lane;
@@ -228,6 +230,7 @@ __global__ void __launch_bounds__(256, 2) lin_state_kernel(const __half* __restr
       st[DH * DH + i] = __uint_as_float(z[0]) + __uint_as_float(w[0]) + (odd ? __uint_as_float(u[0]) : 0.f);
     }
   }
+  if (warp == 0) umma_drain(drain, status, go);
   tc_fence_before();
   __syncthreads();
   if (warp == 0) tmem_dealloc(tmem, Cfg::kCols);

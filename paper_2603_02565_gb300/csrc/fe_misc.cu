@@ -838,21 +838,53 @@ cudaError_t small_matmul_launch(const float* X, int R, int Kd, const float* W, i
   return cudaGetLastError();
 }
 
-// A bounded wait that nothing completes: one thread initialises an mbarrier
-// with an arrival count of one, never arrives on it and waits for its first
-// phase through the batch kernels' bounded wait, with a limit of limit_ns.
-// No copy and no tensor-core work is in flight, so giving up is always safe.
-// Launched only by the wait test hook (fe_debug_wait_probe).
-__global__ void wait_probe_kernel(int* status, uint64_t limit_ns) {
-  __shared__ __align__(8) uint64_t bar;
-  if (threadIdx.x != 0) return;
-  mbar_init(&bar, 1);
-  fence_mbar_init();
-  mbar_wait_bounded_ns(&bar, 0, status, limit_ns);
+// The bounded waits on a barrier that nothing arrives on, with no copy and no
+// tensor-core work in flight: each form of the batch kernels' waits in two warps.
+// One gives up by the limit, the other, whose limit is a hundred times as long,
+// because the first has set the status word they share.  Then each goes on as its role
+// would, for seven more waits: none of them may take long, and an epilogue warp's
+// arrivals after them must not reach its barrier.  The last warp waits for a load that
+// never lands, which only the limit ends.
+// Launched only by the wait test hook (fe_debug_wait_probe): ST_TIMEOUT when every
+// warp behaved so, else ST_NUMERIC.
+constexpr int kWaitForms = 5;
+__global__ void __launch_bounds__(64 * kWaitForms + 32) wait_probe_kernel(int* status, uint32_t limit_us) {
+  __shared__ __align__(8) uint64_t never, hits[2 * kWaitForms];
+  __shared__ int st[kWaitForms + 1];
+  const int warp = threadIdx.x >> 5, form = warp < 2 * kWaitForms ? warp % kWaitForms : kWaitForms;
+  if (threadIdx.x <= kWaitForms) st[threadIdx.x] = threadIdx.x < kWaitForms ? 0 : ST_TIMEOUT;
+  if (threadIdx.x == 0) {
+    mbar_init(&never, 1);
+    for (int i = 0; i < 2 * kWaitForms; ++i) mbar_init(hits + i, 1);
+    fence_mbar_init();
+  }
+  __syncthreads();
+  const uint32_t limit = warp < kWaitForms || form == kWaitForms ? limit_us : 100u * limit_us;
+  uint32_t go = lane0_go();
+  bool ok = true;
+  const uint64_t t0 = globaltimer_ns();
+  if (form == kWaitForms) {
+    mbar_landed(&never, 0, st + form, limit);
+  } else {
+    for (int i = 0; i < 8; ++i) {
+      if (form == 0) mbar_wait_role(&never, 0, st, limit);
+      if (form == 1) mbar_wait_at(smem_u32(&never), 0, st + 1, limit);
+      if (form == 2) mbar_wait_warp(&never, 0, st + 2, go, limit);
+      if (form == 3) mbar_wait_cluster(&never, 0, st + 3, go, limit);
+      if (form == 4) ok = ok && !mbar_wait_ok(&never, 0, st + 4, limit);
+      if (form == 2 || form == 3) mbar_arrive_warp(hits + warp, go);
+    }
+    if (form == 2 || form == 3) ok = go == 0 && !mbar_try_wait(hits + warp, 0);
+  }
+  // the limit once (the timer of mbar_wait_at ticks in 65.5 us) and seven times a few polls of 4 us
+  const long long us = (long long)((globaltimer_ns() - t0) / 1000u), want = limit_us;
+  ok = ok && us >= want - 140 && us <= 2 * want + 4000;
+  const int all = __syncthreads_and(ok);
+  if (threadIdx.x == 0) atomicOr(status, all ? ST_TIMEOUT : ST_NUMERIC);
 }
 
-cudaError_t wait_probe_launch(int* status, uint64_t limit_ns, cudaStream_t s) {
-  wait_probe_kernel<<<1, 32, 0, s>>>(status, limit_ns);
+cudaError_t wait_probe_launch(int* status, uint32_t limit_us, cudaStream_t s) {
+  wait_probe_kernel<<<1, 64 * kWaitForms + 32, 0, s>>>(status, limit_us);
   return cudaGetLastError();
 }
 

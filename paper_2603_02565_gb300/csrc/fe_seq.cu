@@ -463,19 +463,18 @@ __global__ void __launch_bounds__(kThreads, 1)
     // chunk s - LA interleaved, then WQx, WKx, WVx, WOx (with the cross-sequence
     // block), then W1h; two 64-column boxes each.
     const uint32_t go = elect_one();
-    int ws = 0, slot = 0, tl = 0;
+    int slot = 0, tl = 0;
     uint32_t par = 1;       // the parity of the slot's previous release (a fresh barrier passes)
     bool gathered = false;  // the tile's gathers are done: the staging slots are weight slots again
     auto load = [&](const CUtensorMap* m, int x, int y) {
       for (int box = 0; box < 2; ++box) {
         if (slot >= kStageSlot && !gathered) {
-          mbar_wait_warp(a_full, tl & 1, p.sel.status);
+          mbar_wait_role(a_full, tl & 1, p.sel.status);
           gathered = true;
         }
-        mbar_wait_warp(w_empty + slot, par, p.sel.status);
+        mbar_wait_load(w_empty + slot, w_full + slot, par, p.sel.status);
         mbar_arrive_expect_tx_if(w_full + slot, kBox, go);
         tma_load_2d_if(sR + (size_t)slot * kBox, m, x + box * BK, y, w_full + slot, go);
-        ++ws;
         if (++slot == kRing) {
           slot = 0;
           par ^= 1u;
@@ -497,8 +496,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     // the last loads land before this block's shared memory goes away (after a
     // timed-out wait nothing else has waited for them)
-    for (int i = ws < kRing ? 0 : ws - kRing; i < ws; ++i)
-      mbar_wait_warp(w_full + i % kRing, (uint32_t)(i / kRing) & 1u, p.sel.status);
+    mbar_landed_ring(w_full, slot, par, kRing, p.sel.status);
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
     const uint32_t go = elect_one();
@@ -508,7 +506,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     int slot = 0, gf = 0, tl = 0;
     uint32_t par = 0;
     auto wait = [&](uint64_t* bar, uint32_t parity) {
-      mbar_wait_warp(bar, parity, p.sel.status);
+      mbar_wait_role(bar, parity, p.sel.status);
       tc_fence_after();
     };
     // the next weight box landed: its shared-memory address
@@ -632,7 +630,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const float sl2 = p.scale_log2;
     auto pair_sync = [&]() { asm volatile("bar.sync %0, 128;" ::"r"(1 + q) : "memory"); };  // the quadrant's 4 warps
     auto epi_sync = [&]() { asm volatile("bar.sync 5, %0;" ::"n"(32 * kEpiWarps) : "memory"); };
-    auto wait = [&](uint64_t* bar, uint32_t par) { mbar_wait_warp(bar, par, p.sel.status); };
+    auto wait = [&](uint64_t* bar, uint32_t par) { mbar_wait_role(bar, par, p.sel.status); };
     int tl = 0, gf = 0;
     for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++tl) {
       const int b0 = t * G;
@@ -649,6 +647,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int nst = min(p.off[b0 + Gv] - e0, NST);
       const float* sVP = reinterpret_cast<const float*>(sStage + NST * 272);
       if (et == 0) {
+        if (!mbar_test_wait(st_full, (tl & 1) ^ 1)) mbar_landed_slow(st_full, (tl & 1) ^ 1, p.sel.status, kWaitLimitUs);
         mbar_arrive_expect_tx(st_full, (uint32_t)nst * 272u + (uint32_t)L * (D * 4));
         if (nst > 0) {
           bulk_g2s(sStage, p.v_h + (size_t)e0 * D, (uint32_t)nst * 256u, st_full);
@@ -903,6 +902,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       epi_sync();
     }
+    if (ew == 0) mbar_landed(st_full, (tl & 1) ^ 1, p.sel.status);
   }
 
   __syncwarp();

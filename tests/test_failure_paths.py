@@ -4,10 +4,12 @@
   makes a chosen device or page-locked allocation fail as if the device were
   out of memory.  fe_init and a workspace grow must return FE_ERR_OOM, leave no
   allocation behind, and the context must keep working after a failed grow.
-* Bounded waits: fe_debug_wait_probe runs one thread that waits, through the
-  batch kernels' own bounded mbarrier wait, on a barrier nothing arrives on
-  (limit 1 ms, nothing else in flight).  The status must reach the host as
-  FE_ERR_TIMEOUT and the next batch on the same context must be correct.
+* Bounded waits: fe_debug_wait_probe runs each form of the batch kernels' own
+  bounded mbarrier waits in a warp, on a barrier nothing arrives on (limits of
+  0.1 to 3 ms, nothing else in flight).  Each gives up by its limit or because
+  another has, takes part in later waits only for a few polls, and arrives on
+  nothing any more where its role must not (FE_ERR_NUMERIC otherwise).  The status must
+  reach the host as FE_ERR_TIMEOUT and the next batch on the same context must be correct.
 * A weight blob gives the same context as the raw weight array.
 """
 import ctypes
@@ -139,6 +141,16 @@ def test_bounded_wait_reports_timeout_and_the_context_recovers():
     assert ev.last_status == binding.FE_OK
     assert torch.equal(s1, s0) and torch.equal(b1, b0)
     assert L.fe_debug_wait_probe(ev._h, 0, None) == binding.FE_ERR_INVALID_ARG
+    ev.close()
+
+
+@pytest.mark.parametrize("limit_us", [100, 3000])
+def test_every_form_of_wait_gives_up_once(limit_us):
+    L = _lib()
+    stream = torch.cuda.current_stream(torch.device("cuda:0")).cuda_stream
+    w = wl.make_workload("tiny")
+    ev = binding.Evaluator(w.cfg, w.weights)
+    assert L.fe_debug_wait_probe(ev._h, limit_us, ctypes.c_void_p(stream)) == binding.FE_ERR_TIMEOUT
     ev.close()
 
 
