@@ -29,6 +29,15 @@ namespace fe {
 
 namespace {
 
+__device__ __forceinline__ float pow2(int n) { return __int_as_float((127 + n) << 23); }  // |n| <= 126
+
+// f16 value as an integer of the same order
+__device__ __forceinline__ int order_key(__half x) {
+  const int b = __half_as_short(x);
+  return b >= 0 ? b : b ^ 0x7FFF;
+}
+__device__ __forceinline__ __half order_half(int k) { return __short_as_half((short)(k >= 0 ? k : k ^ 0x7FFF)); }
+
 // elu(x) + 1; the exponential branch (x <= 0, result in (0, 1]) through the
 // hardware exponent unit, whose relative error is far below the f16 rounding
 // of the keys and queries it is applied to
@@ -36,6 +45,9 @@ __device__ __forceinline__ float phi(float x) { return x > 0.f ? x + 1.f : __exp
 
 constexpr int kChunk = 64;                // context rows per operand tile
 constexpr uint32_t kAtom = kChunk * 128;  // 64 features x kChunk rows, f16
+constexpr int kFlush = 16;                // chunks that are added up on the tensor core (even)
+constexpr float kLoScale = 2048.f;        // phi's lo plane is stored times 2^11 (at most 2^15)
+constexpr float kPhiSmall = -9.f;         // keys below: phi < 2^-12.98
 
 // MN-major operand descriptor, 128-byte swizzle: atoms of 64 features, kAtom apart, 8-row groups 1024 bytes apart
 __device__ __forceinline__ uint64_t desc_feat(uint32_t saddr) {
@@ -54,8 +66,9 @@ struct StateCfg {
   static constexpr uint32_t kA = 2 * kAtom;
   static constexpr uint32_t kV = (FG == 128 ? 3 : FG == 64 ? 2 : 1) * kAtom;
   static constexpr uint32_t kBuf = 2 * kA + kV;
-  static constexpr size_t kSmem = 2 * kBuf + 64;  // two buffers, barriers
-  // three accumulators: the hi products of even and of odd chunks, the lo products
+  static constexpr size_t kSmem = 2 * kBuf + 64 + FG * 4;  // two buffers, barriers, each feature's largest key
+  // three accumulators: the hi products of even and of odd chunks, the lo products;
+  // 512 columns for FG = 128 (one CTA on an SM at a time), 256 below
   static constexpr int kN = FG + 16;
   static constexpr uint32_t kCols = 3 * kN <= 256 ? 256 : 512;
 };
@@ -64,18 +77,32 @@ struct StateCfg {
 
 // Context states.  A CTA takes one segment, one layer and one group of FG
 // features (FG = min(d, 128): the heads [g FG / DH, (g + 1) FG / DH)).  Per
-// 64 context rows its threads write phi(K), as a hi + lo pair of f16 tiles (22
-// bits), and V, an exact f16 tile followed by 16 columns of ones, and the tensor
-// core adds phi(K)^T [V | 1] to 128 x (FG + 16) accumulators in TMEM (z comes from
-// the ones columns; three accumulators, because the tensor core truncates each
-// addition); at the end each head's diagonal block and z are stored.  Two
-// operand buffers: the next chunk's rows are transformed and written
-// while the current one is multiplied, and the rows of two chunks are in flight.
+// 64 context rows its threads write phi(K), as a hi + lo pair of f16 tiles, and V,
+// an exact f16 tile followed by 16 columns of ones, and the tensor core adds
+// phi(K)^T [V | 1] to 128 x (FG + 16) accumulators in TMEM (z comes from the ones
+// columns).  Two operand buffers: the next chunk's rows are transformed and
+// written while the current one is multiplied, and the rows of two chunks are in flight.
+//
+// Precision: hi + lo hold 22 bits of phi for phi >= 2^-14 (lo is stored times 2^11
+// and its accumulator scaled back), and below that all but 2^-36.  A feature whose
+// largest phi over the context is below 2^-13 would lose bits, and below 2^-36 all of
+// them, so such a segment's group is done over with each of those features' phi times a
+// power of two that brings its largest one to (1/2, 1], undone in the stored
+// state.  The tensor core truncates each addition to its accumulator, so there are three
+// (hi of even and of odd chunks, lo), and their sums go to the stored state, added in
+// fp32, every 16 chunks.  Relative error of S (2-norm) and largest of z against 64 bits, 1000
+// rows: 6.2e-7, 1e-7 with keys ~ N(0, 0.5), 6.3e-7, 2e-7 at mean -12, 6.2e-7, 3e-7 at -20,
+// 8.7e-7, 6e-7 at -40; a chain of fp32 multiply-adds per element: 5.7e-7, 1.1e-6;
+// 6.4e-7, 1.8e-6; 7.3e-7, 1.9e-6; 1.1e-6, 1.5e-6.
+// 2000 rows: 6.2e-7 (7.7e-7).
+//
 // What bounds it: the transform of K (an exponent, two conversions and a 16-byte
 // store per plane for 8 values); the products take 8 MMAs of N = FG + 16 a chunk.
 // 256 segments of 1000 rows, two layers of 64 columns: 107 us with fp32 products on the
-// CUDA cores, 60 us here with one chunk's rows in flight, 53 with two (131 MB of K/V, 20 us
-// at the copy rate); the 512 CTAs are 1.7 waves of two per SM.
+// CUDA cores, 57 here (131 MB of K/V, 20 us at the copy rate; 54 without the scaled lo
+// plane and the largest keys), the 512 CTAs being 1.7 waves of two per SM.  FG = 128:
+// 181 -> 153 at d = 128; there a CTA takes all of the SM's TMEM columns (3 x 144 of
+// 512), so a second one on the SM waits for the first to end.
 template <int DH, int FG>
 __global__ void __launch_bounds__(256, 2) lin_state_kernel(const __half* __restrict__ kv, int hm, int rows_alloc,
                                                            int ld, int C, int d, int H, float* __restrict__ states,
@@ -91,6 +118,7 @@ __global__ void __launch_bounds__(256, 2) lin_state_kernel(const __half* __restr
   uint64_t* free_bar = bars;                // [2] the products of the chunk in this buffer are complete
   uint64_t* drain = bars + 2;               // the products in flight at the end
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 3);
+  int* kmax = reinterpret_cast<int*>(bars + 8);  // [FG] each feature's largest key of the segment (order_key)
   const int s = blockIdx.x, G = d / FG, l = blockIdx.y / G, g = blockIdx.y % G;
   const int kcol = 2 * l * d + g * FG, vcol = (2 * l + 1) * d + g * FG;
   const size_t row0 = (size_t)s * C;
@@ -109,6 +137,7 @@ __global__ void __launch_bounds__(256, 2) lin_state_kernel(const __half* __restr
     mbar_init(drain, 1);
     fence_mbar_init();
   }
+  if (t < FG) kmax[t] = order_key(__ushort_as_half(0xFC00u));  // -inf
   if (warp == 0) tmem_alloc(tmem_slot, Cfg::kCols);
   // features FG .. 127 of phi(K) are zeros, V's columns FG .. FG + 15 ones
   for (int i = t; i < 2 * kChunk; i += 256) {
@@ -142,12 +171,19 @@ __global__ void __launch_bounds__(256, 2) lin_state_kernel(const __half* __restr
   };
   const uint32_t go = elect_one();
   const uint32_t idesc = umma_idesc_f16(128, Cfg::kN) | (1u << 15) | (1u << 16);  // A and B MN-major
+  __half2 km[4];  // the largest keys of this thread's rows, of its 8 features
+#pragma unroll
+  for (int e = 0; e < 4; ++e) km[e] = __half2half2(__ushort_as_half(0xFC00u));
+  float scale[8];  // of its features' phi, in a second pass
+  int used[2] = {0, 0};  // chunks put through each operand buffer
   // chunk it (its pieces in kr, vr; chunk it + 2's are then loaded into them) through operand buffer B
-  auto chunk = [&](auto bufc, int it, uint4* kr, uint4* vr) {
+  auto chunk = [&](auto bufc, auto scaled, int it, uint4* kr, uint4* vr) {
     constexpr int B = decltype(bufc)::value;
+    constexpr bool kScaled = decltype(scaled)::value;
     const int r0 = it * kChunk;
     uint8_t* buf = sm_state + (size_t)B * Cfg::kBuf;
-    if (it >= 2) mbar_wait_role(free_bar + B, ((it >> 1) - 1) & 1, status);
+    if (used[B] > 0) mbar_wait_role(free_bar + B, (uint32_t)(used[B] - 1) & 1u, status);
+    ++used[B];
 #pragma unroll
     for (int q = 0; q < P8; ++q) {
       const int idx = t + 256 * q, r = idx / (FG / 8), c8 = (idx % (FG / 8)) * 8;
@@ -156,12 +192,17 @@ __global__ void __launch_bounds__(256, 2) lin_state_kernel(const __half* __restr
       uint32_t hi[4], lo[4];
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
+        if (!kScaled && valid) km[e] = __hmax2(km[e], hk[e]);
         const float2 x = __half22float2(hk[e]);
-        const float f0 = valid ? phi(x.x) : 0.f, f1 = valid ? phi(x.y) : 0.f;
+        float f0 = valid ? phi(x.x) : 0.f, f1 = valid ? phi(x.y) : 0.f;
+        if (kScaled) {
+          f0 *= scale[2 * e];
+          f1 *= scale[2 * e + 1];
+        }
         const __half2 h = __floats2half2_rn(f0, f1);
         const float2 hf = __half22float2(h);
         hi[e] = *reinterpret_cast<const uint32_t*>(&h);
-        lo[e] = pack_f16x2(f0 - hf.x, f1 - hf.y);
+        lo[e] = pack_f16x2((f0 - hf.x) * kLoScale, (f1 - hf.y) * kLoScale);
       }
       *reinterpret_cast<uint4*>(buf + piece(r, c8)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
       *reinterpret_cast<uint4*>(buf + Cfg::kA + piece(r, c8)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
@@ -179,61 +220,109 @@ __global__ void __launch_bounds__(256, 2) lin_state_kernel(const __half* __restr
       for (int kk = 0; kk < kChunk / 16; ++kk) {
         const uint32_t o = (uint32_t)kk * 16u * 128u;
         umma_bf16_if(tmem + (uint32_t)(B * Cfg::kN), desc_adv(ah, o), desc_adv(bd, o), idesc,
-                     (it > 1 || kk != 0) ? 1u : 0u, go);
-        umma_bf16_if(tmem + 2u * Cfg::kN, desc_adv(al, o), desc_adv(bd, o), idesc, (it | kk) != 0 ? 1u : 0u, go);
+                     (it % kFlush > 1 || kk != 0) ? 1u : 0u, go);
+        umma_bf16_if(tmem + 2u * Cfg::kN, desc_adv(al, o), desc_adv(bd, o), idesc, (it % kFlush | kk) != 0 ? 1u : 0u, go);
       }
       umma_commit_if(free_bar + B, go);
     }
   };
-  pdl_trigger();
-  pdl_wait();
-  uint4 k0[P8], v0[P8], k1[P8], v1[P8];
-  load(0, k0, v0);
-  load(kChunk, k1, v1);
-  const int it_end = (C + kChunk - 1) / kChunk;
-  for (int i = 0; i < it_end; i += 2) {
-    chunk(std::integral_constant<int, 0>{}, i, k0, v0);
-    if (i + 1 < it_end) chunk(std::integral_constant<int, 1>{}, i + 1, k1, v1);
-  }
-  // the last product (and so every earlier one) complete
-  mbar_wait_role(free_bar + ((it_end - 1) & 1), ((it_end - 1) >> 1) & 1, status);
-  tc_fence_after();
-  // lane m of the accumulator: feature m of the group; its head's DH columns, and z in column FG
+  // The sums of the chunks since the last flush (up to number `last`) to the stored state, added to
+  // what it holds unless they are the first.  Lane m of the accumulators: feature m of the
+  // group; its head's DH columns, and z in column FG.
   const int q = warp & 3, sub = warp >> 2, m = 32 * q + lane;
   const int Ly = gridDim.y / G;
-  if (32 * q < FG) {
-    const int hh = m / DH, i = m % DH;
-    float* st = states + (((size_t)s * Ly + l) * H + g * HG + hh) * SB;  // S row-major, then z
-    const uint32_t row = tmem + ((uint32_t)(q * 32) << 16);
-    const bool odd = it_end > 1;  // (a single chunk leaves the second accumulator unwritten)
-    if (sub == 0 || DH == 64) {
-      const uint32_t col = row + (uint32_t)((32 * q) / DH * DH + 32 * sub);
-      float v[32], w[32];
-      tmem_ld32(col, v);
-      tmem_ld32(col + 2u * Cfg::kN, w);
+  float* st = states + (((size_t)s * Ly + l) * H + g * HG + (m < FG ? m / DH : 0)) * SB;  // S row-major, then z
+  auto flush = [&](int last, float f) {
+    // the last product (and so every earlier one) complete
+    const int lb = last & 1;
+    mbar_wait_role(free_bar + lb, (uint32_t)((lb ? used[1] : used[0]) - 1) & 1u, status);
+    tc_fence_after();
+    const bool add = last >= kFlush, odd = last % kFlush > 0;  // (a single chunk leaves the second accumulator unwritten)
+    if (32 * q < FG) {
+      const int i = m % DH;
+      const uint32_t row = tmem + ((uint32_t)(q * 32) << 16);
+      if (sub == 0 || DH == 64) {
+#pragma unroll 1
+        for (int c = 0; c < 32; c += 8) {
+          const uint32_t col = row + (uint32_t)((32 * q) / DH * DH + 32 * sub + c);
+          float* dst = st + i * DH + 32 * sub + c;
+          uint32_t v[8], w[8];
+          float x[8];
+          tmem_ld8(col, v);
+          tmem_ld8(col + 2u * Cfg::kN, w);
 #pragma unroll
-      for (int j = 0; j < 32; ++j) v[j] += w[j];
-      if (odd) {
-        tmem_ld32(col + (uint32_t)Cfg::kN, w);
+          for (int j = 0; j < 8; ++j) x[j] = fmaf(__uint_as_float(w[j]), 1.f / kLoScale, __uint_as_float(v[j]));
+          if (odd) {
+            tmem_ld8(col + (uint32_t)Cfg::kN, w);
 #pragma unroll
-        for (int j = 0; j < 32; ++j) v[j] += w[j];
+            for (int j = 0; j < 8; ++j) x[j] += __uint_as_float(w[j]);
+          }
+          if (add) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) x[j] += dst[j];
+          }
+#pragma unroll
+          for (int j = 0; j < 8; j += 4)
+            *reinterpret_cast<float4*>(dst + j) = make_float4(x[j] * f, x[j + 1] * f, x[j + 2] * f, x[j + 3] * f);
+        }
       }
-#pragma unroll
-      for (int j = 0; j < 32; j += 4)
-        *reinterpret_cast<float4*>(st + i * DH + 32 * sub + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+      if (sub == (DH == 64 ? 0 : 1)) {
+        uint32_t z[8], w[8], u[8];
+        tmem_ld8(row + (uint32_t)FG, z);
+        tmem_ld8(row + (uint32_t)(Cfg::kN + FG), u);
+        tmem_ld8(row + (uint32_t)(2 * Cfg::kN + FG), w);
+        float x = fmaf(__uint_as_float(w[0]), 1.f / kLoScale, __uint_as_float(z[0]));
+        if (odd) x += __uint_as_float(u[0]);
+        st[DH * DH + i] = ((add ? st[DH * DH + i] : 0.f) + x) * f;
+      }
     }
-    if (sub == (DH == 64 ? 0 : 1)) {
-      uint32_t z[8], w[8], u[8];
-      tmem_ld8(row + (uint32_t)FG, z);
-      tmem_ld8(row + (uint32_t)(Cfg::kN + FG), u);
-      tmem_ld8(row + (uint32_t)(2 * Cfg::kN + FG), w);
-      st[DH * DH + i] = __uint_as_float(z[0]) + __uint_as_float(w[0]) + (odd ? __uint_as_float(u[0]) : 0.f);
+    tc_fence_before();
+    __syncthreads();  // the accumulators are read
+  };
+  uint4 k0[P8], v0[P8], k1[P8], v1[P8];
+  const int it_end = (C + kChunk - 1) / kChunk;
+  // every chunk; the last window's sums stay in the accumulators
+  auto pass = [&](auto scaled) {
+    load(0, k0, v0);
+    load(kChunk, k1, v1);
+    for (int i = 0; i < it_end; i += 2) {
+      if (i > 0 && i % kFlush == 0) flush(i - 1, 1.f);
+      chunk(std::integral_constant<int, 0>{}, scaled, i, k0, v0);
+      if (i + 1 < it_end) chunk(std::integral_constant<int, 1>{}, scaled, i + 1, k1, v1);
+    }
+  };
+  pdl_trigger();
+  pdl_wait();
+  pass(std::false_type{});
+  // each feature's largest key, over the lanes and warps that share its columns
+#pragma unroll
+  for (int o = FG / 8; o < 32; o <<= 1)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) km[e] = __hmax2(km[e], __shfl_xor_sync(0xffffffffu, km[e], o));
+  if (lane < FG / 8) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      atomicMax(kmax + 8 * lane + 2 * e, order_key(__low2half(km[e])));
+      atomicMax(kmax + 8 * lane + 2 * e + 1, order_key(__high2half(km[e])));
     }
   }
-  if (warp == 0) umma_drain(drain, status, go);
-  tc_fence_before();
   __syncthreads();
-  if (warp == 0) tmem_dealloc(tmem, Cfg::kCols);
+  // the power of two of feature m: 1 where its largest phi is at least 2^-14
+  auto exponent = [&](int m) {
+    const float x = __half2float(order_half(kmax[m]));
+    return x >= kPhiSmall ? 0 : (int)fminf(126.f, floorf(-x * 1.44269504f));
+  };
+  const int my_exp = t < FG ? exponent(t) : 0;
+  if (__syncthreads_or(my_exp)) {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) scale[e] = pow2(exponent((t % (FG / 8)) * 8 + e));
+    pass(std::true_type{});
+  }
+  flush(it_end - 1, m < FG ? pow2(-exponent(m)) : 1.f);
+  if (warp == 0) {
+    umma_drain(drain, status, go);
+    tmem_dealloc(tmem, Cfg::kCols);
+  }
 }
 
 namespace {
