@@ -454,12 +454,16 @@ __global__ void __launch_bounds__(256) lin_attn_kernel(const __half* __restrict_
 
 namespace {
 // H <= 8 heads of d_h = 64, and a block of rows of width d <= 512 (half a block there)
+int g_lin_sms = 0;
 constexpr int kLinAttnSmemMax = 8 * (64 * 64 + 64) * 4 + kRowBlock / 2 * (512 + 4) * 4;
 }
 
 cudaError_t linattn_prepare() {
-  cudaError_t e = cudaFuncSetAttribute(lin_attn_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       kLinAttnSmemMax);
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g_lin_sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(lin_attn_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLinAttnSmemMax);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(lin_attn_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLinAttnSmemMax);
   auto state = [&](const void* f, size_t smem) {
@@ -500,7 +504,7 @@ cudaError_t lin_attn_launch(const bf16* q, int ldq, const float* states, int n_s
   // rows, 16 per task, 190 us, blocks of 64 and 8 per task 186.4, two CTAs 178.1, more 178.0; for 64 segments
   // 120.1, 113.2, 109.3 with eight), in smaller blocks the more of them there are (64 segments of 100 rows, d =
   // 128: blocks of 32 190, of 16 185; 256 of 60, d = 64, with four CTAs: 178.0 and 180.5).
-  int ny = 4 * 152 / n_seg;
+  int ny = 4 * (g_lin_sms > 0 ? g_lin_sms : 148) / n_seg;
   ny = ny < 1 ? 1 : ny > 8 ? 8 : ny;
   const int row_block = ny >= 4 ? kRowBlock / 4 : ny > 1 || d > 256 ? kRowBlock / 2 : kRowBlock;
   const size_t smem = ((size_t)H * (dh * dh + dh) + (size_t)row_block * (d + 4)) * sizeof(float);
