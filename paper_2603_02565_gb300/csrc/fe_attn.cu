@@ -33,7 +33,8 @@
 // 1024 requests x 512 keys x 8 heads 811 -> 459 us a launch (of which balanced rounds
 // 811 -> 565, shared staging of the output 565 -> 459), K = 1000 cross-sequence
 // attention 103 -> 92, batch of 256 requests 158.0 -> 151.5 us in all.  A lone
-// unit (one request) takes about 2 us longer than with eight warps.  The softmax of
+// unit (one request) takes about 2 us longer than with eight warps, and more the
+// longer its keys, so from 32 chunks on idle groups share it (SPLIT).  The softmax of
 // four groups still takes about 2300 cycles a chunk where the same instructions
 // without barriers take 1400: latency between the roles, not a pipe.
 // Register split: the kernel's arithmetic keeps a chunk's 64 (128) scores per lane
@@ -175,7 +176,11 @@ __device__ __forceinline__ void zero_tail(uint8_t* t, int o0, int end) {
 
 }  // namespace
 
-template <int DH>
+// SPLIT: p.ks groups of a CTA take one unit together (the only one of each of them),
+// group grp its chunks [part kper, (part + 1) kper), part = grp % ks, none of them
+// empty; their outputs, each against its own maximum, are put together at the end
+// through shared memory.
+template <int DH, bool SPLIT>
 __global__ void __launch_bounds__(AttnCfg<DH>::kThreads, 1)
     attn_kernel(const __grid_constant__ CUtensorMap tQ, const __grid_constant__ CUtensorMap tK,
                 const __grid_constant__ CUtensorMap tV, const AttnParams p) {
@@ -188,15 +193,19 @@ __global__ void __launch_bounds__(AttnCfg<DH>::kThreads, 1)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars0 + NG * Cfg::kBars);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // group of this warp: role warps (issuers 0 .. NG - 1, then the loaders, if
+  // any), then four softmax warps each
+  const int grp = warp < kRoleWarps ? warp % NG : (warp - kRoleWarps) >> 2;
+  const int j0 = SPLIT ? grp % p.ks * p.kper : 0;  // this group's first chunk of a unit
   // keys of a unit's segment: a fixed count at a fixed stride, or, for
   // self-attention within segments, the segment's own query rows
   auto kv_count = [&](const Cursor& c) { return p.kv_self ? c.qcnt : p.kv_cnt; };
   auto kv_base = [&](const Cursor& c) { return p.kv_self ? c.qoff : c.b * p.kv_stride; };
-  auto chunks = [&](const Cursor& c) { return (kv_count(c) + CK - 1) / CK; };
+  auto chunks = [&](const Cursor& c) {  // of this group
+    const int n = (kv_count(c) + CK - 1) / CK;
+    return SPLIT ? min(p.kper, n - j0) : n;
+  };
 
-  // group of this warp: role warps (issuers 0 .. NG - 1, then the loaders, if
-  // any), then four softmax warps each
-  const int grp = warp < kRoleWarps ? warp % NG : (warp - kRoleWarps) >> 2;
   uint8_t* sQ = smem + (size_t)grp * Cfg::kGroupBytes;  // [NQ][lane quadrant][32 rows]
   uint8_t* sKV = sQ + NQ * Cfg::kQBytes;                // [NS][K, V]
   uint64_t* bars = bars0 + grp * Cfg::kBars;
@@ -224,7 +233,7 @@ __global__ void __launch_bounds__(AttnCfg<DH>::kThreads, 1)
   tc_fence_after();
   const uint32_t tmem = *tmem_slot + (uint32_t)(grp * Cfg::kGroupCols);
   // the group's head, first segment (none: past the last) and first tile's row
-  const int wi = grp * (int)gridDim.x + (int)blockIdx.x;
+  const int wi = (SPLIT ? grp / p.ks : grp) * (int)gridDim.x + (int)blockIdx.x;
   const int head = wi % p.n_heads;
   const int b0 = wi < p.sb * p.n_heads * p.tp ? (wi / p.n_heads) % p.sb : p.n_segments;
   const int row0 = wi / (p.n_heads * p.sb) * BQ;
@@ -247,7 +256,7 @@ __global__ void __launch_bounds__(AttnCfg<DH>::kThreads, 1)
     auto load_next = [&]() {
       mbar_wait_load(kv_empty + ls, kv_full + ls, lpar, p.status);
       uint8_t* kv = sKV + ls * Cfg::kKVBytes;
-      const int row = kv_base(lc) + lj * CK;
+      const int row = kv_base(lc) + (j0 + lj) * CK;
       mbar_arrive_expect_tx_if(kv_full + ls, Cfg::kKVBytes, go);
       if (p.kv3d) {  // head-major K/V: one contiguous block per head
         tma_load_3d_if(kv, &tK, 0, row, (p.k_col + head * DH) / DH, kv_full + ls, go);
@@ -255,7 +264,7 @@ __global__ void __launch_bounds__(AttnCfg<DH>::kThreads, 1)
       } else {
         tma_load_2d_if(kv, &tK, p.k_col + head * DH, row, kv_full + ls, go);
         if (p.kv_seg)  // rows past the segment's kv_cnt keys are outside the map: zeros
-          tma_load_3d_if(kv + Cfg::kKVTile, &tV, p.v_col + head * DH, lj * CK, lc.b, kv_full + ls, go);
+          tma_load_3d_if(kv + Cfg::kKVTile, &tV, p.v_col + head * DH, (j0 + lj) * CK, lc.b, kv_full + ls, go);
         else
           tma_load_2d_if(kv + Cfg::kKVTile, &tV, p.v_col + head * DH, row, kv_full + ls, go);
       }
@@ -306,7 +315,7 @@ __global__ void __launch_bounds__(AttnCfg<DH>::kThreads, 1)
         // segment: their P is 0, but 0 x NaN is NaN, so they are zeroed here
         // (the chunk has landed; its PV, issued later by this warp, reads them)
         if (pad_v) {
-          const int kval = kv_count(sc) - sj * CK;
+          const int kval = kv_count(sc) - (j0 + sj) * CK;
           if (kval < CK) zero_tail(sKV + ss * Cfg::kKVBytes + Cfg::kKVTile, kval * (int)Cfg::kRowBytes, (int)Cfg::kKVTile);
         }
         ++g_s;
@@ -381,6 +390,15 @@ __global__ void __launch_bounds__(AttnCfg<DH>::kThreads, 1)
         mbar_arrive_if_at(bb + 8u * (uint32_t)buf, go);
       }
     };
+    // SPLIT: a group's output of tile row r (16-byte pieces XOR-swizzled) and its maximum and sum, in
+    // its K/V stages (every product has read them), and the barrier of the groups that share a unit
+    auto part_row = [&](int g2, int k) {
+      return smem + (size_t)g2 * Cfg::kGroupBytes + NQ * Cfg::kQBytes + r * (DH * 4) + ((k ^ (r & 7)) << 4);
+    };
+    auto part_ml = [&](int g2) {
+      return reinterpret_cast<float2*>(smem + (size_t)g2 * Cfg::kGroupBytes + NQ * Cfg::kQBytes + BQ * DH * 4) + r;
+    };
+    auto set_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + grp / p.ks), "r"(128 * p.ks) : "memory"); };
     Cursor c, next;
     cur_first(p, b0, row0, next);
     load_q(next, 0);
@@ -412,7 +430,7 @@ __global__ void __launch_bounds__(AttnCfg<DH>::kThreads, 1)
           __syncwarp();
           mbar_arrive_if_at(bb + kSFull + 8u, go);
           // keys past kv_cnt take no part: -inf gives them P = 0
-          const int kvalid = kv_count(c) - j * CK;
+          const int kvalid = kv_count(c) - (j0 + j) * CK;
           if (kvalid < CK) {
 #pragma unroll
             for (int i = 0; i < CK; ++i)
@@ -495,7 +513,7 @@ __global__ void __launch_bounds__(AttnCfg<DH>::kThreads, 1)
         // row: no bank conflicts), so that a store instruction writes whole row
         // pieces; a lane storing its own row touched 32 rows per instruction
         // (9000 cycles a unit with every group at it)
-        const float inv = 1.f / (l[0] + l[1]);
+        float lt = l[0] + l[1];
         const int left = c.qcnt - c.q0 - (r & ~31);  // rows of this warp's block
         uint32_t hi[DH / 2], lo[DH / 2];
         {
@@ -504,6 +522,38 @@ __global__ void __launch_bounds__(AttnCfg<DH>::kThreads, 1)
             tmem_ld64(t_o, o);
           else
             tmem_ld32(t_o, o);
+          if constexpr (SPLIT) {
+            if (grp % p.ks != 0) {
+#pragma unroll
+              for (int k = 0; k < DH / 4; ++k)
+                *reinterpret_cast<float4*>(part_row(grp, k)) = make_float4(o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
+              *part_ml(grp) = make_float2(m, lt);
+            }
+            set_sync();
+            if (grp % p.ks == 0) {
+              float mx = m;
+              for (int g2 = grp + 1; g2 < grp + p.ks; ++g2) mx = fmaxf(mx, part_ml(g2)->x);
+              float f = ex2_approx(m - mx);
+              lt *= f;
+#pragma unroll
+              for (int i = 0; i < DH; ++i) o[i] *= f;
+#pragma unroll 1
+              for (int g2 = grp + 1; g2 < grp + p.ks; ++g2) {
+                const float2 ml = *part_ml(g2);
+                f = ex2_approx(ml.x - mx);
+                lt = fmaf(ml.y, f, lt);
+#pragma unroll
+                for (int k = 0; k < DH / 4; ++k) {
+                  const float4 x = *reinterpret_cast<const float4*>(part_row(g2, k));
+                  o[4 * k] = fmaf(x.x, f, o[4 * k]);
+                  o[4 * k + 1] = fmaf(x.y, f, o[4 * k + 1]);
+                  o[4 * k + 2] = fmaf(x.z, f, o[4 * k + 2]);
+                  o[4 * k + 3] = fmaf(x.w, f, o[4 * k + 3]);
+                }
+              }
+            }
+          }
+          const float inv = 1.f / lt;
 #pragma unroll
           for (int i = 0; i < DH / 2; ++i) split2(o[2 * i] * inv, o[2 * i + 1] * inv, hi[i], lo[i]);
         }
@@ -519,7 +569,7 @@ __global__ void __launch_bounds__(AttnCfg<DH>::kThreads, 1)
           for (int i = 0; i < NC; ++i) {
             const int row = (i * 32 + lane) / NC, ch = lane % NC;
             const uint4 v = *reinterpret_cast<const uint4*>(sOut + row * Cfg::kRowBytes + (((uint32_t)ch ^ Cfg::swz(row)) << 4));
-            if (row < left) *reinterpret_cast<uint4*>(dst + (size_t)row * p.ldo + ch * 8) = v;
+            if (row < left && (!SPLIT || grp % p.ks == 0)) *reinterpret_cast<uint4*>(dst + (size_t)row * p.ldo + ch * 8) = v;
           }
           __syncwarp();
         };
@@ -528,6 +578,8 @@ __global__ void __launch_bounds__(AttnCfg<DH>::kThreads, 1)
         tc_fence_before();  // read before the next unit's first PV overwrites it (p_full orders the two)
         fence_async_shared();  // staging read before the next load into these rows
         __syncwarp();
+      } else if constexpr (SPLIT) {
+        set_sync();
       }
       ++u;
     }
@@ -544,16 +596,20 @@ __global__ void __launch_bounds__(AttnCfg<DH>::kThreads, 1)
 
 namespace {
 int g_attn_sms = 0;
+constexpr int kSplitChunks = 32;  // of a unit, from which on groups share it
 }
 
 cudaError_t attn_prepare() {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g_attn_sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(attn_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AttnCfg<32>::kSmem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(attn_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AttnCfg<64>::kSmem);
+  auto smem = [&](const void* f, size_t n) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)n);
+  };
+  smem((const void*)attn_kernel<32, false>, AttnCfg<32>::kSmem);
+  smem((const void*)attn_kernel<32, true>, AttnCfg<32>::kSmem);
+  smem((const void*)attn_kernel<64, false>, AttnCfg<64>::kSmem);
+  smem((const void*)attn_kernel<64, true>, AttnCfg<64>::kSmem);
   return e;
 }
 
@@ -566,14 +622,36 @@ cudaError_t attn_launch(int dh, const CUtensorMap* q, const CUtensorMap* k, cons
   // the groups of a full grid take sb segments at a time, and with few of them several query tiles of each
   const int tiles = (p.max_q + BQ - 1) / BQ;
   const int sms = g_attn_sms > 0 ? g_attn_sms : 148;
-  const int groups = sms * (dh == 32 ? AttnCfg<32>::NG : AttnCfg<64>::NG);
-  p.sb = groups / p.n_heads < p.n_segments ? groups / p.n_heads : p.n_segments;
-  p.tp = groups / (p.sb * p.n_heads) < tiles ? groups / (p.sb * p.n_heads) : tiles;
+  const int ng = dh == 32 ? AttnCfg<32>::NG : AttnCfg<64>::NG, groups = sms * ng;
+  // Few units with many keys: as many groups as there are for each take a unit together
+  // (SPLIT), from 32 chunks on.  Unsplit, a unit is one group's chain, 0.6 us a chunk and layer, and with
+  // fewer units than groups the others stand idle: one request, d_h = 32, 2048 keys 134 us in all unsplit and
+  // 109 split, 4096 179 and 128, 65536 1513 and 651; d_h = 64, 4096 keys 148 and 131; 16 requests of 16384 keys
+  // 532 and 325; 64 requests of 4096 keys (two groups a unit) 247 split.  Below 32 chunks the order of the
+  // sums stays the one group's.
+  const int nch = (p.kv_cnt + attn_chunk_keys(dh) - 1) / attn_chunk_keys(dh);
+  const long long units = (long long)p.n_segments * p.n_heads * tiles;
+  p.ks = 1;
+  if (!p.kv_self && nch >= kSplitChunks)
+    for (p.ks = ng; p.ks > 1 && units * p.ks > groups;) p.ks /= 2;
+  p.kper = (nch + p.ks - 1) / p.ks;
+  if (p.ks > 1) {
+    p.sb = p.n_segments;
+    p.tp = tiles;
+  } else {
+    p.sb = groups / p.n_heads < p.n_segments ? groups / p.n_heads : p.n_segments;
+    p.tp = groups / (p.sb * p.n_heads) < tiles ? groups / (p.sb * p.n_heads) : tiles;
+  }
   const int w = p.sb * p.n_heads * p.tp;
   const dim3 g((unsigned)(w < sms ? w : sms));
+  auto go = [&](auto kern, int threads, size_t smem) {
+    return launch_k(kern, g, dim3((unsigned)threads), smem, s, *q, *k, *v, p);
+  };
   if (dh == 32)
-    return launch_k(attn_kernel<32>, g, dim3(AttnCfg<32>::kThreads), AttnCfg<32>::kSmem, s, *q, *k, *v, p);
-  return launch_k(attn_kernel<64>, g, dim3(AttnCfg<64>::kThreads), AttnCfg<64>::kSmem, s, *q, *k, *v, p);
+    return p.ks > 1 ? go(attn_kernel<32, true>, AttnCfg<32>::kThreads, AttnCfg<32>::kSmem)
+                    : go(attn_kernel<32, false>, AttnCfg<32>::kThreads, AttnCfg<32>::kSmem);
+  return p.ks > 1 ? go(attn_kernel<64, true>, AttnCfg<64>::kThreads, AttnCfg<64>::kSmem)
+                  : go(attn_kernel<64, false>, AttnCfg<64>::kThreads, AttnCfg<64>::kSmem);
 }
 
 }  // namespace fe

@@ -279,6 +279,7 @@ struct AttnParams {
   int n_segments, n_heads;
   int max_q;             // largest q_cnt of any segment (grid sizing)
   int sb, tp;            // segments and query tiles of a round (set by attn_launch)
+  int ks, kper;          // groups that share a unit, and the key chunks of each (set by attn_launch)
   const int* q_off_dev;  // null: q_off = b * q_stride
   const int* q_cnt_dev;  // null: q_cnt = q_cnt_fixed
   int q_stride;
