@@ -244,17 +244,10 @@ __device__ __forceinline__ void mbar_landed_at(uint32_t bar, uint32_t parity, in
   __syncwarp();
 }
 // The newest load on each of a ring's S barriers, the next load going to number `slot`
-// with the parity `par` of its wait (mbar_wait_load).  All are asked before one is
-// waited for: as a rule they landed long ago, and the kernel ends behind this.
-static __device__ __noinline__ void mbar_landed_ring_slow(uint64_t* full, int slot, uint32_t par, int S, int* status) {
-  for (int i = 0; i < S; ++i) mbar_landed_slow(full + i, i < slot ? par ^ 1u : par, status, kWaitLimitUs);
-}
+// with the parity `par` of its wait.
 __device__ __forceinline__ void mbar_landed_ring(uint64_t* full, int slot, uint32_t par, int S, int* status) {
-  bool ok = true;
-#pragma unroll 4
-  for (int i = 0; i < S; ++i) ok &= mbar_test_wait(full + i, i < slot ? par ^ 1u : par);
-  if (!ok) mbar_landed_ring_slow(full, slot, par, S, status);
-  __syncwarp();
+#pragma unroll 1
+  for (int i = 0; i < S; ++i) mbar_landed(full + i, i < slot ? par ^ 1u : par, status);
 }
 // The wait before the next load on barrier `full`: its previous load has landed (asked
 // first, off the path from the freed memory to its next load) and its memory is free.
