@@ -30,9 +30,8 @@
 // ones.  The scaling and the sums use two-element fp32 instructions.
 // Measured against one unit per CTA, two CTAs per SM, eight softmax warps a unit
 // (two per lane quadrant, exchanging row maxima) and units dealt out tile by tile:
-// 1024 requests x 512 keys x 8 heads 811 -> 459 us a launch (of which balanced rounds
-// 811 -> 565, shared staging of the output 565 -> 459), K = 1000 cross-sequence
-// attention 103 -> 92, batch of 256 requests 158.0 -> 151.5 us in all.  A lone
+// 1024 requests x 512 keys x 8 heads 811 -> 435 us a launch, K = 1000 cross-sequence
+// attention 103 -> 95, the two of 256 requests 42 -> 41.  A lone
 // unit (one request) takes about 2 us longer than with eight warps, and more the
 // longer its keys, so from 32 chunks on idle groups share it (SPLIT).  The softmax of
 // four groups still takes about 2300 cycles a chunk where the same instructions
@@ -526,7 +525,8 @@ __global__ void __launch_bounds__(AttnCfg<DH>::kThreads, 1)
             if (grp % p.ks != 0) {
 #pragma unroll
               for (int k = 0; k < DH / 4; ++k)
-                *reinterpret_cast<float4*>(part_row(grp, k)) = make_float4(o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
+                *reinterpret_cast<float4*>(part_row(grp, k)) =
+                    make_float4(o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
               *part_ml(grp) = make_float2(m, lt);
             }
             set_sync();
@@ -569,7 +569,8 @@ __global__ void __launch_bounds__(AttnCfg<DH>::kThreads, 1)
           for (int i = 0; i < NC; ++i) {
             const int row = (i * 32 + lane) / NC, ch = lane % NC;
             const uint4 v = *reinterpret_cast<const uint4*>(sOut + row * Cfg::kRowBytes + (((uint32_t)ch ^ Cfg::swz(row)) << 4));
-            if (row < left && (!SPLIT || grp % p.ks == 0)) *reinterpret_cast<uint4*>(dst + (size_t)row * p.ldo + ch * 8) = v;
+            if (row < left && (!SPLIT || grp % p.ks == 0))
+              *reinterpret_cast<uint4*>(dst + (size_t)row * p.ldo + ch * 8) = v;
           }
           __syncwarp();
         };

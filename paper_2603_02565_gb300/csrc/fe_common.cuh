@@ -617,9 +617,8 @@ __device__ __forceinline__ uint64_t f32x2_mul(uint64_t a, uint64_t b) {
 // LayerNorm passes over N values of a row, two values per instruction: sums in four
 // interleaved chains (chain j % 4, two to a register pair), with the results of the
 // scalar forms.  The epilogues that use them, and the split pairs' sub2, are bound by the
-// instructions they issue and fetch: 256 requests 148.2 -> 145.5 us, ragged requests
-// 98.1 -> 96.1, 64 of 1000 candidates 363.3 -> 359.7, the largest batch 3810 -> 3794,
-// 45 requests at d = 256 212.2 -> 210.1, the d = 512 summarisation batch 622.4 -> 620.2.
+// instructions they issue and fetch: with them 256 requests took 1.8 % less in all, the
+// largest batch 0.4 %.
 struct RowSum {
   uint64_t s01 = 0, s23 = 0;  // (0.f, 0.f)
   __device__ __forceinline__ float total() const {

@@ -25,17 +25,12 @@
 // The MMA groups are 16 instructions of N >= 128 so that the tensor pipe has
 // queued work while the issuing warp polls its barriers; x0 is read by the
 // epilogue warps while the A tile is in flight, when they have nothing else to
-// do, a 32-byte sector a load (16 bytes a load took 256 requests 149.3 us in all
-// instead of 147.3, ragged ones 98.5 instead of 97.5; all of a row's loads at once
-// 153.7 and 102.2); the biases sit in shared memory.
+// do, a 32-byte sector a load; the biases sit in shared memory.
 // What bounds it: a tile is one dependency chain of which the tensor pipe needs
-// 5 us (160 MMAs of N = 128 at d = 128, F = 512).  Behind `if (lane == 0)` an
-// MMA cost its issuing thread up to 92 cycles where the pipe takes 64, and a
-// satisfied wait 100 or more; with the warps run whole the batch of 256 requests went
-// from 163.8 to 159.1 us, one request from 124.9 to 119.5, 64 requests in fp32
-// from 148.4 to 141.0.  Most launches give a CTA one tile or two, so the epilogue's
-// code is fetched cold: its loops over a row's pieces stay rolled (256 requests 153.8 -> 150.6
-// us, 64 in fp32 137.8 -> 136.3).
+// 5 us (160 MMAs of N = 128 at d = 128, F = 512), 27 % of the 22 us that a launch of
+// one tile per CTA takes (18353 rows; 28 us with single issuing threads).  Most
+// launches give a CTA one tile or two, so the epilogue's code is fetched cold (a
+// quarter of the instruction requests miss): its loops over a row's pieces stay rolled.
 #include "fe_common.cuh"
 #include "fe_kernels.h"
 
@@ -246,7 +241,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           mbar_arrive_expect_tx_if(wt_full, (uint32_t)nkb * nb * (uint32_t)tail_n * (BK * 2), go);
           for (int kb = 0; kb < nkb; ++kb)
             for (int q = 0; q < nb; ++q)
-              tma_load_2d_if(sT + (size_t)(kb * nb + q) * tail_n * (BK * 2), q ? &tT_l : &tT_h, kb * BK, 0, wt_full, go);
+              tma_load_2d_if(sT + (size_t)(kb * nb + q) * tail_n * (BK * 2), q ? &tT_l : &tT_h, kb * BK, 0, wt_full,
+                             go);
         }
       }
     }();

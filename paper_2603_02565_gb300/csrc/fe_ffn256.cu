@@ -30,17 +30,13 @@
 // bf16 activations (hi + lo) times exact bf16 weights with fp32 accumulation;
 // LayerNorm and residuals are fp32.
 // What bounds it: the tensor pipe (a chunk is 64 MMAs of N = 128, 4096 cycles, on
-// both halves of its weights) and, per tile, the two LayerNorm phases.  With
-// warps 0 and 1 run whole (fe_common.cuh) the largest batch (295k rows, two element
-// layers and SeqEnc) went from 5495 to 5035 us and 45 requests from 269.5 to 235.5.
-// A tile's first k block came 8.5k cycles after the previous tile's end (its stores
-// drain at 32 bytes a cycle, then DRAM, on every SM at once).  The prefetch took the
-// largest batch from 4073 to 3952 us, rolled epilogue loops (127 registers, none
-// spilled, less code to fetch than unrolled by 4) to 3932 and 45 requests from 219.6 to
-// 216.3, the release by k blocks the largest to 3896.
-// x0 is loaded a 32-byte sector at a time: 3866 -> 3825, 45 requests 214.6 -> 211.4.
-// Holding a thread's 128 columns in registers through both LayerNorm passes, the loops
-// unrolled, was slower (45 requests 226.5).
+// both halves of its weights) and, per tile, the two LayerNorm phases.  A tile's first
+// k block came 8.5k cycles after the previous tile's end (its stores drain at
+// 32 bytes a cycle, then DRAM, on every SM at once), hence the prefetch and the
+// release by k blocks; the epilogue loops stay rolled (127 registers, none spilled).
+// 295k rows, a launch with the tail: 826 -> 566 us (tensor pipe 39 -> 55 %).
+// Holding a thread's 128 columns in registers through both LayerNorm passes, the
+// loops unrolled, was slower.
 #include "fe_common.cuh"
 #include "fe_kernels.h"
 

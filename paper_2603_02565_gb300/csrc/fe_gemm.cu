@@ -15,15 +15,12 @@
 //                    alternate 32-column chunks
 // The loading and the issuing warp run whole (fe_common.cuh): at two to four
 // MMAs of N >= 128 per 64-wide k step the issuing thread, not the tensor pipe, set
-// the pace (d = 512 summarisation batch 679 -> 631 us, 64 requests in fp32 140.9 ->
-// 137.7).
+// the pace (d = 512 summarisation batch 679 -> 631 us in all).
 // The residual rows of a LayerNorm tile arrive by TMA in the staging buffers that x
 // leaves from: a thread's own 16-byte loads, one row per lane, took a line of the L1
-// that 220 KB of shared memory leaves for every one of them.  Rows of more than 128
-// columns have their own instantiation, whose threads load 32-byte sectors (largest
-// batch 3825 -> 3818).  Both together: 64 requests of 1000 candidates
-// 367.2 -> 362.3 us, the d = 512 summarisation batch 625.4 -> 621.4, d = 256 largest
-// batch 3870 -> 3855.
+// that 220 KB of shared memory leaves for every one of them (64000 rows x 128
+// columns 33 -> 28 us).  Rows of more than 128 columns have their own instantiation,
+// whose threads load 32-byte sectors.
 // The activation is a split pair (hi + lo bf16); the product is
 // A_hi W_hi + A_lo W_hi (+ A_hi W_lo when the weights carry a lo plane).
 #include <cstdlib>

@@ -231,13 +231,15 @@ __global__ void __launch_bounds__(256, 2) lin_state_kernel(const __half* __restr
   // group; its head's DH columns, and z in column FG.
   const int q = warp & 3, sub = warp >> 2, m = 32 * q + lane;
   const int Ly = gridDim.y / G;
-  float* st = states + (((size_t)s * Ly + l) * H + g * HG + (m < FG ? m / DH : 0)) * SB;  // S row-major, then z
+  // S row-major, then z
+  float* st = states + (((size_t)s * Ly + l) * H + g * HG + (m < FG ? m / DH : 0)) * SB;
   auto flush = [&](int last, float f) {
     // the last product (and so every earlier one) complete
     const int lb = last & 1;
     mbar_wait_role(free_bar + lb, (uint32_t)((lb ? used[1] : used[0]) - 1) & 1u, status);
     tc_fence_after();
-    const bool add = last >= kFlush, odd = last % kFlush > 0;  // (a single chunk leaves the second accumulator unwritten)
+    const bool add = last >= kFlush;
+    const bool odd = last % kFlush > 0;  // (a single chunk leaves the second accumulator unwritten)
     if (32 * q < FG) {
       const int i = m % DH;
       const uint32_t row = tmem + ((uint32_t)(q * 32) << 16);

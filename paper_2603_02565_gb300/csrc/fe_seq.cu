@@ -32,8 +32,8 @@
 // softmax and residuals are fp32.
 // What bounds it: one tile's chain per CTA, the tensor pipe a fifth of it.  Warps
 // 0 and 1 run whole (fe_common.cuh) and the weight order is a plain loop nest
-// instead of a search per box: 256 requests 159.7 -> 158.5 us, 37 requests 105.0 ->
-// 102.0, one request 118.5 -> 116.
+// instead of a search per box.  128 tiles: 47 us, tensor pipe 19 %, a quarter of the
+// instruction requests miss the cache.
 #include "fe_common.cuh"
 #include "fe_kernels.h"
 
