@@ -47,7 +47,8 @@ constexpr int kChunk = 64;                // context rows per operand tile
 constexpr uint32_t kAtom = kChunk * 128;  // 64 features x kChunk rows, f16
 constexpr int kFlush = 16;                // chunks that are added up on the tensor core (even)
 constexpr float kLoScale = 2048.f;        // phi's lo plane is stored times 2^11 (at most 2^15)
-constexpr float kPhiSmall = -9.f;         // keys below: phi < 2^-12.98
+constexpr float kPhiSmall = 1.f / 8192;   // 2^-13
+constexpr float kKeySmall = -9.f;         // keys below: phi < 2^-12.98
 
 // MN-major operand descriptor, 128-byte swizzle: atoms of 64 features, kAtom apart, 8-row groups 1024 bytes apart
 __device__ __forceinline__ uint64_t desc_feat(uint32_t saddr) {
@@ -86,9 +87,9 @@ struct StateCfg {
 // Precision: hi + lo hold 22 bits of phi for phi >= 2^-14 (lo is stored times 2^11
 // and its accumulator scaled back), and below that all but 2^-36.  A feature whose
 // largest phi over the context is below 2^-13 would lose bits, and below 2^-36 all of
-// them, so such a segment's group is done over with each of those features' phi times a
-// power of two that brings its largest one to (1/2, 1], undone in the stored
-// state.  The tensor core truncates each addition to its accumulator, so there are three
+// them, so such a segment's group (z / C tells) is done over with each of those
+// features' phi times a power of two that brings its largest one to (1/2, 1], undone
+// in the stored state.  The tensor core truncates each addition to its accumulator, so there are three
 // (hi of even and of odd chunks, lo), and their sums go to the stored state, added in
 // fp32, every 16 chunks.  Relative error of S (2-norm) and largest of z against 64 bits, 1000
 // rows: 6.2e-7, 1e-7 with keys ~ N(0, 0.5), 6.3e-7, 2e-7 at mean -12, 6.2e-7, 3e-7 at -20,
@@ -100,8 +101,8 @@ struct StateCfg {
 // store per plane for 8 values); the products take 8 MMAs of N = FG + 16 a chunk.
 // 256 segments of 1000 rows, two layers of 64 columns: 107 us with fp32 products on the
 // CUDA cores, 57 here (131 MB of K/V, 20 us at the copy rate; 54 without the scaled lo
-// plane and the largest keys), the 512 CTAs being 1.7 waves of two per SM.  FG = 128:
-// 181 -> 153 at d = 128; there a CTA takes all of the SM's TMEM columns (3 x 144 of
+// plane, the test of z and the flushes), the 512 CTAs being 1.7 waves of two per SM.
+// FG = 128: 181 -> 151 at d = 128; there a CTA takes all of the SM's TMEM columns (3 x 144 of
 // 512), so a second one on the SM waits for the first to end.
 template <int DH, int FG>
 __global__ void __launch_bounds__(256, 2) lin_state_kernel(const __half* __restrict__ kv, int hm, int rows_alloc,
@@ -171,10 +172,7 @@ __global__ void __launch_bounds__(256, 2) lin_state_kernel(const __half* __restr
   };
   const uint32_t go = elect_one();
   const uint32_t idesc = umma_idesc_f16(128, Cfg::kN) | (1u << 15) | (1u << 16);  // A and B MN-major
-  __half2 km[4];  // the largest keys of this thread's rows, of its 8 features
-#pragma unroll
-  for (int e = 0; e < 4; ++e) km[e] = __half2half2(__ushort_as_half(0xFC00u));
-  float scale[8];  // of its features' phi, in a second pass
+  float scale[8];  // of this thread's features' phi, in a second pass
   int used[2] = {0, 0};  // chunks put through each operand buffer
   // chunk it (its pieces in kr, vr; chunk it + 2's are then loaded into them) through operand buffer B
   auto chunk = [&](auto bufc, auto scaled, int it, uint4* kr, uint4* vr) {
@@ -192,7 +190,6 @@ __global__ void __launch_bounds__(256, 2) lin_state_kernel(const __half* __restr
       uint32_t hi[4], lo[4];
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        if (!kScaled && valid) km[e] = __hmax2(km[e], hk[e]);
         const float2 x = __half22float2(hk[e]);
         float f0 = valid ? phi(x.x) : 0.f, f1 = valid ? phi(x.y) : 0.f;
         if (kScaled) {
@@ -233,11 +230,26 @@ __global__ void __launch_bounds__(256, 2) lin_state_kernel(const __half* __restr
   const int Ly = gridDim.y / G;
   // S row-major, then z
   float* st = states + (((size_t)s * Ly + l) * H + g * HG + (m < FG ? m / DH : 0)) * SB;
-  auto flush = [&](int last, float f) {
-    // the last product (and so every earlier one) complete
+  const bool z_warp = 32 * q < FG && sub == (DH == 64 ? 0 : 1);  // holds z of feature m
+  // every product up to chunk `last`'s complete
+  auto settle = [&](int last) {
     const int lb = last & 1;
     mbar_wait_role(free_bar + lb, (uint32_t)((lb ? used[1] : used[0]) - 1) & 1u, status);
     tc_fence_after();
+  };
+  // z of feature m up to chunk `last` (a z_warp's)
+  auto z_sum = [&](int last) {
+    const uint32_t row = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)FG;
+    uint32_t z[8], w[8], u[8];
+    tmem_ld8(row, z);
+    tmem_ld8(row + (uint32_t)Cfg::kN, u);
+    tmem_ld8(row + (uint32_t)(2 * Cfg::kN), w);
+    float x = fmaf(__uint_as_float(w[0]), 1.f / kLoScale, __uint_as_float(z[0]));
+    if (last % kFlush > 0) x += __uint_as_float(u[0]);
+    return last >= kFlush ? st[DH * DH + m % DH] + x : x;
+  };
+  auto flush = [&](int last, float f) {
+    settle(last);
     const bool add = last >= kFlush;
     const bool odd = last % kFlush > 0;  // (a single chunk leaves the second accumulator unwritten)
     if (32 * q < FG) {
@@ -268,16 +280,8 @@ __global__ void __launch_bounds__(256, 2) lin_state_kernel(const __half* __restr
             *reinterpret_cast<float4*>(dst + j) = make_float4(x[j] * f, x[j + 1] * f, x[j + 2] * f, x[j + 3] * f);
         }
       }
-      if (sub == (DH == 64 ? 0 : 1)) {
-        uint32_t z[8], w[8], u[8];
-        tmem_ld8(row + (uint32_t)FG, z);
-        tmem_ld8(row + (uint32_t)(Cfg::kN + FG), u);
-        tmem_ld8(row + (uint32_t)(2 * Cfg::kN + FG), w);
-        float x = fmaf(__uint_as_float(w[0]), 1.f / kLoScale, __uint_as_float(z[0]));
-        if (odd) x += __uint_as_float(u[0]);
-        st[DH * DH + i] = ((add ? st[DH * DH + i] : 0.f) + x) * f;
-      }
     }
+    if (z_warp) st[DH * DH + m % DH] = z_sum(last) * f;
     tc_fence_before();
     __syncthreads();  // the accumulators are read
   };
@@ -296,31 +300,40 @@ __global__ void __launch_bounds__(256, 2) lin_state_kernel(const __half* __restr
   pdl_trigger();
   pdl_wait();
   pass(std::false_type{});
-  // each feature's largest key, over the lanes and warps that share its columns
+  // A feature with z >= 2^-13 C has a phi of 2^-13 or more.  Where one has not: each feature's
+  // largest key, and with it the power of two of its phi (1 if that is 2^-13 or more)
+  float f = 1.f;
+  settle(it_end - 1);
+  const bool low = z_warp && z_sum(it_end - 1) < kPhiSmall * (float)C;
+  tc_fence_before();
+  if (__syncthreads_or(low)) {
+    __half2 km[4];  // of this thread's 8 features
 #pragma unroll
-  for (int o = FG / 8; o < 32; o <<= 1)
+    for (int e = 0; e < 4; ++e) km[e] = __half2half2(__ushort_as_half(0xFC00u));
+    for (int i = t; i < C * (FG / 8); i += 256) {
+      const uint4 k = *reinterpret_cast<const uint4*>(kv + at(row0 + i / (FG / 8), kcol + (i % (FG / 8)) * 8));
+      const __half2* hk = reinterpret_cast<const __half2*>(&k);
 #pragma unroll
-    for (int e = 0; e < 4; ++e) km[e] = __hmax2(km[e], __shfl_xor_sync(0xffffffffu, km[e], o));
-  if (lane < FG / 8) {
+      for (int e = 0; e < 4; ++e) km[e] = __hmax2(km[e], hk[e]);
+    }
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      atomicMax(kmax + 8 * lane + 2 * e, order_key(__low2half(km[e])));
-      atomicMax(kmax + 8 * lane + 2 * e + 1, order_key(__high2half(km[e])));
+      atomicMax(kmax + (t % (FG / 8)) * 8 + 2 * e, order_key(__low2half(km[e])));
+      atomicMax(kmax + (t % (FG / 8)) * 8 + 2 * e + 1, order_key(__high2half(km[e])));
+    }
+    __syncthreads();
+    auto exponent = [&](int mm) {
+      const float x = __half2float(order_half(kmax[mm]));
+      return x >= kKeySmall ? 0 : (int)fminf(126.f, floorf(-x * 1.44269504f));
+    };
+    if (__syncthreads_or(t < FG && exponent(t) != 0)) {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) scale[e] = pow2(exponent((t % (FG / 8)) * 8 + e));
+      pass(std::true_type{});
+      if (m < FG) f = pow2(-exponent(m));
     }
   }
-  __syncthreads();
-  // the power of two of feature m: 1 where its largest phi is at least 2^-14
-  auto exponent = [&](int m) {
-    const float x = __half2float(order_half(kmax[m]));
-    return x >= kPhiSmall ? 0 : (int)fminf(126.f, floorf(-x * 1.44269504f));
-  };
-  const int my_exp = t < FG ? exponent(t) : 0;
-  if (__syncthreads_or(my_exp)) {
-#pragma unroll
-    for (int e = 0; e < 8; ++e) scale[e] = pow2(exponent((t % (FG / 8)) * 8 + e));
-    pass(std::true_type{});
-  }
-  flush(it_end - 1, m < FG ? pow2(-exponent(m)) : 1.f);
+  flush(it_end - 1, f);
   if (warp == 0) {
     umma_drain(drain, status, go);
     tmem_dealloc(tmem, Cfg::kCols);
